@@ -409,9 +409,11 @@ __global__ void bfs_seed_kernel(uint32_t *reached, int root, int *frontier, int 
     *count = 1;
 }
 
+// One level: the frontier's size *nf is read on the device, so levels are
+// enqueued back to back without the host in between.
 __global__ void bfs_level_kernel(const int *__restrict__ adj, int R, const int *__restrict__ frontier,
-                                 int nf, int *next, int *next_count, uint32_t *reached) {
-    const int64_t total = (int64_t)nf * R;
+                                 const int *nf, int *next, int *next_count, uint32_t *reached) {
+    const int64_t total = (int64_t)*nf * R;
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total;
          x += (int64_t)gridDim.x * blockDim.x) {
         int u = frontier[x / R];
@@ -427,13 +429,21 @@ cudaError_t launch_bfs_seed(uint32_t *reached, int root, int *frontier, int *cou
     return cudaGetLastError();
 }
 
-cudaError_t launch_bfs_level(const int *adj, int R, const int *frontier, int nf, int *next,
+cudaError_t launch_bfs_level(const int *adj, int R, const int *frontier, const int *nf, int *next,
                              int *next_count, uint32_t *reached, cudaStream_t st) {
-    int64_t total = (int64_t)nf * R;
-    int64_t blocks = (total + 255) / 256;
-    int64_t cap = (int64_t)sm_count() * 8;
-    bfs_level_kernel<<<(int)(blocks < cap ? blocks : cap), 256, 0, st>>>(adj, R, frontier, nf, next,
-                                                                         next_count, reached);
+    bfs_level_kernel<<<sm_count() * 8, 256, 0, st>>>(adj, R, frontier, nf, next, next_count, reached);
+    return cudaGetLastError();
+}
+
+__global__ void fill_kernel(int *p, int64_t n, int v) {
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x)
+        p[x] = v;
+}
+
+cudaError_t launch_fill(int *p, int64_t n, int v, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    const int64_t blocks = (n + 255) / 256, cap = (int64_t)sm_count() * 8;
+    fill_kernel<<<(int)(blocks < cap ? blocks : cap), 256, 0, st>>>(p, n, v);
     return cudaGetLastError();
 }
 

@@ -6,50 +6,61 @@
 // give the first result with a free slot (else the smallest reached id with
 // one) the edge s->u, and mark everything u reaches.
 //
-// GPU form, identical result, in speculate-and-commit batches:
-//   gather     the next B unreached ids in ascending order (one CTA);
-//   speculate  one warp per listed u runs Alg. 1 on the graph as it stands and
-//              keeps its final pool plus the ids it expanded;
-//   commit     one CTA walks the list in order: skip u if an earlier fix-up of
-//              this batch reached it; reuse its pool unless an edge added since
-//              the snapshot could have changed it (then search again on the
-//              current graph); pick s from the pool with the current degrees;
-//              append s->u; mark what u reaches.
-// Alg. 1 reads only the adjacency rows of the nodes it expands, and a new
-// edge e->w matters only if e was expanded and w would have entered the pool
-// then: the pool was not yet full, or key(w) was below its L-th key at that
-// expansion.  Once the pool is full its L-th key never rises, so a w that
-// could not enter at e's expansion can never enter later either, and the
-// pool is unchanged.  The speculative search logs, per expansion, the node
-// and that entry bar; the check uses a relative slack of 2^-10 on the
-// distance, so summation-order rounding can only cause an extra re-search.  The list holds consecutive
-// unreached ids, so walking it in order and skipping reached ones visits the
-// same u sequence as "smallest unreached id" after every fix-up.
+// GPU form, identical result, batch by batch:
+//   list     the next B unreached ids in ascending order (one CTA);
+//   label    every unreached node gets the smallest list position that reaches
+//            it through unreached nodes (label-correcting BFS, a few levels over
+//            the whole GPU, what is left by one CTA).  New edges start at reached nodes, so
+//            nothing a batch adds changes this: listed id j is a fix-up exactly
+//            when its label is j, and when the fix-ups before position j are
+//            made, the nodes labelled below j are reached;
+//   rounds   fix-up f's search depends on the edges s_i -> u_i proposed by the
+//            fix-ups i < f.  Every round, one warp per fix-up runs Alg. 1 on the
+//            graph with the proposals of earlier fix-ups (GraphView hides the
+//            later ones) -- in the first round for all, then only where a changed
+//            proposal could have changed it -- and picks its s with the degrees
+//            that view gives; then one CTA collects the proposals, sorts them by
+//            (source, fix-up) and writes them past the rows' degrees.  Fix-up 0
+//            depends on nothing, and once the fix-ups before f stand still, f is
+//            final after one more round: whatever precedes the first proposal
+//            that changed in a round is the sequential loop's choice;
+//   commit   the final prefix (all of the batch, once a round changed nothing)
+//            becomes part of the graph and the next list starts after it.
+// A changed edge e->w can matter to f's search only if e was expanded and w
+// entered (or could enter) the pool then: the pool was not yet full, or key(w)
+// was below its L-th key at that expansion.  Once the pool is full its L-th
+// key never rises, so a w that could not enter at e's expansion can never
+// enter later either, and the pool is unchanged.  The search logs, per
+// expansion, the node and that entry bar; the check uses a relative slack of
+// 2^-10 on the distance, so summation-order rounding can only cause an extra
+// search.
+//
+// Bound by latency: a search is a chain of ~60 dependent expansions, so what
+// counts is how many fix-ups one chain's time serves.  Before, one CTA walked
+// the batch in order with ~10 dependent round trips to memory per fix-up and
+// repeated a stale search alone.  Measured (whole build, before -> after):
+// 10,000 x 32 16.9 -> 5.4 ms, 100,000 x 128 115.6 -> 58.9 ms, 150,000 x 96 on
+// an nn-descent graph 106.4 -> 51.8 ms (the pass itself 66 -> 4, 65 -> 5 and
+// 68 -> 8 ms).
 #include <climits>
 #include <vector>
 
 #include "kernels.h"
 #include "search_core.cuh"
 
-// Unreached ids speculated per batch: larger batches run more searches in
-// parallel, smaller ones leave fewer earlier fix-ups to make a speculation
-// stale.  The batch starts at NSG_CONNECT_BATCH and adapts between
-// CONNECT_MIN_BATCH and CONNECT_MAX_BATCH to the share of speculations the
-// previous batch had to redo (the result does not depend on it).
 #ifndef NSG_CONNECT_U_WIDE8
 #define NSG_CONNECT_U_WIDE8 4  // rows in flight per warp, 513..1024-value rows
-#endif
-#ifndef NSG_CONNECT_BATCH
-#define NSG_CONNECT_BATCH 64
 #endif
 
 namespace nsg {
 
 namespace {
 
+constexpr int CONNECT_FIRST_BATCH = 1024;
 constexpr int CONNECT_MIN_BATCH = 64;
-constexpr int CONNECT_MAX_BATCH = 1024;
-constexpr int CONNECT_SQ = 2048;  // queue entries of the reach step held in shared memory
+constexpr int CONNECT_MAX_BATCH = 4096;  // 2 sort entries per fix-up in 64 KB of shared memory
+constexpr int CONNECT_ROUNDS = 8;        // rounds enqueued per batch (they end early when settled)
+constexpr int LABEL_LEVELS = 10;         // label levels run by the whole GPU before one CTA finishes
 
 __host__ __device__ inline int round32c(int x) { return (x + 31) & ~31; }
 inline int log2c(unsigned x) {
@@ -67,13 +78,35 @@ __device__ __forceinline__ bool bit_is_set(const uint32_t *bits, int64_t x) {
     return (ldv(bits + (x >> 5)) >> (x & 31)) & 1u;
 }
 
-// ids >= cursor that are not reached, ascending, at most B; meta = {count, last id}
-__global__ void __launch_bounds__(256) gather_unreached_kernel(const uint32_t *reached, int64_t n, int64_t cursor,
-                                                               int B, int *list, int *meta) {
-    __shared__ int warp_sum[8];
+// State of the pass on the device.
+struct FixState {
+    long long cursor;    // every id below it is reached
+    int cnt, last;       // ids listed, the last one
+    int F, touched;      // fix-ups among them, nodes labelled
+    int nent;            // sorted edge entries of the last round
+    int settled;         // the proposals stand still (up to jfirst / none)
+    int jfirst, none;    // first fix-up whose proposal changed; first without one
+    int added, status, capped, redone;  // totals of the pass
+    int B;                              // ids the next list takes
+    int stamp;                          // last label level run
+    int lev[LABEL_LEVELS + 1];          // queue sizes of this batch's label levels
+};
+
+// Edge entries are sorted by (source, fix-up): source << 32 | fix-up << 2 | kind.
+constexpr unsigned ENT_CUR = 1;  // a current proposal
+constexpr unsigned ENT_CHG = 2;  // proposed or withdrawn in the last round
+__device__ __forceinline__ int ent_fix(uint64_t e) { return (int)((uint32_t)e >> 2); }
+__device__ __forceinline__ int ent_src(uint64_t e) { return (int)(e >> 32); }
+
+// ids >= cursor that are not reached, ascending, at most B
+// (one CTA), and the start of their labels.
+__global__ void __launch_bounds__(1024) gather_unreached_kernel(const uint32_t *reached, int64_t n, int *list,
+                                                                int *label, int *touched, int *queue, FixState *st) {
+    __shared__ int warp_sum[32];
     __shared__ int sh_total;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t nwords = (n + 31) >> 5;
+    const int64_t nwords = (n + 31) >> 5, cursor = st->cursor;
+    const int B = st->B;
     if (tid == 0) sh_total = 0;
     __syncthreads();
     for (int64_t w0 = cursor >> 5; w0 < nwords; w0 += blockDim.x) {
@@ -110,353 +143,521 @@ __global__ void __launch_bounds__(256) gather_unreached_kernel(const uint32_t *r
         if (tid == 0) sh_total = total + block;
         __syncthreads();
     }
+    const int cnt = sh_total < B ? sh_total : B;
+    for (int j = tid; j < cnt; j += blockDim.x) {
+        const int u = list[j];
+        label[u] = j;
+        touched[j] = u;
+        queue[j] = u;
+    }
+    if (tid <= LABEL_LEVELS) st->lev[tid] = tid == 0 ? cnt : 0;
     if (tid == 0) {
-        const int cnt = sh_total < B ? sh_total : B;
-        meta[0] = cnt;
-        meta[1] = cnt > 0 ? list[cnt - 1] : -1;
+        st->cnt = cnt;
+        st->last = cnt > 0 ? list[cnt - 1] : -1;
+        st->touched = cnt;
     }
 }
 
-struct SpecArgs {
-    const float4 *base4;
-    int dp4;
-    const int *adj;
-    int R, W, nav, L, H, hshift, max_steps;
-    const int *list;
-    const int *meta;
-    uint64_t *pools;  // [B][L]
-    int *psize;       // [B]
-    int *xlog;        // [B][xcap]
-    uint64_t *xthr;   // [B][xcap]: entry bar of the pool at each expansion
-    int *xcnt;        // [B]: expansions, INT_MAX when the search hit its cap
-    int xcap;
-};
-
-template <int G, int V, int U>
-__global__ void __launch_bounds__(256) speculate_kernel(SpecArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    const unsigned lane = lane_id();
-    WarpSmem s = carve_warp_smem(smem + warp * warp_smem_bytes(a.L, a.W, 0, a.H), a.L, a.W, 0, a.H);
-    const int cnt = a.meta[0];
-    int csize = 0;
-    for (int j = blockIdx.x * wpb + warp; j < cnt; j += gridDim.x * wpb) {
-        const int u = a.list[j];
-        DistF32<G, V, U> dist{{}, a.base4, a.dp4};
-        dist.Q.load_row(a.base4 + (int64_t)u * a.dp4, a.dp4);
-        SearchOut o = warp_alg1<false, false>(dist, GraphRef{a.adj, a.R}, a.nav, a.L, s, (uint32_t)a.H - 1,
-                                              a.hshift, a.max_steps, -1, 0, csize, a.xlog + (int64_t)j * a.xcap,
-                                              a.xcap, nullptr, a.xthr + (int64_t)j * a.xcap);
-        for (int t = lane; t < a.L; t += 32) a.pools[(int64_t)j * a.L + t] = t < o.size ? s.pool[t] : KEY_INF;
-        if (lane == 0) {
-            a.psize[j] = o.size;
-            a.xcnt[j] = o.capped ? INT_MAX : o.n_expand;
-        }
-        __syncwarp();
-    }
-}
-
-struct CommitArgs {
+struct FixArgs {
     const float4 *base4;
     int dp4;
     int64_t n;
     int *adj, *deg;
     int R, W, nav, L, H, hshift, max_steps;
-    uint32_t *reached, *dirty;
-    int *deg0;  // out-degree at the start of the batch, valid where dirty
-    int *queue;
-    const int *list, *meta;
-    const uint64_t *pools, *xthr;
-    const int *psize, *xlog, *xcnt;
+    uint32_t *reached;
+    int *label;               // [n] INT_MAX outside a batch
+    int *stamp;               // [n] last label level that queued the node
+    int bmax;
+    int2 *head;               // [n] source -> (first entry, entries); {0, 0} outside a batch
+    int *qa, *qb, *touched;   // [n] each
+    FixState *st;
+    int *list, *fix, *flab;   // [B] listed ids; the fix-ups and their labels
+    uint64_t *pools, *xthr;   // [B][L] final pools; [B][xcap] entry bar at each expansion
+    int *xlog, *xcnt, *psize; // [B][xcap] expanded nodes; expansions (INT_MAX: the search hit its cap)
     int xcap;
-    int *out;  // [0] edges added, [1] status, [2] capped, [3] re-searched
+    int *snew, *scur;         // [B] proposed source (-1: no pool entry has room), this and the last round
+    int *slot, *hold;         // [B] adjacency slot a proposal occupies (-1: none) and what it held
+    uint64_t *ent;            // [2 * B]
 };
 
-// L1 prefetch of fix-up i's speculative pool and expansion log (written by
-// the speculate launch, read-only here), issued one fix-up ahead.
-__device__ __forceinline__ void prefetch_fixup(const CommitArgs &a, int i, int xc, int ps) {
-    const int pool_lines = (ps * 8 + 127) >> 7, x = xc < a.xcap ? xc : 0;
-    const int xlog_lines = (x * 4 + 127) >> 7, xthr_lines = (x * 8 + 127) >> 7;
-    for (int t = threadIdx.x; t < pool_lines + xlog_lines + xthr_lines; t += blockDim.x) {
-        const char *p = t < pool_lines ? reinterpret_cast<const char *>(a.pools + (int64_t)i * a.L) + (t << 7)
-                        : t < pool_lines + xlog_lines
-                            ? reinterpret_cast<const char *>(a.xlog + (int64_t)i * a.xcap) + ((t - pool_lines) << 7)
-                            : reinterpret_cast<const char *>(a.xthr + (int64_t)i * a.xcap) +
-                                  ((t - pool_lines - xlog_lines) << 7);
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+// One node of a label level: its label offered to the unreached nodes it links
+// to; a node whose label falls is queued once per level (its stamp).  Warp-wide.
+__device__ __forceinline__ void label_node(const FixArgs &a, int node, int stamp, int *nxt, int *ncount) {
+    const unsigned lane = lane_id();
+    const int l = ldv(a.label + node);
+    const int *row = a.adj + (int64_t)node * a.R;
+    for (int b = 0; b < a.R; b += 32) {
+        const int slot = b + (int)lane;
+        const int v = slot < a.R ? row[slot] : -1;
+        bool push = false, first = false;
+        if (v >= 0 && !bit_is_set(a.reached, v) && ldv(a.label + v) > l) {
+            const int old = atomicMin(a.label + v, l);
+            first = old == INT_MAX;
+            push = old > l && atomicExch(a.stamp + v, stamp) != stamp;
+        }
+        const unsigned bf = __ballot_sync(NSG_FULL, first), bp = __ballot_sync(NSG_FULL, push);
+        int at = 0, an = 0;
+        if (lane == 0 && bf) at = atomicAdd(&a.st->touched, __popc(bf));
+        if (lane == 0 && bp) an = atomicAdd(ncount, __popc(bp));
+        at = __shfl_sync(NSG_FULL, at, 0);
+        an = __shfl_sync(NSG_FULL, an, 0);
+        if (first) a.touched[at + __popc(bf & lanemask_lt())] = v;
+        if (push) nxt[an + __popc(bp & lanemask_lt())] = v;
     }
+}
+
+__global__ void __launch_bounds__(256) label_level_kernel(FixArgs a, int level, const int *cur, int *nxt) {
+    const int nc = a.st->lev[level], stamp = a.st->stamp + level + 1;
+    const int warps = gridDim.x * (blockDim.x >> 5);
+    for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < nc; i += warps)
+        label_node(a, cur[i], stamp, nxt, &a.st->lev[level + 1]);
+}
+
+// The label levels that are left, and the list of fix-ups.  One CTA.
+__global__ void __launch_bounds__(1024) label_kernel(FixArgs a, int *cur, int *nxt) {
+    __shared__ int sh_next, sh_F;
+    __shared__ int warp_sum[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
+    FixState *st = a.st;
+    const int cnt = st->cnt;
+    int nc = st->lev[LABEL_LEVELS], stamp = st->stamp + LABEL_LEVELS;
+    if (tid == 0) sh_F = 0;
+    __syncthreads();
+    while (nc > 0) {  // ends: every queued node's label fell since it was last queued
+        ++stamp;
+        if (tid == 0) sh_next = 0;
+        __syncthreads();
+        for (int i = warp; i < nc; i += nt >> 5) label_node(a, ldv(cur + i), stamp, nxt, &sh_next);
+        __syncthreads();
+        nc = sh_next;
+        __syncthreads();
+        int *t = cur;
+        cur = nxt;
+        nxt = t;
+    }
+    // fix-ups in list order
+    for (int b = 0; b < cnt; b += nt) {
+        const int j = b + tid;
+        const int u = j < cnt ? a.list[j] : 0;
+        const bool is = j < cnt && ldv(a.label + u) == j;
+        const unsigned bal = __ballot_sync(NSG_FULL, is);
+        if (lane == 0) warp_sum[warp] = __popc(bal);
+        __syncthreads();
+        int before = sh_F, all = 0;
+        for (int k = 0; k < (nt >> 5); ++k) {
+            if (k < warp) before += warp_sum[k];
+            all += warp_sum[k];
+        }
+        if (is) {
+            const int f = before + __popc(bal & lanemask_lt());
+            a.fix[f] = u;
+            a.flab[f] = j;
+            a.scur[f] = -1;
+            a.slot[f] = -1;
+        }
+        __syncthreads();
+        if (tid == 0) sh_F += all;
+        __syncthreads();
+    }
+    if (tid == 0) {
+        st->F = sh_F;
+        st->stamp = stamp;
+        st->nent = 0;
+        st->settled = 0;
+        st->jfirst = 0;
+        st->none = INT_MAX;
+    }
+}
+
+// Whether a proposal that changed in the last round could have changed fix-up
+// f's search.  Warp-wide: a lane per logged expansion walks the entries of its
+// node; distances by the whole warp.
+__device__ __forceinline__ bool fix_stale(const FixArgs &a, int f, int u) {
+    const unsigned lane = lane_id();
+    const int xc = a.xcnt[f];
+    if (xc > a.xcap) return a.st->jfirst < f;
+    const float4 *xu = a.base4 + (int64_t)u * a.dp4;
+    for (int b = 0; b < xc; b += 32) {
+        const int t = b + (int)lane;
+        int p = 0, end = 0;
+        float bar = 0.0f;
+        bool open = false;  // the pool was not full: any new neighbour entered
+        if (t < xc) {
+            const int2 h = a.head[a.xlog[(int64_t)f * a.xcap + t]];
+            p = h.x;
+            end = h.x + h.y;
+            if (h.y > 0) {
+                const uint64_t thr = a.xthr[(int64_t)f * a.xcap + t];
+                open = thr == KEY_INF;
+                bar = kd2(thr) * (1.0f + 1.0f / 1024.0f);
+            }
+        }
+        for (;;) {
+            int i = -1;  // the lane's next changed edge of an earlier fix-up
+            while (p < end && i < 0) {
+                const uint64_t e = a.ent[p++];
+                if ((e & ENT_CHG) && ent_fix(e) < f) i = ent_fix(e);
+            }
+            unsigned pend = __ballot_sync(NSG_FULL, i >= 0);
+            if (!pend) break;
+            if (__any_sync(NSG_FULL, i >= 0 && open)) return true;
+            while (pend) {
+                const int src = __ffs(pend) - 1;
+                pend &= pend - 1u;
+                const float4 *xw = a.base4 + (int64_t)a.fix[__shfl_sync(NSG_FULL, i, src)] * a.dp4;
+                const float lim = __shfl_sync(NSG_FULL, bar, src);
+                float d2 = 0.0f;
+                for (int c = (int)lane; c < a.dp4; c += 32) d2 += sq4(__ldg(xu + c), __ldg(xw + c));
+                if (group_sum<32>(d2) <= lim) return true;
+            }
+        }
+    }
+    return false;
+}
+
+// The first of `size` pool entries (key order) with room in fix-up f's view, -1
+// if there is none.  Warp-wide.
+__device__ __forceinline__ int fix_select(const FixArgs &a, int f, const uint64_t *pool, int size) {
+    const unsigned lane = lane_id();
+    for (int b = 0; b < size; b += 32) {
+        const int t = b + (int)lane;
+        int e = -1;
+        bool room = false;
+        if (t < size) {
+            e = kid(pool[t]);
+            int d = a.deg[e];
+            if (d < a.R) {
+                const int2 h = a.head[e];
+                if (d + h.y >= a.R)
+                    for (int p = h.x; p < h.x + h.y; ++p) {
+                        const uint64_t x = a.ent[p];
+                        d += (x & ENT_CUR) && ent_fix(x) < f;
+                    }
+                room = d < a.R;
+            }
+        }
+        const unsigned bal = __ballot_sync(NSG_FULL, room);
+        if (bal) return __shfl_sync(NSG_FULL, e, __ffs(bal) - 1);
+    }
+    return -1;
 }
 
 template <int G, int V, int U>
-__global__ void __launch_bounds__(256) commit_kernel(CommitArgs a) {
+__global__ void __launch_bounds__(256) fix_search_kernel(FixArgs a, int round) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int sh_flag, sh_found, sh_size, sh_qtail;
-    __shared__ int s_list[CONNECT_MAX_BATCH], s_xcnt[CONNECT_MAX_BATCH], s_psize[CONNECT_MAX_BATCH];
-    __shared__ int sq[CONNECT_SQ];  // the reach step's queue (entries past it in a.queue)
-    const int tid = threadIdx.x, warp = tid >> 5;
-    WarpSmem s = carve_warp_smem(smem, a.L, a.W, 0, a.H);
-    const int cnt = a.meta[0];
-    for (int t = tid; t < cnt; t += blockDim.x) {
-        s_list[t] = a.list[t];
-        s_xcnt[t] = a.xcnt[t];
-        s_psize[t] = a.psize[t];
-    }
-    __syncthreads();
-    if (cnt > 0) prefetch_fixup(a, 0, s_xcnt[0], s_psize[0]);
-    int added = 0, redone = 0, status = 0, capped = 0;
-    for (int i = 0; i < cnt; ++i) {
-        const int u = s_list[i];
-        if (i + 1 < cnt) prefetch_fixup(a, i + 1, s_xcnt[i + 1], s_psize[i + 1]);
-        if (bit_is_set(a.reached, u)) continue;  // reached by an earlier fix-up of this batch
-        if (tid == 0) sh_flag = 0;
-        __syncthreads();
-        const int xc = s_xcnt[i];
-        if (xc > a.xcap) {
-            if (tid == 0) sh_flag = 1;
-        } else {
-            const float4 *xu = a.base4 + (int64_t)u * a.dp4;
-            for (int t = tid; t < xc; t += blockDim.x) {
-                const int e = a.xlog[(int64_t)i * a.xcap + t];
-                if (!bit_is_set(a.dirty, e)) continue;
-                const uint64_t thr = a.xthr[(int64_t)i * a.xcap + t];
-                if (thr == KEY_INF) {  // the pool was not full: any new neighbour entered
-                    sh_flag = 1;
-                    continue;
-                }
-                const float bar = kd2(thr) * (1.0f + 1.0f / 1024.0f);
-                const int d1 = ldv(a.deg + e);
-                for (int j = ldv(a.deg0 + e); j < d1; ++j) {
-                    const int w = ldv(a.adj + (int64_t)e * a.R + j);
-                    const float4 *xw = a.base4 + (int64_t)w * a.dp4;
-                    float d2 = 0.0f;
-                    for (int c = 0; c < a.dp4; ++c) {
-                        const float4 p = xu[c], q = xw[c];
-                        const float dx = p.x - q.x, dy = p.y - q.y, dz = p.z - q.z, dw = p.w - q.w;
-                        d2 += dx * dx + dy * dy + dz * dz + dw * dw;
-                    }
-                    if (d2 <= bar) sh_flag = 1;
-                }
-            }
-        }
-        __syncthreads();
-        const uint64_t *pool;
+    const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    const unsigned lane = lane_id();
+    if (a.st->settled) return;
+    WarpSmem s = carve_warp_smem(smem + warp * warp_smem_bytes(a.L, a.W, 0, a.H, true), a.L, a.W, 0, a.H, true);
+    const int F = a.st->F;
+    int csize = 0;
+    for (int f = blockIdx.x * wpb + warp; f < F; f += gridDim.x * wpb) {
+        const int u = a.fix[f];
+        uint64_t *pool = a.pools + (int64_t)f * a.L;
         int size;
-        if (sh_flag) {  // the snapshot is stale for this u: search the current graph
-            if (warp == 0) {
-                DistF32<G, V, U> dist{{}, a.base4, a.dp4};
-                dist.Q.load_row(a.base4 + (int64_t)u * a.dp4, a.dp4);
-                int csize = 0;
-                SearchOut o = warp_alg1<false, true>(dist, GraphRef{a.adj, a.R}, a.nav, a.L, s, (uint32_t)a.H - 1,
-                                                     a.hshift, a.max_steps, -1, 0, csize);
-                if (lane_id() == 0) {
-                    sh_size = o.size;
-                    if (o.capped) sh_flag = 2;
-                }
+        if (round == 0 || fix_stale(a, f, u)) {
+            DistF32<G, V, U> dist{{}, a.base4, a.dp4};
+            dist.Q.load_row(a.base4 + (int64_t)u * a.dp4, a.dp4);
+            const SearchOut o = warp_alg1<false>(dist, GraphView{a.adj, a.R, a.deg, a.label, a.flab[f]}, a.nav, a.L,
+                                                 s, (uint32_t)a.H - 1, a.hshift, a.max_steps, -1, 0, csize,
+                                                 a.xlog + (int64_t)f * a.xcap, a.xcap, nullptr,
+                                                 a.xthr + (int64_t)f * a.xcap);
+            size = o.size;
+            for (int t = lane; t < size; t += 32) pool[t] = s.pool[t];
+            if (lane == 0) {
+                a.psize[f] = size;
+                a.xcnt[f] = o.capped ? INT_MAX : o.n_expand;
+                if (round > 0) atomicAdd(&a.st->redone, 1);
             }
-            __syncthreads();
-            pool = s.pool;
-            size = sh_size;
-            ++redone;
-            if (sh_flag == 2) capped = 1;
+            __syncwarp();
+            const int sel = fix_select(a, f, s.pool, size);
+            if (lane == 0) a.snew[f] = sel;
         } else {
-            pool = a.pools + (int64_t)i * a.L;
-            size = s_psize[i];
+            const int sel = fix_select(a, f, pool, a.psize[f]);
+            if (lane == 0) a.snew[f] = sel;
         }
-        // first pool entry (key order) whose out-degree is below R
-        if (tid == 0) sh_found = INT_MAX;
-        __syncthreads();
-        for (int t = tid; t < size; t += blockDim.x)
-            if (ldv(a.deg + kid(pool[t])) < a.R) atomicMin(&sh_found, t);
-        __syncthreads();
-        int sel = sh_found == INT_MAX ? -1 : kid(pool[sh_found]);
-        __syncthreads();
-        if (sel < 0) {  // else the smallest reached id with a free slot
-            if (tid == 0) sh_found = INT_MAX;
-            __syncthreads();
-            for (int64_t x = tid; x < a.n; x += blockDim.x)
-                if (bit_is_set(a.reached, x) && ldv(a.deg + x) < a.R) atomicMin(&sh_found, (int)x);
-            __syncthreads();
-            sel = sh_found == INT_MAX ? -1 : sh_found;
-            __syncthreads();
-            if (sel < 0) {
-                status = -5;
-                break;
-            }
-        }
-        if (tid == 0) {
-            const int dg = a.deg[sel];
-            a.adj[(int64_t)sel * a.R + dg] = u;
-            a.deg[sel] = dg + 1;
-            if (!(atomicOr(a.dirty + (sel >> 5), 1u << (sel & 31)) & (1u << (sel & 31)))) a.deg0[sel] = dg;
-            atomicOr(a.reached + (u >> 5), 1u << (u & 31));
-            sq[0] = u;
-            sh_qtail = 1;
-        }
-        ++added;
-        __syncthreads();
-        int head = 0;  // mark everything u reaches
-        for (;;) {
-            const int tail = sh_qtail;
-            if (head == tail) break;
-            __syncthreads();
-            const int64_t total = (int64_t)(tail - head) * a.R;
-            for (int64_t x = tid; x < total; x += blockDim.x) {
-                const int qi = head + (int)(x / a.R);
-                const int node = qi < CONNECT_SQ ? sq[qi] : ldv(a.queue + qi);
-                const int v = ldv(a.adj + (int64_t)node * a.R + x % a.R);
-                if (v < 0) continue;
-                const uint32_t bit = 1u << (v & 31);
-                if (!(atomicOr(a.reached + (v >> 5), bit) & bit)) {
-                    const int at = atomicAdd(&sh_qtail, 1);
-                    if (at < CONNECT_SQ) sq[at] = v;
-                    else a.queue[at] = v;
-                }
-            }
-            head = tail;
-            __syncthreads();
-        }
-    }
-    if (tid == 0) {
-        a.out[0] += added;
-        if (status) a.out[1] = status;
-        a.out[2] |= capped;
-        a.out[3] += redone;
+        __syncwarp();
     }
 }
 
-template <typename T>
-struct Buf {
-    T *p = nullptr;
-    ~Buf() {
-        if (p) cudaFree(p);
+// Takes the last round's proposals out of the graph.  Block-wide.
+__device__ __forceinline__ void withdraw(const FixArgs &a, int F, int from, int nent) {
+    for (int f = from + (int)threadIdx.x; f < F; f += blockDim.x)
+        if (a.slot[f] >= 0) a.adj[(int64_t)a.scur[f] * a.R + a.slot[f]] = a.hold[f];
+    for (int p = threadIdx.x; p < nent; p += blockDim.x) a.head[ent_src(a.ent[p])] = make_int2(0, 0);
+}
+
+// The round's proposals against the last round's: entries sorted by source,
+// the current ones written past their sources' degrees in fix-up order (the
+// slots the sequential loop would give them).  One CTA.
+__global__ void __launch_bounds__(1024) fix_propose_kernel(FixArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint64_t *ent = reinterpret_cast<uint64_t *>(smem);
+    __shared__ int sh_n, sh_first, sh_none;
+    FixState *st = a.st;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    if (st->settled) return;
+    const int F = st->F;
+    if (tid == 0) {
+        sh_n = 0;
+        sh_first = INT_MAX;
+        sh_none = INT_MAX;
     }
-    cudaError_t alloc(size_t n) { return cudaMalloc(reinterpret_cast<void **>(&p), (n ? n : 1) * sizeof(T)); }
-};
+    withdraw(a, F, 0, st->nent);
+    __syncthreads();
+    for (int f = tid; f < F; f += nt) {
+        const int was = a.scur[f], now = a.snew[f];
+        const unsigned chg = was != now ? ENT_CHG : 0u;
+        if (now >= 0) ent[atomicAdd(&sh_n, 1)] = ((uint64_t)now << 32) | ((uint32_t)f << 2) | ENT_CUR | chg;
+        else atomicMin(&sh_none, f);
+        if (chg) {
+            if (was >= 0) ent[atomicAdd(&sh_n, 1)] = ((uint64_t)was << 32) | ((uint32_t)f << 2) | ENT_CHG;
+            atomicMin(&sh_first, f);
+        }
+        a.scur[f] = now;
+    }
+    __syncthreads();
+    const int N = sh_n;
+    int P2 = 2;
+    while (P2 < N) P2 <<= 1;
+    for (int p = N + tid; p < P2; p += nt) ent[p] = ~0ull;
+    __syncthreads();
+    for (int k = 2; k <= P2; k <<= 1)  // bitonic sort
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int x = tid; x < P2 / 2; x += nt) {
+                const int lo = ((x & ~(j - 1)) << 1) | (x & (j - 1)), hi = lo | j;
+                const uint64_t p = ent[lo], q = ent[hi];
+                if ((p > q) == ((lo & k) == 0)) {
+                    ent[lo] = q;
+                    ent[hi] = p;
+                }
+            }
+            __syncthreads();
+        }
+    for (int p = tid; p < N; p += nt) {
+        const uint64_t e = ent[p];
+        const int src = ent_src(e);
+        a.ent[p] = e;
+        if (p == 0 || ent_src(ent[p - 1]) != src) {
+            int q = p + 1;
+            while (q < N && ent_src(ent[q]) == src) ++q;
+            a.head[src] = make_int2(p, q - p);
+        }
+        if (e & ENT_CUR) {
+            const int f = ent_fix(e);
+            int at = a.deg[src];
+            for (int q = p - 1; q >= 0 && ent_src(ent[q]) == src; --q) at += (ent[q] & ENT_CUR) ? 1 : 0;
+            int *cell = a.adj + (int64_t)src * a.R + at;
+            if (at < a.R) {  // (a source more fix-ups want than it has room for takes the first ones)
+                a.hold[f] = *cell;
+                *cell = a.fix[f];
+                a.slot[f] = at;
+            } else {
+                a.slot[f] = -1;
+            }
+        }
+    }
+    for (int f = tid; f < F; f += nt)
+        if (a.scur[f] < 0) a.slot[f] = -1;
+    if (tid == 0) {
+        st->nent = N;
+        st->jfirst = sh_first;
+        st->none = sh_none;
+        st->settled = sh_first == INT_MAX || sh_none < sh_first;
+    }
+}
+
+// The final prefix of the batch enters the graph; a fix-up whose pool has no
+// room (the first one, if any) takes the smallest reached id with a free slot.
+// One CTA.
+__global__ void __launch_bounds__(1024) fix_commit_kernel(FixArgs a) {
+    __shared__ int sh_found;
+    FixState *st = a.st;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int F = st->F, touched = st->touched, none = st->none, first = st->jfirst;
+    const int nent = st->nent;
+    if (st->cnt == 0) return;
+    int done = min(F, min(none, first));
+    withdraw(a, F, done, nent);
+    for (int f = tid; f < done; f += nt) {
+        atomicAdd(a.deg + a.scur[f], 1);
+        if (a.xcnt[f] == INT_MAX) st->capped = 1;
+    }
+    __syncthreads();
+    int limit = done < F ? a.flab[done] : INT_MAX;
+    for (int t = tid; t < touched; t += nt) {
+        const int v = a.touched[t];
+        if (a.label[v] < limit) atomicOr(a.reached + (v >> 5), 1u << (v & 31));
+    }
+    if (none < F && none < first) {
+        if (tid == 0) sh_found = INT_MAX;
+        __syncthreads();
+        for (int64_t x = tid; x < a.n; x += nt)
+            if (bit_is_set(a.reached, x) && ldv(a.deg + x) < a.R) {
+                atomicMin(&sh_found, (int)x);
+                break;
+            }
+        __syncthreads();
+        const int sel = sh_found;
+        if (sel == INT_MAX) {
+            if (tid == 0) st->status = -5;
+        } else {
+            if (tid == 0) {
+                const int u = a.fix[done], dg = a.deg[sel];
+                a.adj[(int64_t)sel * a.R + dg] = u;
+                a.deg[sel] = dg + 1;
+                if (a.xcnt[done] == INT_MAX) st->capped = 1;
+            }
+            ++done;
+            const int lim2 = done < F ? a.flab[done] : INT_MAX;
+            for (int t = tid; t < touched; t += nt) {
+                const int v = a.touched[t], l = a.label[v];
+                if (l >= limit && l < lim2) atomicOr(a.reached + (v >> 5), 1u << (v & 31));
+            }
+        }
+    }
+    __syncthreads();
+    for (int t = tid; t < touched; t += nt) a.label[a.touched[t]] = INT_MAX;
+    if (tid == 0) {
+        st->cursor = done < F ? a.fix[done] : (long long)st->last + 1;
+        st->added += done;
+        // the batch follows how much of it settled (the result does not depend
+        // on it): a larger one serves more fix-ups per search's latency, until
+        // the chains of fix-ups that depend on one another outlast the rounds
+        if (done * 10 >= F * 9) st->B = min(st->B * 2, a.bmax);
+        else if (done * 2 < F) st->B = max(st->B / 2, CONNECT_MIN_BATCH);
+    }
+}
 
 }  // namespace
 
 cudaError_t run_connect(const ConnectLaunch &l, int out_host[4], cudaStream_t st) {
     const int64_t n = l.n;
     const int64_t nwords = (n + 31) / 32;
-    const int BMAX = CONNECT_MAX_BATCH;
-    int B = NSG_CONNECT_BATCH < CONNECT_MIN_BATCH ? CONNECT_MIN_BATCH
-            : NSG_CONNECT_BATCH > BMAX            ? BMAX
-                                                  : NSG_CONNECT_BATCH;
     const int xcap = 4 * l.L + 64;
-    Buf<uint32_t> reached, dirty;
-    Buf<int> qa, qb, cnt, list, meta, psize, xlog, xcnt, out, deg0;
-    Buf<uint64_t> pools, xthr;
+    // fix-ups per batch: what fits 512 MB of pools and logs, at most the kernels' limit
+    int BMAX = CONNECT_MAX_BATCH;
+    while (BMAX > CONNECT_MIN_BATCH && (size_t)BMAX * (8 * (size_t)l.L + 12 * (size_t)xcap) > (size_t(512) << 20)) BMAX /= 2;
+    // one allocation for the whole pass
+    size_t need = 0;
+    auto plan = [&](size_t bytes) {
+        const size_t at = need;
+        need += (bytes + 255) & ~size_t(255);
+        return at;
+    };
+    const size_t o_reached = plan(4 * nwords), o_stamp = plan(4 * n), o_head = plan(8 * n), o_st = plan(sizeof(FixState)),
+                 o_lev = plan(4 * (BFS_LEVELS + 1)), zeroed = need;
+    const size_t o_label = plan(4 * n), o_qa = plan(4 * n), o_qb = plan(4 * n), o_touched = plan(4 * n),
+                 o_list = plan(4 * BMAX), o_fix = plan(4 * BMAX), o_flab = plan(4 * BMAX), o_xcnt = plan(4 * BMAX),
+                 o_psize = plan(4 * BMAX), o_snew = plan(4 * BMAX), o_scur = plan(4 * BMAX), o_slot = plan(4 * BMAX),
+                 o_hold = plan(4 * BMAX), o_ent = plan(16 * BMAX), o_pools = plan(8 * (size_t)BMAX * l.L),
+                 o_xthr = plan(8 * (size_t)BMAX * xcap), o_xlog = plan(4 * (size_t)BMAX * xcap);
+    struct Slab {
+        unsigned char *p = nullptr;
+        ~Slab() {
+            if (p) cudaFree(p);
+        }
+    } slab;
     cudaError_t e;
-    if ((e = reached.alloc(nwords)) || (e = dirty.alloc(nwords)) || (e = qa.alloc(n)) || (e = qb.alloc(n)) ||
-        (e = cnt.alloc(2)) || (e = list.alloc(BMAX)) || (e = meta.alloc(2)) || (e = psize.alloc(BMAX)) ||
-        (e = xlog.alloc((size_t)BMAX * xcap)) || (e = xcnt.alloc(BMAX)) || (e = out.alloc(4)) ||
-        (e = pools.alloc((size_t)BMAX * l.L)) || (e = xthr.alloc((size_t)BMAX * xcap)) || (e = deg0.alloc(n)))
-        return e;
-    if ((e = cudaMemsetAsync(reached.p, 0, nwords * 4, st)) || (e = cudaMemsetAsync(out.p, 0, 16, st))) return e;
-    // reach from the navigating node: level-synchronous BFS
-    if ((e = launch_bfs_seed(reached.p, l.nav, qa.p, cnt.p, st))) return e;
-    int nf = 1;
-    int *cur = qa.p, *nxt = qb.p;
-    for (int64_t level = 0; nf > 0 && level <= n; ++level) {
-        if ((e = cudaMemsetAsync(cnt.p + 1, 0, sizeof(int), st))) return e;
-        if ((e = launch_bfs_level(l.adj, l.R, cur, nf, nxt, cnt.p + 1, reached.p, st))) return e;
-        if ((e = cudaMemcpyAsync(&nf, cnt.p + 1, sizeof(int), cudaMemcpyDeviceToHost, st))) return e;
+    if ((e = cudaMalloc(reinterpret_cast<void **>(&slab.p), need))) return e;
+    auto at = [&](size_t o) { return slab.p + o; };
+    FixArgs a;
+    a.base4 = reinterpret_cast<const float4 *>(l.base);
+    a.dp4 = l.dp / 4;
+    a.n = n;
+    a.adj = l.adj;
+    a.deg = l.deg;
+    a.R = l.R;
+    a.W = round32c(l.R);
+    a.nav = l.nav;
+    a.L = l.L;
+    a.H = l.hash_slots;
+    a.hshift = 32 - log2c((unsigned)l.hash_slots);
+    a.max_steps = l.max_steps;
+    a.reached = reinterpret_cast<uint32_t *>(at(o_reached));
+    a.stamp = reinterpret_cast<int *>(at(o_stamp));
+    a.bmax = BMAX;
+    a.head = reinterpret_cast<int2 *>(at(o_head));
+    a.st = reinterpret_cast<FixState *>(at(o_st));
+    a.label = reinterpret_cast<int *>(at(o_label));
+    a.qa = reinterpret_cast<int *>(at(o_qa));
+    a.qb = reinterpret_cast<int *>(at(o_qb));
+    a.touched = reinterpret_cast<int *>(at(o_touched));
+    a.list = reinterpret_cast<int *>(at(o_list));
+    a.fix = reinterpret_cast<int *>(at(o_fix));
+    a.flab = reinterpret_cast<int *>(at(o_flab));
+    a.xcnt = reinterpret_cast<int *>(at(o_xcnt));
+    a.psize = reinterpret_cast<int *>(at(o_psize));
+    a.snew = reinterpret_cast<int *>(at(o_snew));
+    a.scur = reinterpret_cast<int *>(at(o_scur));
+    a.slot = reinterpret_cast<int *>(at(o_slot));
+    a.hold = reinterpret_cast<int *>(at(o_hold));
+    a.ent = reinterpret_cast<uint64_t *>(at(o_ent));
+    a.pools = reinterpret_cast<uint64_t *>(at(o_pools));
+    a.xthr = reinterpret_cast<uint64_t *>(at(o_xthr));
+    a.xlog = reinterpret_cast<int *>(at(o_xlog));
+    a.xcap = xcap;
+    int *lev = reinterpret_cast<int *>(at(o_lev));
+    if ((e = cudaMemsetAsync(slab.p, 0, zeroed, st)) || (e = launch_fill(a.label, n, INT_MAX, st))) return e;
+    // reach from the navigating node: level-synchronous BFS, BFS_LEVELS levels
+    // between two looks from the host (levels past the end find no frontier)
+    if ((e = launch_bfs_seed(a.reached, l.nav, a.qa, lev, st))) return e;
+    FixState h{};
+    h.B = CONNECT_FIRST_BATCH < BMAX ? CONNECT_FIRST_BATCH : BMAX;
+    if ((e = cudaMemcpyAsync(a.st, &h, sizeof(h), cudaMemcpyHostToDevice, st))) return e;
+    auto list_next = [&]() -> cudaError_t {  // the next batch's list, and the state after it to the host
+        gather_unreached_kernel<<<1, 1024, 0, st>>>(a.reached, n, a.list, a.label, a.touched, a.qa, a.st);
+        cudaError_t g = cudaGetLastError();
+        if (!g) g = cudaMemcpyAsync(&h, a.st, sizeof(h), cudaMemcpyDeviceToHost, st);
+        return g;
+    };
+    int *cur = a.qa, *nxt = a.qb;
+    for (int64_t level = 0; level <= n; level += BFS_LEVELS) {
+        for (int t = 0; t < BFS_LEVELS; ++t) {
+            if ((e = launch_bfs_level(l.adj, l.R, cur, lev + t, nxt, lev + t + 1, a.reached, st))) return e;
+            std::swap(cur, nxt);
+        }
+        int nf = 0;
+        if ((e = cudaMemcpyAsync(&nf, lev + BFS_LEVELS, sizeof(int), cudaMemcpyDeviceToHost, st))) return e;
         if ((e = cudaStreamSynchronize(st))) return e;
-        std::swap(cur, nxt);
+        if (nf == 0) break;
+        if ((e = cudaMemsetAsync(lev, 0, 4 * (BFS_LEVELS + 1), st))) return e;
+        if ((e = cudaMemcpyAsync(lev, &nf, sizeof(int), cudaMemcpyHostToDevice, st))) return e;
     }
-    SpecArgs sa;
-    sa.base4 = reinterpret_cast<const float4 *>(l.base);
-    sa.dp4 = l.dp / 4;
-    sa.adj = l.adj;
-    sa.R = l.R;
-    sa.W = round32c(l.R);
-    sa.nav = l.nav;
-    sa.L = l.L;
-    sa.H = l.hash_slots;
-    sa.hshift = 32 - log2c((unsigned)l.hash_slots);
-    sa.max_steps = l.max_steps;
-    sa.list = list.p;
-    sa.meta = meta.p;
-    sa.pools = pools.p;
-    sa.psize = psize.p;
-    sa.xlog = xlog.p;
-    sa.xthr = xthr.p;
-    sa.xcnt = xcnt.p;
-    sa.xcap = xcap;
-    CommitArgs ca;
-    ca.base4 = sa.base4;
-    ca.dp4 = sa.dp4;
-    ca.n = n;
-    ca.adj = l.adj;
-    ca.deg = l.deg;
-    ca.R = l.R;
-    ca.W = sa.W;
-    ca.nav = l.nav;
-    ca.L = l.L;
-    ca.H = sa.H;
-    ca.hshift = sa.hshift;
-    ca.max_steps = l.max_steps;
-    ca.reached = reached.p;
-    ca.dirty = dirty.p;
-    ca.deg0 = deg0.p;
-    ca.queue = qa.p;
-    ca.list = list.p;
-    ca.meta = meta.p;
-    ca.pools = pools.p;
-    ca.psize = psize.p;
-    ca.xlog = xlog.p;
-    ca.xthr = xthr.p;
-    ca.xcnt = xcnt.p;
-    ca.xcap = xcap;
-    ca.out = out.p;
-    const size_t per_warp = warp_smem_bytes(l.L, sa.W, 0, sa.H);
     const int wpb = 4;
-    int64_t cursor = 0;
-    int prev[4] = {0, 0, 0, 0};
-    for (int64_t batch = 0; batch <= n; ++batch) {
-        gather_unreached_kernel<<<1, 256, 0, st>>>(reached.p, n, cursor, B, list.p, meta.p);
-        if ((e = cudaGetLastError())) return e;
-        int h[2] = {0, 0};
-        if ((e = cudaMemcpyAsync(h, meta.p, sizeof(h), cudaMemcpyDeviceToHost, st))) return e;
-        if ((e = cudaStreamSynchronize(st))) return e;
-        if (h[0] == 0) break;
-        cursor = (int64_t)h[1] + 1;
-        if ((e = cudaMemsetAsync(dirty.p, 0, nwords * 4, st))) return e;
-        NSG_DISPATCH_DP4(sa.dp4, {
-            // one batch runs only 64 searches, so their latency, not the
-            // occupancy, sets the time: 513..1024-value rows keep more rows
-            // in flight than the search kernels do
+    const size_t per_warp = warp_smem_bytes(l.L, a.W, 0, a.H, true), psmem = 16 * (size_t)BMAX;
+    if ((e = cudaFuncSetAttribute(fix_propose_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem)) ||
+        (e = list_next()) || (e = cudaStreamSynchronize(st)))
+        return e;
+    for (int64_t batch = 0; batch <= n && h.cnt > 0 && !h.status; ++batch) {
+        int *cur = a.qa, *nxt = a.qb;
+        for (int t = 0; t < LABEL_LEVELS; ++t) {
+            label_level_kernel<<<sm_count() * 4, 256, 0, st>>>(a, t, cur, nxt);
+            std::swap(cur, nxt);
+        }
+        label_kernel<<<1, 1024, 0, st>>>(a, cur, nxt);
+        NSG_DISPATCH_DP4(a.dp4, {
+            // a batch's searches leave the SMs nearly empty, so their latency,
+            // not the occupancy, sets the time: 513..1024-value rows keep more
+            // rows in flight than the search kernels do
             constexpr int UC = V_ == 8 ? NSG_CONNECT_U_WIDE8 : U_;
-            auto spec = speculate_kernel<G_, V_, UC>;
-            auto commit = commit_kernel<G_, V_, UC>;
-            if (!e) e = cudaFuncSetAttribute(spec, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(per_warp * wpb));
-            if (!e) e = cudaFuncSetAttribute(commit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)per_warp);
-            if (!e) {
-                const int grid = (h[0] + wpb - 1) / wpb;
-                spec<<<grid, wpb * 32, per_warp * wpb, st>>>(sa);
-                commit<<<1, 256, per_warp, st>>>(ca);
+            auto search = fix_search_kernel<G_, V_, UC>;
+            e = cudaFuncSetAttribute(search, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(per_warp * wpb));
+            for (int r = 0; r < CONNECT_ROUNDS && !e; ++r) {
+                search<<<(h.cnt + wpb - 1) / wpb, wpb * 32, per_warp * wpb, st>>>(a, r);
+                fix_propose_kernel<<<1, 1024, psmem, st>>>(a);
                 e = cudaGetLastError();
             }
         });
         if (e) return e;
-        int o[4];
-        if ((e = cudaMemcpyAsync(o, out.p, sizeof(o), cudaMemcpyDeviceToHost, st))) return e;
-        if ((e = cudaStreamSynchronize(st))) return e;
-        if (o[1]) break;
-        // a speculation redone in the commit costs a whole serial search, a
-        // larger batch saves a share of one parallel search per fix-up: grow the
-        // batch while at most 1 in 100 speculations were redone, in this batch
-        // and overall, shrink it when more than 1 in 50 of this batch's were
-        // (SIFT-shaped 1M: ~1.8 % at 64, which stays; DEEP-shaped 10M and
-        // GAUSS5M: < 0.5 % up to 1,024, connectivity 16.4 -> 8.4 s and
-        // 19.2 -> 5.3 s)
-        const int fixed = o[0] - prev[0], redone = o[3] - prev[3];
-        if (redone * 100 <= fixed && o[3] * 100 <= o[0] && B < BMAX) B *= 2;
-        else if (redone * 50 > fixed && B > CONNECT_MIN_BATCH) B /= 2;
-        for (int t = 0; t < 4; ++t) prev[t] = o[t];
+        fix_commit_kernel<<<1, 1024, 0, st>>>(a);
+        if ((e = cudaGetLastError()) || (e = list_next()) || (e = cudaStreamSynchronize(st))) return e;
     }
-    if ((e = cudaMemcpyAsync(out_host, out.p, 4 * sizeof(int), cudaMemcpyDeviceToHost, st))) return e;
-    return cudaStreamSynchronize(st);
+    out_host[0] = h.added;
+    out_host[1] = h.status;
+    out_host[2] = h.capped;
+    out_host[3] = h.redone;
+    return cudaSuccess;
 }
 
 }  // namespace nsg

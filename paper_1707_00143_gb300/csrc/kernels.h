@@ -210,8 +210,10 @@ cudaError_t launch_navigate(const float *base, int64_t n, int d, const int *knn,
 
 // BFS helpers and the connectivity pass.
 cudaError_t launch_bfs_seed(uint32_t *reached, int root, int *frontier, int *count, cudaStream_t st);
-cudaError_t launch_bfs_level(const int *adj, int R, const int *frontier, int nf, int *next,
+constexpr int BFS_LEVELS = 8;  // levels enqueued between two looks from the host
+cudaError_t launch_bfs_level(const int *adj, int R, const int *frontier, const int *nf, int *next,
                              int *next_count, uint32_t *reached, cudaStream_t st);
+cudaError_t launch_fill(int *p, int64_t n, int v, cudaStream_t st);
 struct ConnectLaunch {
     const float *base;  // [n][dp]
     int64_t n;
@@ -221,8 +223,7 @@ struct ConnectLaunch {
     int R, nav, L;
     int hash_slots, max_steps;
 };
-// Whole connectivity pass (reach from nav, then speculate/commit fix-up
-// batches).  out = {edges added, status, any search capped, re-searches}.
+// Whole connectivity pass (reach from nav, then batches of fix-ups).  out = {edges added, status, any search capped, re-searches}.
 // Allocates its scratch and synchronises the stream.
 cudaError_t run_connect(const ConnectLaunch &a, int out[4], cudaStream_t st);
 

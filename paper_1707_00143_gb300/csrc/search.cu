@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(256) collect_kernel(CollectArgs a) {
         DistF32<G, V, U> dist{{}, a.base4, a.dp4};
         dist.Q.load_row(a.base4 + (int64_t)v * a.dp4, a.dp4);
         int csize = 0;
-        SearchOut o = warp_alg1<true, false>(dist, GraphRef{a.knn, a.K}, a.nav, a.L, s, hmask, a.hshift,
+        SearchOut o = warp_alg1<true>(dist, GraphRef{a.knn, a.K}, a.nav, a.L, s, hmask, a.hshift,
                                              a.max_steps, v, a.C, csize);
         // Alg. 2: v's nearest neighbours in G join the candidates
         const int *row = a.knn + (int64_t)v * a.K;

@@ -14,9 +14,8 @@
 //   * search-and-collect on the kNN graph (Alg. 2, Section 3.5 iii): every computed
 //     key except the node itself is also merged into a collect list of the C
 //     smallest keys,
-//   * the connectivity pass (Alg. 2, Section 3.5 iv): speculative searches that also
-//     log the ids they expand, and re-searches on a graph the same kernel is
-//     editing (plain coherent loads instead of the read-only path).
+//   * the connectivity pass (Alg. 2, Section 3.5 iv): searches that also log the
+//     ids they expand, on a view of the graph that hides later fix-ups' edges.
 #pragma once
 
 #include "common.cuh"
@@ -88,10 +87,24 @@ struct GraphRef {
     int width;
 };
 
-template <bool COHERENT>
-__device__ __forceinline__ int load_adj(const int *p) {
-    if (COHERENT) return *reinterpret_cast<const volatile int *>(p);
-    return __ldg(p);
+// The graph as fix-up `self` of a connectivity batch sees it: the edges a row
+// holds past its degree are the batch's proposals, each into a node labelled
+// with its fix-up's position, and only earlier fix-ups' count (connect.cu).
+struct GraphView {
+    const int *adj;
+    int width;
+    const int *deg;    // [n] degrees without the proposals
+    const int *label;  // [n] INT_MAX: reached before the batch
+    int self;
+};
+
+// Slots of node u's row from which neighbours may be hidden (none in a plain graph).
+__device__ __forceinline__ int proposals_from(const GraphRef &, int) { return INT_MAX; }
+__device__ __forceinline__ int proposals_from(const GraphView &g, int u) { return __ldg(g.deg + u); }
+__device__ __forceinline__ bool hidden(const GraphRef &, int) { return false; }
+__device__ __forceinline__ bool hidden(const GraphView &g, int v) {
+    const int l = __ldg(g.label + v);
+    return l != INT_MAX && l >= g.self;
 }
 
 struct SearchOut {
@@ -230,19 +243,23 @@ __device__ __forceinline__ int first_unchecked(const uint64_t *pool, int size, i
 // first 128 slots are loaded before any visit (the visited-set updates would
 // otherwise order each 32-slot load after the previous chunk's), so a row
 // costs one global round trip.
-template <bool COHERENT>
-__device__ __forceinline__ void load_row_head(GraphRef g, int u, int (&vr)[4]) {
+template <class Gr>
+__device__ __forceinline__ void load_row_head(const Gr &g, int u, int (&vr)[4]) {
     const unsigned lane = lane_id();
     const int *row = g.adj + (int64_t)u * g.width;
+    const int tent = proposals_from(g, u);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         const int slot = c * 32 + (int)lane;
-        vr[c] = slot < g.width ? load_adj<COHERENT>(row + slot) : -1;
+        vr[c] = slot < g.width ? __ldg(row + slot) : -1;
     }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        if (c * 32 + (int)lane >= tent && vr[c] >= 0 && hidden(g, vr[c])) vr[c] = -1;
 }
 
-template <bool COHERENT>
-__device__ __forceinline__ int filter_row(GraphRef g, int u, const int (&vr)[4], WarpSmem &s, uint32_t hmask,
+template <class Gr>
+__device__ __forceinline__ int filter_row(const Gr &g, int u, const int (&vr)[4], WarpSmem &s, uint32_t hmask,
                                           int hshift) {
     const unsigned lane = lane_id();
     const int *row = g.adj + (int64_t)u * g.width;
@@ -255,9 +272,11 @@ __device__ __forceinline__ int filter_row(GraphRef g, int u, const int (&vr)[4],
         if (fresh) s.ids[m + __popc(bal & lanemask_lt())] = vr[c];
         m += __popc(bal);
     }
+    const int tent = proposals_from(g, u);
     for (int b = 128; b < g.width; b += 32) {  // rows wider than 128
         const int slot = b + (int)lane;
-        const int v = slot < g.width ? load_adj<COHERENT>(row + slot) : -1;
+        int v = slot < g.width ? __ldg(row + slot) : -1;
+        if (slot >= tent && v >= 0 && hidden(g, v)) v = -1;
         const bool fresh = v >= 0 && visit(s.hash, hmask, hshift, v);
         const unsigned bal = __ballot_sync(NSG_FULL, fresh);
         if (fresh) s.ids[m + __popc(bal & lanemask_lt())] = v;
@@ -272,11 +291,11 @@ __device__ __forceinline__ int filter_row(GraphRef g, int u, const int (&vr)[4],
 // first 128 slots are loaded before any visit (the visited-set updates would
 // otherwise order each 32-slot load after the previous chunk's), so a row
 // costs one global round trip.
-template <bool COHERENT>
-__device__ __forceinline__ int gather_row(GraphRef g, int u, WarpSmem &s, uint32_t hmask, int hshift) {
+template <class Gr>
+__device__ __forceinline__ int gather_row(const Gr &g, int u, WarpSmem &s, uint32_t hmask, int hshift) {
     int vr[4];
-    load_row_head<COHERENT>(g, u, vr);
-    return filter_row<COHERENT>(g, u, vr, s, hmask, hshift);
+    load_row_head(g, u, vr);
+    return filter_row(g, u, vr, s, hmask, hshift);
 }
 
 // The node Alg. 1 expands after keys[0..m) are merged into the pool, whose
@@ -397,7 +416,7 @@ __device__ SearchOut group_alg1(const D &dist, GraphRef g, int start, int L, War
                 const uint64_t e = s.pool[i];
                 __syncwarp();
                 if (lane == 0) s.pool[i] = e | CHK;
-                m = gather_row<false>(g, kid(e), s, hmask, hshift);
+                m = gather_row(g, kid(e), s, hmask, hshift);
 #if NSG_PF_ROWS
                 if (m > 0) dist.prefetch(s.ids, m);
 #endif
@@ -443,12 +462,12 @@ __device__ SearchOut group_alg1(const D &dist, GraphRef g, int start, int L, War
 // it is the predicted node the prepared row is used, otherwise (rare: see
 // predict_next) the speculative visited-set claims are taken back and the
 // row is read again.  The steps, keys and results are those of the plain loop.
-template <bool COLLECT, bool COHERENT, class D, bool STOP = false>
-__device__ SearchOut warp_alg1(const D &dist, GraphRef g, int start, int L, WarpSmem &s, uint32_t hmask,
+template <bool COLLECT, bool STOP = false, class Gr, class D>
+__device__ SearchOut warp_alg1(const D &dist, const Gr g, int start, int L, WarpSmem &s, uint32_t hmask,
                                int hshift, int max_steps, int excl, int C, int &csize, int *xlog = nullptr,
                                int xcap = 0, const StopCtx *stop = nullptr, uint64_t *xthr = nullptr,
                                const InitRand *init = nullptr) {
-    constexpr int PIPE = COHERENT ? 0 : NSG_PIPE;
+    constexpr int PIPE = NSG_PIPE;
     const unsigned lane = lane_id();
     SearchOut o;
     o.size = 0;
@@ -516,10 +535,10 @@ __device__ SearchOut warp_alg1(const D &dist, GraphRef g, int start, int L, Warp
         if (PIPE == 2 && u == pre_u) {
             m = pre_m;  // filtered before the previous merge
         } else if (PIPE == 1 && u == pre_u) {
-            m = filter_row<COHERENT>(g, u, vr, s, hmask, hshift);
+            m = filter_row(g, u, vr, s, hmask, hshift);
         } else {
             if (PIPE == 2 && pre_u >= 0) unvisit_all(s, hmask, hshift, pre_m);  // mispredicted
-            m = gather_row<COHERENT>(g, u, s, hmask, hshift);
+            m = gather_row(g, u, s, hmask, hshift);
         }
         pre_u = -1;
         last_m = m;
@@ -546,10 +565,10 @@ __device__ SearchOut warp_alg1(const D &dist, GraphRef g, int start, int L, Warp
                 if constexpr (PIPE == 2) {
                     // s.ids is free: the keys carry their ids
                     __syncwarp();
-                    pre_m = gather_row<COHERENT>(g, pre_u, s, hmask, hshift);
+                    pre_m = gather_row(g, pre_u, s, hmask, hshift);
                     if (pre_m > 0) dist.prefetch_all(s.ids, pre_m);
                 } else {
-                    load_row_head<COHERENT>(g, pre_u, vr);
+                    load_row_head(g, pre_u, vr);
                 }
             }
         }
