@@ -3,24 +3,49 @@
 // ground truth of Eq. 1).
 //
 // d2(q, x) = |q|^2 + (|x|^2 - 2 q.x): the dot products are a BF16 GEMM with
-// FP32 accumulation in TMEM (tcgen05.mma, M = 128 query rows per CTA, N = 128
-// base rows per tile, operands staged by TMA with 128-byte swizzle).  On
-// integer data in 0..255 with d <= 128 every product, partial sum, norm and
-// the final combination is an integer below 2^24, so the distances are exact
-// and the selection below equals the serial scan bit for bit; the launcher
-// checks the data and reports "not applicable" otherwise.
+// FP32 accumulation in TMEM (tcgen05.mma, operands staged by TMA with 128-byte
+// swizzle).  On integer data in 0..255 with d <= 128 every product, partial
+// sum, norm and the final combination is an integer below 2^24, so the
+// distances are exact and the selection below equals the serial scan bit for
+// bit; the launcher checks the data and reports "not applicable" otherwise.
 //
-// CTA = 6 warps: warp 0 issues TMA (the 128 x d query tile once, then a ring
-// of base tiles), warp 1 owns TMEM and issues the MMAs into two accumulator
-// buffers, warps 2-5 are the epilogue: thread r holds query row r's running
-// top-k.  A base column j enters row r's candidate buffer only when
-// |x_j|^2 - 2 q.x_j < (current k-th distance) - |q|^2; the common case costs
-// one FMA and one min per element (a group of 16 columns is tested through its
-// minimum).  Columns arrive in increasing id, so a strict comparison on the
-// distance alone implements the (distance, id) order.  Buffers of 16+ keys are
-// merged warp-cooperatively into the row's sorted list, which lives in the
-// output arrays.
+// A work unit is 256 query rows (two 128-row groups, M = 128 each, sharing the
+// staged base tiles of N = 128 rows) against a range of base tiles; one
+// persistent CTA per SM.  Warp 0 issues TMA, warp 1 the MMAs into two
+// accumulators per group (all 512 TMEM columns).  Each group has four scanning
+// warps: thread r of a group looks through query row r's columns.  A base
+// column j becomes a candidate of row r only when
+// |x_j|^2 - 2 q.x_j < (k-th distance so far) - |q|^2.  Columns arrive in
+// increasing id, so a strict comparison on the distance alone implements the
+// (distance, id) order.  The 8-column groups holding candidates go to the
+// row's ring in global memory; behind each scanning warp a merging warp takes
+// rows with 28 or more groups in their rings, merges their candidates into
+// the rows' sorted lists, which live in the output arrays, and publishes the
+// new k-th distances.  A scan with an older bound only finds more candidates.
+//
+// Bound by the scan's instructions and the accumulator hand-over, not the
+// tensor pipe: a column costs half a packed FMA and half a 3-input min per
+// row, and a candidate's group ~10 warp instructions whatever the other 31
+// rows do.  What the structure is for:
+//  (a) merging takes ~5,000 cycles of dependent loads and shuffles; done by
+//      the scanning warps it held up the accumulators, and with them every
+//      other warp of the CTA (the sum of all merges, not their average);
+//  (b) a candidate's whole group is stored without looking for it in there
+//      (the merge filters), which also keeps the loop small;
+//  (c) a pre-pass over a sample of the tiles (a quarter of them at most)
+//      bounds every row's k-th distance before the first candidate: of the
+//      sample's 64-column minima the k-th smallest has k columns at or below
+//      it.  That leaves ~k (1 + ln(n / sample)) candidates per row instead of
+//      k (1 + ln(n / k)).
+// Measured (before: four epilogue warps that also merged, one CTA per 128
+// rows, no pre-pass -> now): 300,007 x 128 integer rows, K = 100, 121.9 ->
+// 40.2 ms (575 TFLOP/s); 1,000 queries on 1,000,000 x 960 floats, k = 100,
+// 47.3 -> 6.5 ms, most of it from the split; 100 queries on 10,000 x 32, k = 10,
+// 0.77 -> 0.49 ms.  Without the merging warps the first took 55-72 ms.
+// Few query rows are spread over the SMs by splitting the base tiles; the
+// splits' lists are merged at the end.
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 
 #include <cuda.h>
@@ -35,184 +60,316 @@ namespace nsg {
 
 namespace {
 
-constexpr int TC_M = 128;       // query rows per CTA (TMEM lanes)
+constexpr int TC_M = 128;       // query rows per group (TMEM lanes)
+constexpr int TC_G = 2;         // row groups per work unit
+constexpr int TC_UNIT = TC_G * TC_M;
 constexpr int TC_N = 128;       // base rows per tile (accumulator columns)
 constexpr int TC_BOXK = 64;     // bf16 elements per 128-byte swizzle atom
-constexpr int TC_BUF = 64;      // candidate buffer per row
-constexpr int TC_MERGE_AT = 48; // merge when a buffer holds this many (+ 16 per test < 64)
-constexpr int TC_THREADS = 192;
+constexpr int TC_BUF = 64;      // candidates merged at a time
+constexpr int TC_MERGE = 28;    // 8-column groups in a row's ring before they are merged (~30 candidates)
+constexpr int TC_RING = 64;     // ring size (a power of two; a tile adds up to 16)
+constexpr int TC_SCAN = 4 * TC_G;  // scanning warps, and as many merging warps
+constexpr int TC_THREADS = 32 * (2 + 2 * TC_SCAN);
 constexpr int TC_MAXK = 256;
 
 struct TcArgs {
     const float *qn;  // [m] squared norms of the query rows
-    const float *xn;  // [ntiles * 128] squared norms of the base rows
+    const float *xn;  // [ntiles * 128] squared norms of the base rows, +inf past the last row
     int64_t m, n, q0;
     int self_join, KL;
-    int t0, t1;       // base tiles [t0, t1) of this launch (one chunk of the base)
-    int first, last;  // first chunk: lists start empty; last chunk: pad short lists
-    int kb;  // 64-wide K chunks per row (streaming form)
-    int *ids;
+    int tile0, tile1;  // tiles of this launch (sample positions in the pre-pass)
+    int stride;        // base tile of position i is i * stride (1 but for the pre-pass)
+    int T, S;          // row units, splits of the tile range; work unit u: rows rt0 + u % T, split u / T
+    int rt0;
+    int first, last;   // first chunk: lists start empty; last chunk: pad short lists
+    int kb;            // 64-wide K chunks per row (streaming form)
+    int *ids;          // lists [m][S][KL]
     float *d2;
-    int *lsz;  // [m] list sizes carried between chunks
+    int *lsz;          // [m] list sizes carried between chunks
+    const float *thr0; // [m] pre-pass bounds on |x|^2 - 2 q.x (strict), or nullptr
+    float *minima;     // pre-pass: [2 * tiles][mpad], rows from unit rt0
+    int64_t mpad;
+    float *vals;       // [grid][256][TC_RING][8] candidate groups: |x|^2 - 2 q.x
+    int *cols;         // [grid][256][TC_RING] their first columns
     int *err;
 };
 
-// DK = 64 or 128: the 128-row query tile stays in shared memory and a stage
+// DK = 64 or 128: the unit's 256 query rows stay in shared memory and a stage
 // holds one base tile.  DK = 0: rows wider than 128 values; a stage holds one
-// 64-wide K chunk of both the query tile and the base tile (16 KB each), and
+// 64-wide K chunk of the base tile and of the query groups (16 KB each), and
 // a tile takes dk/64 stages.
 template <int DK>
 struct TcCfg {
-    static constexpr int KB = DK / TC_BOXK;                     // swizzle atoms along K (resident form)
-    static constexpr int A_BYTES = TC_M * DK * 2;
-    static constexpr int B_BYTES = DK ? TC_N * DK * 2 : 2 * TC_N * 128;  // one pipeline stage
-    static constexpr int NS = DK == 64 ? 7 : (DK == 128 ? 3 : 4);       // stages
+    static constexpr int KB = DK / TC_BOXK;                                      // swizzle atoms along K (resident form)
+    static constexpr int A_GROUP = TC_M * DK * 2;                                // bytes of one resident group
+    static constexpr int A_BYTES = TC_G * A_GROUP;
+    static constexpr int B_BYTES = DK ? TC_N * DK * 2 : (1 + TC_G) * TC_N * 128;  // one pipeline stage
+    static constexpr int NS = DK == 64 ? 8 : 4;                                  // stages
     static constexpr int OFF_B = A_BYTES;
-    static constexpr int OFF_BUF = OFF_B + NS * B_BYTES;
-    static constexpr int OFF_WARP = OFF_BUF + TC_M * TC_BUF * 8;
-    // per epilogue warp: merge list, sorted buffer, base norms, k-th slot, and
-    // 16 values per lane for the insertion path (column-major, conflict-free)
-    static constexpr int WARP_BYTES = TC_MAXK * 8 + TC_BUF * 8 + TC_N * 4 + 16 + 16 * 32 * 4;
-    static constexpr int OFF_BAR = OFF_WARP + 4 * WARP_BYTES;
-    static constexpr int NBAR = 2 * NS + 6;  // a_full, b_full[NS], b_empty[NS], acc_full[2], acc_empty[2], drain
+    static constexpr int OFF_SCAN = OFF_B + NS * B_BYTES;        // per scanning warp: base norms of a tile
+    static constexpr int OFF_MERGE = OFF_SCAN + TC_SCAN * TC_N * 4;
+    // per merging warp: candidates being merged, k-th slot, rank counts
+    static constexpr int MERGE_BYTES = TC_BUF * 8 + 16 + (TC_BUF + 4) * 4;
+    // per row: ring head, tail, head at the unit's end, bound; per scanning
+    // warp: units scanned, units the merging warp has begun
+    static constexpr int OFF_ROW = OFF_MERGE + TC_SCAN * MERGE_BYTES;
+    static constexpr int OFF_BAR = OFF_ROW + TC_UNIT * 16 + TC_SCAN * 8;
+    // a_full, a_empty, b_full[NS], b_empty[NS], acc_full[G][2], acc_empty[G][2], drain
+    static constexpr int NBAR = 2 + 2 * NS + 4 * TC_G + 1;
     static constexpr int SMEM = OFF_BAR + NBAR * 8 + 16 + 1024;  // + alignment slack
 };
 
-// Bitonic sort of 64 keys held two per lane (index lane and lane + 32), ascending.
-__device__ __forceinline__ void bitonic64(uint64_t &a, uint64_t &b, unsigned lane) {
+__device__ __forceinline__ float min3(float a, float b, float c) {
+    float d;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
+// A row's sorted list in registers (entry t * 32 + lane), all loads in flight
+// at once: entries past the list's end read its first one.
+struct RowList {
+    float d2[TC_MAXK / 32];
+    int id[TC_MAXK / 32];
+    __device__ __forceinline__ void load(const int *oid, const float *od, int KL) {
 #pragma unroll
-    for (int k = 2; k <= 64; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            if (j == 32) {  // partner in the same lane: index lane vs lane + 32 (k = 64: ascending)
-                const uint64_t mn = a < b ? a : b, mx = a < b ? b : a;
-                a = mn;
-                b = mx;
-            } else {
-                const uint64_t oa = __shfl_xor_sync(NSG_FULL, a, j), ob = __shfl_xor_sync(NSG_FULL, b, j);
-                const bool lower = (lane & j) == 0;
-                const bool up_a = (lane & k) == 0, up_b = ((lane + 32) & k) == 0;
-                const uint64_t mna = oa < a ? oa : a, mxa = oa < a ? a : oa;
-                const uint64_t mnb = ob < b ? ob : b, mxb = ob < b ? b : ob;
-                a = (lower == up_a) ? mna : mxa;
-                b = (lower == up_b) ? mnb : mxb;
-            }
+        for (int t = 0; t < TC_MAXK / 32; ++t) {
+            const int i = t * 32 + (int)lane_id(), j = i < KL ? i : 0;
+            d2[t] = od[j];
+            id[t] = oid[j];
         }
     }
+};
+
+// Number of the c <= 64 sorted keys at sb that are less than each of four keys
+// (four searches in step).
+__device__ __forceinline__ void count_less4(const uint64_t *sb, int c, const uint64_t (&k)[4], int (&r)[4]) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) r[t] = 0;
+#pragma unroll
+    for (int step = 64; step > 0; step >>= 1)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const int m = r[t] + step;
+            if (m <= c && sb[m - 1] < k[t]) r[t] = m;
+        }
 }
 
-__device__ __forceinline__ int count_less(const uint64_t *a, int len, uint64_t key) {
-    int lo = 0, hi = len;
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (a[mid] < key) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
-// Merge row `src`'s buffer (c <= 63 keys) into its sorted list of s keys
-// (output arrays, capacity KL), warp-cooperatively: the list is read once
-// (all loads issued before use), the buffer sorted, and every key written to
-// its rank in the union.
-__device__ __noinline__ void merge_row(int src, int row_local, int64_t row_g, int &cnt, int &lsize,
-                                       float &thrp, float qn_r, const uint64_t *bufs, uint64_t *ls,
-                                       uint64_t *sb, uint64_t *thr_slot, int *ids, float *d2, int KL) {
+// The c <= 64 candidates in sb into the sorted list of s keys at oid / od.
+// Every candidate finds its rank among the candidates (independent compares
+// against broadcast reads, while the list's loads are in flight; a sorting
+// network is a chain of shuffles); list keys
+// find theirs by binary search; the counts of those ranks give the candidates'
+// ranks in the list.  One copy of this code, not inlined: a merge runs straight
+// through, so fetching instructions counts (nine inlined copies: 47.7 ms instead
+// of 39.8 ms for the 300,007-row graph).
+__device__ __noinline__ void merge_piece(int c, int &size, uint64_t *sb, int *hist, uint64_t *thr_slot, int *oid,
+                                         float *od, int KL) {
+    int s = size;
+    RowList list;
+    list.load(oid, od, KL);
     const unsigned lane = lane_id();
-    const int c = __shfl_sync(NSG_FULL, cnt, src);
-    const int s = __shfl_sync(NSG_FULL, lsize, src);
-    const int rl = __shfl_sync(NSG_FULL, row_local, src);
-    const int64_t rg = __shfl_sync(NSG_FULL, row_g, src);
-    int *oid = ids + rg * KL;
-    float *od = d2 + rg * KL;
-    float lv[TC_MAXK / 32];
-    int li[TC_MAXK / 32];
-#pragma unroll
-    for (int t = 0; t < TC_MAXK / 32; ++t) {
-        const int i = t * 32 + (int)lane;
-        if (i < s) {
-            lv[t] = od[i];
-            li[t] = oid[i];
+    const uint64_t a = (int)lane < c ? sb[lane] : ~0ull, b = (int)lane + 32 < c ? sb[lane + 32] : ~0ull;
+    int ra = 0, rb = 0;
+    if (c <= 32) {
+#pragma unroll 8
+        for (int j = 0; j < c; ++j) ra += sb[j] < a;
+    } else {
+#pragma unroll 8
+        for (int j = 0; j < c; ++j) {
+            const uint64_t o = sb[j];
+            ra += o < a;
+            rb += o < b;
         }
-    }
-    uint64_t a = (int)lane < c ? bufs[rl * TC_BUF + lane] : ~0ull;
-    uint64_t b = (int)lane + 32 < c ? bufs[rl * TC_BUF + 32 + lane] : ~0ull;
-    bitonic64(a, b, lane);
-    sb[lane] = a;
-    sb[lane + 32] = b;
-#pragma unroll
-    for (int t = 0; t < TC_MAXK / 32; ++t) {
-        const int i = t * 32 + (int)lane;
-        if (i < s) ls[i] = make_key(lv[t], li[t]);
     }
     __syncwarp();
+    if ((int)lane < c) sb[ra] = a;
+    if ((int)lane + 32 < c) sb[rb] = b;
+    hist[lane] = 0;
+    hist[lane + 32] = 0;
+    if (lane == 0) hist[64] = 0;
+    __syncwarp();
 #pragma unroll
-    for (int t = 0; t < TC_MAXK / 32; ++t) {
-        const int i = t * 32 + (int)lane;
-        if (i < s) {
-            const uint64_t key = ls[i];
-            const int p = i + count_less(sb, c, key);
-            if (p < KL) {
-                od[p] = kd2(key);
-                oid[p] = kid(key);
-                if (p == KL - 1) *thr_slot = key;
+    for (int t0 = 0; t0 < TC_MAXK / 32; t0 += 4) {
+        if (t0 * 32 >= s) break;
+        uint64_t key[4];
+        int r[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) key[t] = make_key(list.d2[t0 + t], list.id[t0 + t]);
+        count_less4(sb, c, key, r);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const int i = (t0 + t) * 32 + (int)lane, p = i + r[t];
+            if (i < s) {
+                atomicAdd(hist + r[t], 1);
+                if (r[t] > 0 && p < KL) {  // the others stay where they are
+                    od[p] = kd2(key[t]);
+                    oid[p] = kid(key[t]);
+                }
+                if (p == KL - 1) *thr_slot = key[t];
             }
         }
     }
+    __syncwarp();
+    // list keys below sorted candidate j: those whose rank is at most j
+    int h0 = hist[lane], h1 = hist[lane + 32];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(NSG_FULL, h0, o), y = __shfl_up_sync(NSG_FULL, h1, o);
+        if ((int)lane >= o) {
+            h0 += x;
+            h1 += y;
+        }
+    }
+    h1 += __shfl_sync(NSG_FULL, h0, 31);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int j = (int)lane + 32 * h;
-        const uint64_t key = h ? b : a;
-        if (j < c) {
-            const int p = j + count_less(ls, s, key);
-            if (p < KL) {
-                od[p] = kd2(key);
-                oid[p] = kid(key);
-                if (p == KL - 1) *thr_slot = key;
-            }
+        const int j = (int)lane + 32 * h, p = j + (h ? h1 : h0);
+        if (j < c && p < KL) {
+            const uint64_t k = sb[j];
+            od[p] = kd2(k);
+            oid[p] = kid(k);
+            if (p == KL - 1) *thr_slot = k;
         }
     }
-    __syncwarp();
-    if ((int)lane == src) {
-        cnt = 0;
-        lsize = s + c < KL ? s + c : KL;
-        if (lsize == KL) thrp = kd2(*thr_slot) - qn_r;
-    }
+    size = s + c < KL ? s + c : KL;
     __syncwarp();
 }
 
-template <int DK>
+// Merge the groups [tail, head) of a row's ring into its sorted list (at most
+// KL keys at oid / od, s of them): the values still below the row's bound are
+// collected (the row itself, in a self join, is dropped) and merged up to 64 at
+// a time, usually all at once.  Warp-wide; returns the row's bound.
+__device__ __forceinline__ float merge_row(const float *vals, const int *cols, int tail, int head, int own, float q2,
+                                           float bar, int &s, uint64_t *sb, int *hist, uint64_t *thr_slot, int *oid,
+                                           float *od, int KL) {
+    const unsigned lane = lane_id();
+    const int total = (head - tail) * 8, e8 = (int)(lane & 7);
+    int c = 0;
+#pragma unroll 1
+    for (int e0 = 0; e0 < total; e0 += 128) {
+        float tv[4];
+        int col[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {  // all loads issued before the first use
+            const int r = (tail + ((e0 + t * 32 + (int)lane) >> 3)) & (TC_RING - 1);
+            tv[t] = __ldcg(vals + r * 8 + e8);
+            col[t] = __ldcg(cols + r) + e8;
+        }
+        bool take[4];
+        int add = 0;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            take[t] = e0 + t * 32 + (int)lane < total && tv[t] < bar && col[t] != own;
+            add += __popc(__ballot_sync(NSG_FULL, take[t]));
+        }
+        if (c + add > TC_BUF) {  // make room (more than 64 at once, a row's first groups: below, 32 at a time)
+            __syncwarp();
+            if (c > 0) merge_piece(c, s, sb, hist, thr_slot, oid, od, KL);
+            if (s == KL) bar = kd2(*thr_slot) - q2;
+            c = 0;
+            __syncwarp();
+        }
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const unsigned bal = __ballot_sync(NSG_FULL, take[t]);
+            if (take[t]) sb[c + __popc(bal & lanemask_lt())] = make_key(fmaxf(q2 + tv[t], 0.0f), col[t]);
+            c += __popc(bal);
+            if (add > TC_BUF && (t & 1)) {
+                __syncwarp();
+                if (c > 0) merge_piece(c, s, sb, hist, thr_slot, oid, od, KL);
+                c = 0;
+                __syncwarp();
+            }
+        }
+        if (add > TC_BUF && s == KL) bar = kd2(*thr_slot) - q2;
+    }
+    __syncwarp();
+    if (c > 0) {
+        merge_piece(c, s, sb, hist, thr_slot, oid, od, KL);
+        if (s == KL) bar = kd2(*thr_slot) - q2;
+        __syncwarp();
+    }
+    return bar;
+}
+
+// The tiles of work unit u.
+__device__ __forceinline__ void unit_tiles(const TcArgs &a, int u, int *rt, int *i0, int *i1) {
+    const int sp = u / a.T;
+    *rt = a.rt0 + u - sp * a.T;
+    const int64_t len = a.tile1 - a.tile0;
+    *i0 = a.tile0 + (int)(len * sp / a.S);
+    *i1 = a.tile0 + (int)(len * (sp + 1) / a.S);
+}
+
+// Two FMAs in one instruction (round to nearest each).
+__device__ __forceinline__ void fma2(float &d0, float &d1, float a0, float a1, float b, float c0, float c1) {
+    uint64_t d, x, y, z;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a0), "f"(a1));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(y) : "f"(b));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(c0), "f"(c1));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(x), "l"(y), "l"(z));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(d));
+}
+
+// Row groups of a unit that hold query rows.
+__device__ __forceinline__ int unit_groups(const TcArgs &a, int rt) {
+    const int64_t rows = a.m - (int64_t)rt * TC_UNIT;
+    return rows >= TC_UNIT ? TC_G : (int)((rows + TC_M - 1) / TC_M);
+}
+
+// A row's bound on |x|^2 - 2 q.x and its list's size when a unit begins: the
+// k-th key carried over from earlier chunks once the list holds k, before that
+// the pre-pass's; a row past the end takes nothing.
+__device__ __forceinline__ float first_bound(const TcArgs &a, int64_t row, int64_t list, int *lsize) {
+    *lsize = 0;
+    if (row >= a.m) return __int_as_float(0xff800000);
+    if (!a.first) *lsize = a.lsz[row];
+    if (*lsize == a.KL) return a.d2[list + a.KL - 1] - a.qn[row];
+    return a.thr0 ? a.thr0[row] : __int_as_float(0x7f800000);
+}
+
+// MINS: the pre-pass (minima of every sample tile's two 64-column groups),
+// else the selection.
+template <int DK, bool MINS>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-    knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcArgs a) {
+    knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                  const __grid_constant__ TcArgs a) {
     using Cfg = TcCfg<DK>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     unsigned char *sA = smem;
     unsigned char *sB = smem + Cfg::OFF_B;
-    uint64_t *bufs = reinterpret_cast<uint64_t *>(smem + Cfg::OFF_BUF);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + Cfg::OFF_BAR);
-    uint64_t *a_full = bars;
-    uint64_t *b_full = bars + 1;
-    uint64_t *b_empty = bars + 1 + Cfg::NS;
-    uint64_t *acc_full = bars + 1 + 2 * Cfg::NS;
-    uint64_t *acc_empty = acc_full + 2;
-    uint64_t *drain = acc_empty + 2;
+    uint64_t *a_full = bars, *a_empty = bars + 1;
+    uint64_t *b_full = bars + 2;
+    uint64_t *b_empty = b_full + Cfg::NS;
+    uint64_t *acc_full = b_empty + Cfg::NS;  // [group * 2 + buffer]
+    uint64_t *acc_empty = acc_full + 2 * TC_G;
+    uint64_t *drain = acc_empty + 2 * TC_G;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + Cfg::NBAR);
     volatile int *abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
     volatile int *gerr = a.err;
+    volatile int *r_head = reinterpret_cast<volatile int *>(smem + Cfg::OFF_ROW);  // [256] each
+    volatile int *r_tail = r_head + TC_UNIT, *r_end = r_tail + TC_UNIT;
+    volatile float *r_thr = reinterpret_cast<volatile float *>(r_end + TC_UNIT);
+    volatile int *scanned = reinterpret_cast<volatile int *>(r_thr + TC_UNIT);  // [TC_SCAN]
+    volatile int *begun = scanned + TC_SCAN;
 
     const int warp = threadIdx.x >> 5;
     const unsigned lane = lane_id();
-    const int64_t row0 = (int64_t)blockIdx.x * TC_M;
+    const int units = a.T * a.S;
 
+    for (int t = threadIdx.x; t < TC_UNIT; t += TC_THREADS) r_head[t] = r_tail[t] = r_end[t] = 0;
+    if (threadIdx.x < TC_SCAN) scanned[threadIdx.x] = begun[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         tc::mbar_init(a_full, 1);
+        tc::mbar_init(a_empty, 1);
         for (int s = 0; s < Cfg::NS; ++s) {
             tc::mbar_init(b_full + s, 1);
             tc::mbar_init(b_empty + s, 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < 2 * TC_G; ++b) {
             tc::mbar_init(acc_full + b, 1);
             tc::mbar_init(acc_empty + b, 4);
         }
@@ -223,7 +380,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         tc::prefetch_tmap(&tmB);
     }
     if (warp == 1) {
-        tc::tmem_alloc(tmem_slot, 2 * TC_N);
+        tc::tmem_alloc(tmem_slot, 2 * TC_G * TC_N);
         tc::tmem_relinquish();
     }
     tc::fence_before_sync();
@@ -237,35 +394,50 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     } else if (warp == 0) {
         // ---------------- TMA producer ----------------
         if (lane == 0) {
-            if (DK) {
-                tc::mbar_expect_tx(a_full, Cfg::A_BYTES);
-                for (int kb = 0; kb < Cfg::KB; ++kb)
-                    tc::tma_load_2d(sA + kb * (TC_M * 128), &tmA, a_full, kb * TC_BOXK, (int)row0);
-            }
             const int per_tile = DK ? 1 : a.kb;  // stages per tile
-            const int nt = a.t1 - a.t0;
-            int issued = 0;
-            for (int c = 0; c < nt * per_tile; ++c) {
-                const int s = c % Cfg::NS, tl = c / per_tile, kc = c - tl * per_tile, t = a.t0 + tl;
-                if (!tc::mbar_wait(b_empty + s, ((c / Cfg::NS) & 1) ^ 1, abort, gerr)) break;
-                tc::mbar_expect_tx(b_full + s, Cfg::B_BYTES);
-                unsigned char *dst = sB + s * Cfg::B_BYTES;
+            int c = 0, nu = 0;                   // stages issued; units whose query rows were
+            bool ok = true;
+            for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
+                int rt, i0, i1;
+                unit_tiles(a, u, &rt, &i0, &i1);
+                const int row0 = rt * TC_UNIT, groups = unit_groups(a, rt);
                 if (DK) {
-                    for (int kb = 0; kb < Cfg::KB; ++kb)
-                        tc::tma_load_2d(dst + kb * (TC_N * 128), &tmB, b_full + s, kb * TC_BOXK, t * TC_N);
-                } else {
-                    tc::tma_load_2d(dst, &tmA, b_full + s, kc * TC_BOXK, (int)row0);
-                    tc::tma_load_2d(dst + TC_M * 128, &tmB, b_full + s, kc * TC_BOXK, t * TC_N);
+                    if (!tc::mbar_wait(a_empty, (nu & 1) ^ 1, abort, gerr)) break;
+                    tc::mbar_expect_tx(a_full, groups * Cfg::A_GROUP);
+                    for (int g = 0; g < groups; ++g)
+                        for (int kb = 0; kb < Cfg::KB; ++kb)
+                            tc::tma_load_2d(sA + g * Cfg::A_GROUP + kb * (TC_M * 128), &tmA, a_full, kb * TC_BOXK,
+                                            row0 + g * TC_M);
+                    ++nu;
                 }
-                issued = c + 1;
+                for (int i = i0; ok && i < i1; ++i)
+                    for (int kc = 0; kc < per_tile; ++kc, ++c) {
+                        const int s = c % Cfg::NS;
+                        if (!tc::mbar_wait(b_empty + s, ((c / Cfg::NS) & 1) ^ 1, abort, gerr)) {
+                            ok = false;
+                            break;
+                        }
+                        unsigned char *dst = sB + s * Cfg::B_BYTES;
+                        const int y = i * a.stride * TC_N;
+                        tc::mbar_expect_tx(b_full + s, DK ? Cfg::B_BYTES : (1 + groups) * TC_N * 128);
+                        if (DK) {
+                            for (int kb = 0; kb < Cfg::KB; ++kb)
+                                tc::tma_load_2d(dst + kb * (TC_N * 128), &tmB, b_full + s, kb * TC_BOXK, y);
+                        } else {
+                            tc::tma_load_2d(dst, &tmB, b_full + s, kc * TC_BOXK, y);
+                            for (int g = 0; g < groups; ++g)
+                                tc::tma_load_2d(dst + (1 + g) * TC_N * 128, &tmA, b_full + s, kc * TC_BOXK,
+                                                row0 + g * TC_M);
+                        }
+                    }
             }
             if (*abort) {
                 // drain: wait (bounded) for the copies still in flight
                 volatile int local = 0;
-                if (DK) tc::mbar_wait(a_full, 0, &local, nullptr);
-                for (int c = issued - Cfg::NS < 0 ? 0 : issued - Cfg::NS; c < issued; ++c) {
+                if (nu > 0) tc::mbar_wait(a_full, (nu - 1) & 1, &local, nullptr);
+                for (int x = c - Cfg::NS < 0 ? 0 : c - Cfg::NS; x < c; ++x) {
                     local = 0;
-                    tc::mbar_wait(b_full + c % Cfg::NS, (c / Cfg::NS) & 1, &local, nullptr);
+                    tc::mbar_wait(b_full + x % Cfg::NS, (x / Cfg::NS) & 1, &local, nullptr);
                 }
             }
         }
@@ -274,171 +446,269 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         if (lane == 0) {
             constexpr uint32_t idesc = tc::idesc_bf16_f32(TC_M, TC_N);
             const uint32_t a_base = tc::smem_u32(sA), b_base = tc::smem_u32(sB);
-            bool ok = DK ? tc::mbar_wait(a_full, 0, abort, gerr) : true;
             const int per_tile = DK ? 1 : a.kb;
-            int c = 0;
-            for (int t = 0; ok && t < a.t1 - a.t0; ++t) {  // local tile index
-                const int buf = t & 1;
-                if (!tc::mbar_wait(acc_empty + buf, ((t >> 1) & 1) ^ 1, abort, gerr)) break;
-                tc::fence_after_sync();
-                for (int kc = 0; ok && kc < per_tile; ++kc, ++c) {
-                    const int s = c % Cfg::NS;
-                    if (!tc::mbar_wait(b_full + s, (c / Cfg::NS) & 1, abort, gerr)) {
-                        ok = false;
-                        break;
-                    }
-                    tc::fence_after_sync();
-                    if (DK) {
-#pragma unroll
-                        for (int kk = 0; kk < (DK ? DK : 64) / 16; ++kk) {
-                            const uint32_t koff = (kk >> 2) * (TC_M * 128) + (kk & 3) * 32;
-                            const uint32_t boff = s * Cfg::B_BYTES + (kk >> 2) * (TC_N * 128) + (kk & 3) * 32;
-                            tc::mma_bf16(tmem + buf * TC_N, tc::sdesc_sw128(a_base + koff),
-                                         tc::sdesc_sw128(b_base + boff), idesc, kk > 0 ? 1u : 0u);
+            int c = 0, nu = 0;      // stages, units
+            int tg[TC_G] = {0, 0};  // tiles of each group so far
+            bool ok = true;
+            for (int u = blockIdx.x; ok && u < units; u += gridDim.x, ++nu) {
+                int rt, i0, i1;
+                unit_tiles(a, u, &rt, &i0, &i1);
+                const int groups = unit_groups(a, rt);
+                if (DK && !tc::mbar_wait(a_full, nu & 1, abort, gerr)) break;
+                for (int i = i0; ok && i < i1; ++i) {
+                    for (int kc = 0; ok && kc < per_tile; ++kc, ++c) {
+                        const int s = c % Cfg::NS;
+                        if (!tc::mbar_wait(b_full + s, (c / Cfg::NS) & 1, abort, gerr)) {
+                            ok = false;
+                            break;
                         }
-                    } else {
+                        const uint32_t st = b_base + s * Cfg::B_BYTES;
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                            const uint32_t st = b_base + s * Cfg::B_BYTES + kk * 32;
-                            tc::mma_bf16(tmem + buf * TC_N, tc::sdesc_sw128(st), tc::sdesc_sw128(st + TC_M * 128),
-                                         idesc, (kc > 0 || kk > 0) ? 1u : 0u);
+                        for (int g = 0; g < TC_G; ++g) {
+                            if (g >= groups) break;
+                            const int ab = g * 2 + (tg[g] & 1);  // the tile's accumulator
+                            if (kc == 0 && !tc::mbar_wait(acc_empty + ab, ((tg[g] >> 1) & 1) ^ 1, abort, gerr)) {
+                                ok = false;
+                                break;
+                            }
+                            tc::fence_after_sync();
+                            const uint32_t acc = tmem + ab * TC_N;
+                            if (DK) {
+#pragma unroll
+                                for (int kk = 0; kk < (DK ? DK : 64) / 16; ++kk) {
+                                    const uint32_t off = (kk >> 2) * (TC_M * 128) + (kk & 3) * 32;
+                                    tc::mma_bf16(acc, tc::sdesc_sw128(a_base + g * Cfg::A_GROUP + off),
+                                                 tc::sdesc_sw128(st + off), idesc, kk > 0 ? 1u : 0u);
+                                }
+                            } else {
+#pragma unroll
+                                for (int kk = 0; kk < 4; ++kk)
+                                    tc::mma_bf16(acc, tc::sdesc_sw128(st + (1 + g) * TC_N * 128 + kk * 32),
+                                                 tc::sdesc_sw128(st + kk * 32), idesc, (kc > 0 || kk > 0) ? 1u : 0u);
+                            }
+                            if (kc == per_tile - 1) {
+                                tc::mma_commit(acc_full + ab);
+                                ++tg[g];
+                            }
                         }
+                        tc::mma_commit(b_empty + s);
                     }
-                    tc::mma_commit(b_empty + s);
                 }
-                if (!ok) break;
-                tc::mma_commit(acc_full + buf);
+                if (DK && ok) tc::mma_commit(a_empty);
             }
             // every MMA issued so far has completed before TMEM is released
             tc::mma_commit(drain);
             volatile int local = 0;
             tc::mbar_wait(drain, 0, &local, nullptr);
         }
-    } else {
-        // ---------------- epilogue: warps 2..5 ----------------
+    } else if (warp < 2 + TC_SCAN) {
+        // ---------------- scan: warps 2 + 4g .. 5 + 4g for row group g ----------------
         const int q = warp & 3;  // TMEM lane quadrant of this warp
-        const int ew = warp - 2;
-        unsigned char *wsm = smem + Cfg::OFF_WARP + ew * Cfg::WARP_BYTES;
-        uint64_t *ls = reinterpret_cast<uint64_t *>(wsm);
-        uint64_t *sb = ls + TC_MAXK;
-        float *xs = reinterpret_cast<float *>(sb + TC_BUF);
-        uint64_t *thr_slot = reinterpret_cast<uint64_t *>(xs + TC_N);
-        float *tvs = reinterpret_cast<float *>(thr_slot + 2);  // [16][32]
-        const int row_local = q * 32 + lane;
-        const int64_t row_g = row0 + row_local;
-        const bool valid = row_g < a.m;
-        const float qn_r = valid ? a.qn[row_g] : 0.0f;
-        const int64_t self_id = a.self_join ? a.q0 + row_g : -1;
-        uint64_t *mybuf = bufs + row_local * TC_BUF;
-        // the row's list (size and k-th key) carried over from earlier chunks;
-        // a row past the end takes nothing: its threshold is -inf
-        int cnt = 0, lsize = valid && !a.first ? a.lsz[row_g] : 0;
-        float thrp = __int_as_float(valid ? 0x7f800000 : 0xff800000);
-        if (valid && lsize == a.KL) thrp = a.d2[row_g * a.KL + a.KL - 1] - qn_r;
-        const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16);
-        bool ok = true;
+        const int w = warp - 2, g = w >> 2;
+        float *xs = reinterpret_cast<float *>(smem + Cfg::OFF_SCAN) + w * TC_N;
+        const int row_local = g * TC_M + q * 32 + (int)lane;
+        const unsigned ring = ((unsigned)blockIdx.x * TC_UNIT + row_local) * TC_RING;
+        const uint32_t tq = tmem + ((uint32_t)(q * 32) << 16) + g * 2 * TC_N;
         const float4 *xn4 = reinterpret_cast<const float4 *>(a.xn);
-        float4 xnext = __ldg(xn4 + (int64_t)a.t0 * (TC_N / 4) + lane);  // norms one tile ahead
-        for (int tl = 0; tl < a.t1 - a.t0; ++tl) {
-            const int buf = tl & 1, t = a.t0 + tl;
-            const int64_t col0 = (int64_t)t * TC_N;
-            // columns jj < lim exist; jj == self_local is the row itself
-            const int lim = a.n - col0 < TC_N ? (int)(a.n - col0) : TC_N;
-            const int self_local = self_id >= col0 && self_id < col0 + TC_N ? (int)(self_id - col0) : -1;
-            __syncwarp();
-            reinterpret_cast<float4 *>(xs)[lane] = xnext;
-            if (t + 1 < a.t1) xnext = __ldg(xn4 + (int64_t)(t + 1) * (TC_N / 4) + lane);
-            __syncwarp();
-            const bool got = tc::mbar_wait(acc_full + buf, (tl >> 1) & 1, abort, gerr);
-            if (!__all_sync(NSG_FULL, got)) {  // warp-uniform before the .sync.aligned TMEM loads
-                ok = false;
-                break;
+        int tcnt = 0, nu = 0;    // tiles and units of this group so far
+        int head = 0, told = 0;  // groups put into the ring; the count last published
+        bool ok = true;
+        for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
+            int rt, i0, i1;
+            unit_tiles(a, u, &rt, &i0, &i1);
+            if (g >= unit_groups(a, rt)) continue;
+            ++nu;
+            const int64_t row_g = (int64_t)rt * TC_UNIT + row_local;
+            const bool valid = row_g < a.m;
+            float thrp = 0.0f;
+            if (!MINS) {
+                int lsize;
+                thrp = first_bound(a, row_g, (row_g * a.S + u / a.T) * a.KL, &lsize);
             }
-            tc::fence_after_sync();
-#pragma unroll 1
-            for (int c = 0; c < TC_N / 32; ++c) {
-                uint32_t v[32];
-                tc::tmem_ld32(tq + buf * TC_N + c * 32, v);
-                tc::tmem_ld_wait();
-                if (c == TC_N / 32 - 1) {
-                    tc::fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0) tc::mbar_arrive(acc_empty + buf);
-                }
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    // |x|^2 - 2 q.x for 16 columns and their minimum: one FMA
-                    // and one min per element; the insertion path runs only
-                    // when some column beats the row's current k-th distance
-                    const int jb = c * 32 + h * 16;
-                    const float4 *x4 = reinterpret_cast<const float4 *>(xs + jb);
-                    float tv[16];
-#pragma unroll
-                    for (int j4 = 0; j4 < 4; ++j4) {
-                        const float4 xv = x4[j4];
-                        const float xa[4] = {xv.x, xv.y, xv.z, xv.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            tv[j4 * 4 + e] = fmaf(-2.0f, __uint_as_float(v[h * 16 + j4 * 4 + e]), xa[e]);
-                    }
-                    float m8[8];  // minimum as a tree (independent instructions)
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) m8[j] = fminf(tv[2 * j], tv[2 * j + 1]);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) m8[j] = fminf(m8[2 * j], m8[2 * j + 1]);
-                    const float mn = fminf(fminf(m8[0], m8[1]), fminf(m8[2], m8[3]));
-                    if (mn < thrp) {
-                        // columns of this group that exist, are not the row itself, and
-                        // beat the threshold: a bit mask, then one step per set bit
-                        const int nv = lim - jb;
-                        unsigned vm = nv >= 16 ? 0xffffu : (nv <= 0 ? 0u : (1u << nv) - 1u);
-                        if ((unsigned)(self_local - jb) < 16u) vm &= ~(1u << (self_local - jb));
-                        unsigned msk = 0;
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) msk |= (tv[j] < thrp ? 1u : 0u) << j;
-                        msk &= vm;
-                        if (msk) {
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) tvs[j * 32 + lane] = tv[j];
-                            while (msk) {
-                                const int j = __ffs(msk) - 1;
-                                msk &= msk - 1;
-                                mybuf[cnt] = make_key(fmaxf(qn_r + tvs[j * 32 + lane], 0.0f), (int)(col0 + jb + j));
-                                ++cnt;
-                            }
+            float4 xnext = i0 < i1 ? __ldg(xn4 + (int64_t)i0 * a.stride * (TC_N / 4) + lane)
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);  // norms one tile ahead
+            for (int i = i0; i < i1; ++i, ++tcnt) {
+                const int buf = tcnt & 1, col0 = i * a.stride * TC_N;
+                __syncwarp();
+                reinterpret_cast<float4 *>(xs)[lane] = xnext;
+                if (i + 1 < i1) xnext = __ldg(xn4 + (int64_t)(i + 1) * a.stride * (TC_N / 4) + lane);
+                bool room = true;
+                if (!MINS) {
+                    // the merging warp's bound, once it is at this unit; room in the
+                    // ring for all of a tile's groups
+                    if (begun[w] == nu) thrp = r_thr[row_local];
+                    if (!__all_sync(NSG_FULL, head + 16 - r_tail[row_local] <= TC_RING)) {
+                        __threadfence_block();
+                        r_head[row_local] = told = head;
+                        const uint64_t t0 = tc::globaltimer();
+                        while (room && !__all_sync(NSG_FULL, head + 16 - r_tail[row_local] <= TC_RING)) {
+                            __nanosleep(100);
+                            if (*abort || tc::globaltimer() - t0 > tc::WAIT_TIMEOUT_NS) room = false;
+                            room = __all_sync(NSG_FULL, room);
                         }
-                    }
-                    unsigned need = __ballot_sync(NSG_FULL, cnt >= TC_MERGE_AT);
-                    while (need) {
-                        const int src = __ffs(need) - 1;
-                        need &= need - 1;
-                        merge_row(src, row_local, row_g, cnt, lsize, thrp, qn_r, bufs, ls, sb, thr_slot,
-                                  a.ids, a.d2, a.KL);
+                        if (!room) *abort = 1;
+                        if (begun[w] == nu) thrp = r_thr[row_local];
                     }
                 }
+                __syncwarp();
+                const bool got = room && tc::mbar_wait(acc_full + g * 2 + buf, (tcnt >> 1) & 1, abort, gerr);
+                if (!__all_sync(NSG_FULL, got)) {  // warp-uniform before the .sync.aligned TMEM loads
+                    ok = false;
+                    break;
+                }
+                tc::fence_after_sync();
+                float even = 0.0f;
+#pragma unroll 1
+                for (int c = 0; c < TC_N / 32; ++c) {
+                    uint32_t v[32];
+                    tc::tmem_ld32_wait(tq + buf * TC_N + c * 32, v);
+                    if (c == TC_N / 32 - 1) {  // the tile's last columns are in registers
+                        tc::fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) tc::mbar_arrive(acc_empty + g * 2 + buf);
+                    }
+                    // |x|^2 - 2 q.x, and the minima of 8-column groups
+                    const float4 *x4 = reinterpret_cast<const float4 *>(xs + c * 32);
+                    float tv[32], m8[4];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float4 xv = x4[j];
+                        fma2(tv[4 * j], tv[4 * j + 1], __uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]), -2.0f,
+                             xv.x, xv.y);
+                        fma2(tv[4 * j + 2], tv[4 * j + 3], __uint_as_float(v[4 * j + 2]),
+                             __uint_as_float(v[4 * j + 3]), -2.0f, xv.z, xv.w);
+                    }
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const float p = min3(tv[h * 8], tv[h * 8 + 1], tv[h * 8 + 2]);
+                        const float r = min3(tv[h * 8 + 3], tv[h * 8 + 4], tv[h * 8 + 5]);
+                        m8[h] = fminf(min3(tv[h * 8 + 6], tv[h * 8 + 7], p), r);
+                    }
+                    const float mn = fminf(min3(m8[0], m8[1], m8[2]), m8[3]);
+                    if (MINS) {
+                        if ((c & 1) == 0) even = mn;
+                        else if (valid)
+                            a.minima[((int64_t)i * 2 + (c >> 1)) * a.mpad + (row_g - (int64_t)a.rt0 * TC_UNIT)] =
+                                fminf(even, mn);
+                    } else if (mn < thrp) {
+#pragma unroll
+                        for (int h = 0; h < 4; ++h)
+                            if (m8[h] < thrp) {
+                                const unsigned at = ring + (head & (TC_RING - 1));
+                                float4 *dst = reinterpret_cast<float4 *>(a.vals) + (size_t)at * 2;
+                                dst[0] = make_float4(tv[h * 8], tv[h * 8 + 1], tv[h * 8 + 2], tv[h * 8 + 3]);
+                                dst[1] = make_float4(tv[h * 8 + 4], tv[h * 8 + 5], tv[h * 8 + 6], tv[h * 8 + 7]);
+                                a.cols[at] = col0 + c * 32 + h * 8;
+                                ++head;
+                            }
+                    }
+                    __syncwarp();
+                }
+                if (!MINS && __any_sync(NSG_FULL, head - told >= TC_MERGE / 2)) {
+                    __threadfence_block();
+                    r_head[row_local] = told = head;
+                }
+            }
+            if (!MINS && ok) {
+                // at most one unit ahead of the merging warp
+                const uint64_t t0 = tc::globaltimer();
+                while (ok && begun[w] != nu) {
+                    __nanosleep(200);
+                    if (*abort || tc::globaltimer() - t0 > tc::WAIT_TIMEOUT_NS) ok = false;
+                }
+                ok = __all_sync(NSG_FULL, ok);
+                if (!ok) *abort = 1;
+                r_end[row_local] = r_head[row_local] = told = head;
+                __threadfence_block();
+                __syncwarp();
+                if (lane == 0) scanned[w] = nu;
             }
         }
-        if (ok) {
-            unsigned need = __ballot_sync(NSG_FULL, cnt > 0);
-            while (need) {
-                const int src = __ffs(need) - 1;
-                need &= need - 1;
-                merge_row(src, row_local, row_g, cnt, lsize, thrp, qn_r, bufs, ls, sb, thr_slot, a.ids,
-                          a.d2, a.KL);
+    } else if (!MINS) {
+        // ---------------- merge: one warp behind each scanning warp ----------------
+        const int w = warp - 2 - TC_SCAN, g = w >> 2, q = (w + 2) & 3;
+        unsigned char *wsm = smem + Cfg::OFF_MERGE + w * Cfg::MERGE_BYTES;
+        uint64_t *sb = reinterpret_cast<uint64_t *>(wsm);
+        uint64_t *thr_slot = sb + TC_BUF;
+        int *hist = reinterpret_cast<int *>(thr_slot + 2);
+        const int row_local = g * TC_M + q * 32 + (int)lane;
+        const size_t ring0 = ((size_t)blockIdx.x * TC_UNIT + g * TC_M + q * 32) * TC_RING;
+        int nu = 0, tail = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
+            int rt, i0, i1;
+            unit_tiles(a, u, &rt, &i0, &i1);
+            if (g >= unit_groups(a, rt)) continue;
+            ++nu;
+            const int64_t row_g = (int64_t)rt * TC_UNIT + row_local;
+            const bool valid = row_g < a.m;
+            const int64_t list0 = (row_g * a.S + u / a.T) * a.KL;
+            const int self = a.self_join ? (int)(a.q0 + row_g) : -1;
+            const float qn_r = valid ? a.qn[row_g] : 0.0f;
+            int lsize;
+            float thrp = first_bound(a, row_g, list0, &lsize);
+            r_thr[row_local] = thrp;
+            __threadfence_block();
+            __syncwarp();
+            if (lane == 0) begun[w] = nu;
+            uint64_t t0 = tc::globaltimer();
+            for (;;) {
+                // the head is read before the flag: a head past the unit's end is
+                // published only after the flag
+                int head = tc::lds_acquire(r_head + row_local);
+                const bool fin = __shfl_sync(NSG_FULL, tc::lds_acquire(scanned + w), 0) >= nu;
+                if (fin) head = r_end[row_local];
+                unsigned need = __ballot_sync(NSG_FULL, head - tail >= (fin ? 1 : TC_MERGE));
+                if (!need) {
+                    if (fin) break;
+                    __nanosleep(500);
+                    const bool gone = *abort || tc::globaltimer() - t0 > tc::WAIT_TIMEOUT_NS;
+                    if (__any_sync(NSG_FULL, gone)) {
+                        *abort = 1;
+                        ok = false;
+                        break;
+                    }
+                    continue;
+                }
+                while (need) {
+                    const int src = __ffs(need) - 1;
+                    need &= need - 1;
+                    const int rt0 = __shfl_sync(NSG_FULL, tail, src), rh = __shfl_sync(NSG_FULL, head, src);
+                    const int own = __shfl_sync(NSG_FULL, self, src);
+                    const float q2 = __shfl_sync(NSG_FULL, qn_r, src);
+                    const int64_t lr = __shfl_sync(NSG_FULL, list0, src);
+                    int s = __shfl_sync(NSG_FULL, lsize, src);
+                    const float *vals = a.vals + (ring0 + (size_t)src * TC_RING) * 8;
+                    const float bar = merge_row(vals, a.cols + ring0 + (size_t)src * TC_RING, rt0, rh, own, q2,
+                                                __shfl_sync(NSG_FULL, thrp, src), s, sb, hist, thr_slot, a.ids + lr,
+                                                a.d2 + lr, a.KL);
+                    if ((int)lane == src) {
+                        lsize = s;
+                        thrp = bar;
+                        tail = rh;
+                        // (the ring's entries have been read: no fence, which would
+                        // wait for the list's stores, thousands of cycles)
+                        r_thr[row_local] = bar;
+                        r_tail[row_local] = rh;
+                    }
+                    __syncwarp();
+                }
+                t0 = tc::globaltimer();
             }
+            if (!ok) break;
             if (!a.last) {  // carry the list size to the next chunk
                 if (valid) a.lsz[row_g] = lsize;
             } else  // pad rows holding fewer than k candidates
-            for (int src = 0; src < 32; ++src) {
-                const int s = __shfl_sync(NSG_FULL, lsize, src);
-                const int64_t rg = __shfl_sync(NSG_FULL, row_g, src);
-                const bool v = __shfl_sync(NSG_FULL, valid ? 1 : 0, src);
-                if (!v) continue;
-                for (int i = s + lane; i < a.KL; i += 32) {
-                    a.ids[rg * a.KL + i] = -1;
-                    a.d2[rg * a.KL + i] = __int_as_float(0x7f800000);
+                for (int src = 0; src < 32; ++src) {
+                    const int s = __shfl_sync(NSG_FULL, lsize, src);
+                    const int64_t lr = __shfl_sync(NSG_FULL, list0, src);
+                    const bool v = __shfl_sync(NSG_FULL, valid ? 1 : 0, src);
+                    if (!v) continue;
+                    for (int x = s + (int)lane; x < a.KL; x += 32) {
+                        a.ids[lr + x] = -1;
+                        a.d2[lr + x] = __int_as_float(0x7f800000);
+                    }
                 }
-            }
         }
     }
     tc::fence_before_sync();
@@ -446,32 +716,137 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     if (*abort && !skip && threadIdx.x == 0) atomicExch(a.err, 1);
     if (warp == 1) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, 2 * TC_N);
+        tc::tmem_dealloc(tmem, 2 * TC_G * TC_N);
     }
 }
 
-// Row-wise BF16 copy with K padded to DK, squared norms of the rounded values,
-// and a flag raised when a value is not an integer in 0..255.
-__global__ void bf16_rows_kernel(const float *__restrict__ src, int64_t rows, int dp, __nv_bfloat16 *dst,
-                                 int dk, float *norms, int64_t rows_pad, int *nonint) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
+// A float's bits as an unsigned number of the same order, and back.
+__device__ __forceinline__ unsigned order_bits(float f) {
+    const unsigned u = __float_as_uint(f);
+    return u & 0x80000000u ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float from_order_bits(unsigned u) {
+    return __uint_as_float(u & 0x80000000u ? u & 0x7fffffffu : ~u);
+}
+
+// A strict bound just above the `rank`-th smallest of each row's `count`
+// minima (to 2^-11 relative: the search over the order bits stops 12 bits
+// early, rounding up).  One warp per row, at most KPL minima per lane.
+template <int KPL>
+__global__ void __launch_bounds__(256) knn_bound_kernel(const float *minima, int count, int64_t mpad, int64_t m,
+                                                        int rank, float *thr) {
     const unsigned lane = lane_id();
-    for (int64_t r = warp; r < rows_pad; r += nw) {
-        float acc = 0.0f;
-        bool bad = false;
-        for (int c = lane; c < dk; c += 32) {
-            float v = (r < rows && c < dp) ? src[r * dp + c] : 0.0f;
-            __nv_bfloat16 h = __float2bfloat16_rn(v);
-            float hv = __bfloat162float(h);
-            acc += hv * hv;
-            bad |= !(v >= 0.0f && v <= 255.0f && v == rintf(v));
-            if (r < rows) dst[r * dk + c] = h;
+    for (int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); r < m; r += (int64_t)gridDim.x * 8) {
+        unsigned k[KPL];
+#pragma unroll
+        for (int t = 0; t < KPL; ++t) {
+            const int i = t * 32 + (int)lane;
+            k[t] = i < count ? order_bits(__ldg(minima + (int64_t)i * mpad + r)) : ~0u;
         }
-        acc = group_sum<32>(acc);
-        if (lane == 0) norms[r] = r < rows ? acc : 0.0f;
-        if (__any_sync(NSG_FULL, bad) && lane == 0 && r < rows) atomicOr(nonint, 1);
+        unsigned t0 = 0;  // fewer than `rank` keys are below t0
+#pragma unroll 1
+        for (int bit = 31; bit >= 12; --bit) {
+            const unsigned c = t0 | (1u << bit);
+            int below = 0;
+#pragma unroll
+            for (int t = 0; t < KPL; ++t) below += k[t] < c;
+            if (__reduce_add_sync(NSG_FULL, below) < rank) t0 = c;
+        }
+        if (lane == 0) {
+            const unsigned inf = 0xff800000u;  // order bits of +inf
+            thr[r] = t0 >= inf || t0 + 0x1000u >= inf ? __int_as_float(0x7f800000) : from_order_bits(t0 + 0x1000u);
+        }
     }
+}
+
+// The KL smallest keys of each row's S split lists [m][S][KL] (sorted, -1
+// padded): one block per row, every warp merges its share of the lists, then
+// one warp the eight results.
+__global__ void __launch_bounds__(256) knn_merge_kernel(const int *ids_in, const float *d2_in, int64_t m, int S, int KL,
+                                                        int *ids, float *d2) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int sizes[8];
+    const int warp = threadIdx.x >> 5;
+    const unsigned lane = lane_id();
+    // per warp: list, candidates, ck, sk [KL] (u64); cp, sp [KL] (int)
+    uint64_t *list = reinterpret_cast<uint64_t *>(smem) + (size_t)warp * 5 * KL;
+    uint64_t *cand = list + KL, *ck = cand + KL, *sk = ck + KL;
+    int *cp = reinterpret_cast<int *>(sk + KL), *sp = cp + KL;
+    for (int64_t r = blockIdx.x; r < m; r += gridDim.x) {
+        int size = 0;
+        for (int p = warp; p < S; p += 8) {
+            const int64_t at = (r * S + p) * KL;
+            int c = 0;
+            for (int b = 0; b < KL; b += 32) {
+                const int j = b + (int)lane;
+                const int id = j < KL ? ids_in[at + j] : -1;
+                const unsigned bal = __ballot_sync(NSG_FULL, id >= 0);
+                if (id >= 0) cand[c + __popc(bal & lanemask_lt())] = make_key(d2_in[at + j], id);
+                c += __popc(bal);
+            }
+            __syncwarp();
+            if (c > 0) warp_merge(list, KL, size, cand, c, ck, cp, sk, sp);
+        }
+        if (lane == 0) sizes[warp] = size;
+        __syncthreads();
+        if (warp == 0) {
+            for (int w = 1; w < 8; ++w)
+                if (sizes[w] > 0)
+                    warp_merge(list, KL, size, reinterpret_cast<uint64_t *>(smem) + (size_t)w * 5 * KL, sizes[w], ck,
+                               cp, sk, sp);
+            for (int c = lane; c < KL; c += 32) {
+                const bool has = c < size;
+                ids[r * KL + c] = has ? kid(list[c]) : -1;
+                d2[r * KL + c] = has ? kd2(list[c]) : __int_as_float(0x7f800000);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Row-wise BF16 copy with K padded to DK, squared norms of the rounded values
+// (+inf past the last row: such a column is never a candidate), and a flag
+// raised when a value is not an integer in 0..255.  Bound by memory: a warp
+// has four rows of 16-byte loads in flight.
+__global__ void __launch_bounds__(256) bf16_rows_kernel(const float4 *__restrict__ src, int64_t rows, int dp4,
+                                                        uint2 *dst, int dk4, float *norms, int64_t rows_pad,
+                                                        int *nonint) {
+    constexpr int RW = 4;
+    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const unsigned lane = lane_id();
+    bool bad = false;
+    for (int64_t r0 = warp * RW; r0 < rows_pad; r0 += nw * RW) {
+        float acc[RW] = {0.0f, 0.0f, 0.0f, 0.0f};
+        for (int c = lane; c < dk4; c += 32) {
+            float4 v[RW];
+#pragma unroll
+            for (int j = 0; j < RW; ++j)
+                v[j] = r0 + j < rows && c < dp4 ? __ldg(src + (r0 + j) * dp4 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int j = 0; j < RW; ++j) {
+                const float f[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
+                unsigned short h[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const __nv_bfloat16 b = __float2bfloat16_rn(f[e]);
+                    const float hv = __bfloat162float(b);
+                    acc[j] += hv * hv;
+                    bad |= !(f[e] >= 0.0f && f[e] <= 255.0f && f[e] == rintf(f[e]));
+                    h[e] = __bfloat16_as_ushort(b);
+                }
+                if (r0 + j < rows)
+                    dst[(r0 + j) * dk4 + c] =
+                        make_uint2(h[0] | ((unsigned)h[1] << 16), h[2] | ((unsigned)h[3] << 16));
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < RW; ++j) {
+            const float s = group_sum<32>(acc[j]);
+            if (lane == 0 && r0 + j < rows_pad) norms[r0 + j] = r0 + j < rows ? s : __int_as_float(0x7f800000);
+        }
+    }
+    if (__any_sync(NSG_FULL, bad) && lane == 0) atomicOr(nonint, 1);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -510,6 +885,42 @@ struct Scratch {
     cudaError_t alloc(size_t n) { return cudaMalloc(reinterpret_cast<void **>(&p), n * sizeof(T) + 16); }
 };
 
+// Work split of one selection over `ntiles` base tiles: as few splits as
+// finish the (row unit, split) pairs in about the least number of waves; a
+// unit costs its tiles and, once, about 40 tiles' time to fill its lists.
+int knn_splits(int T, int64_t ntiles, int64_t m, int KL) {
+    const int sms = sm_count();
+    double best = 0.0;
+    int bs = 1;
+    for (int S = 1; S <= 256 && S * 8 <= std::max<int64_t>(ntiles, 8); ++S) {
+        if (S > 1 && (size_t)m * S * KL * 8 > (size_t(1) << 30)) break;
+        const int64_t waves = ((int64_t)T * S + sms - 1) / sms;
+        const double cost = (double)waves * ((double)ntiles / S + 40.0);
+        if (S == 1 || cost < 0.9 * best) {
+            best = cost;
+            bs = S;
+        }
+    }
+    return bs;
+}
+
+template <int DK, bool MINS>
+cudaError_t launch_tc(const CUtensorMap &mA, const CUtensorMap &mB, const TcArgs &a, cudaStream_t st) {
+    auto kern = knn_tc_kernel<DK, MINS>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<DK>::SMEM);
+    if (e != cudaSuccess) return e;
+    const int64_t units = (int64_t)a.T * a.S;
+    kern<<<(unsigned)std::min<int64_t>(units, sm_count()), TC_THREADS, TcCfg<DK>::SMEM, st>>>(mA, mB, a);
+    return cudaGetLastError();
+}
+
+template <bool MINS>
+cudaError_t launch_tc(int dk, const CUtensorMap &mA, const CUtensorMap &mB, const TcArgs &a, cudaStream_t st) {
+    return dk == 64 ? launch_tc<64, MINS>(mA, mB, a, st)
+           : dk == 128 ? launch_tc<128, MINS>(mA, mB, a, st)
+                       : launch_tc<0, MINS>(mA, mB, a, st);
+}
+
 }  // namespace
 
 // Tensor-core kNN when the data allows an exact answer (integer 0..255,
@@ -530,13 +941,15 @@ cudaError_t launch_knn_tc(const KnnLaunch &l, int *used, cudaStream_t st) {
     if ((e = flag.alloc(2)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(flag.p, 0, 2 * sizeof(int), st)) != cudaSuccess) return e;
     const int grid_rows = sm_count() * 8;
-    bf16_rows_kernel<<<grid_rows, 256, 0, st>>>(l.base, l.n, l.dp, xb.p, dk, xn.p, npad, flag.p);
+    bf16_rows_kernel<<<grid_rows, 256, 0, st>>>(reinterpret_cast<const float4 *>(l.base), l.n, l.dp / 4,
+                                                reinterpret_cast<uint2 *>(xb.p), dk / 4, xn.p, npad, flag.p);
     const __nv_bfloat16 *qsrc = xb.p + (l.self_join ? l.q0 * dk : 0);
     const float *qnorm = xn.p + (l.self_join ? l.q0 : 0);
     if (!l.self_join) {
         if ((e = qb.alloc((size_t)l.nq * dk)) != cudaSuccess) return e;
         if ((e = qn.alloc((size_t)l.nq)) != cudaSuccess) return e;
-        bf16_rows_kernel<<<grid_rows, 256, 0, st>>>(l.queries, l.nq, l.dp, qb.p, dk, qn.p, l.nq, flag.p);
+        bf16_rows_kernel<<<grid_rows, 256, 0, st>>>(reinterpret_cast<const float4 *>(l.queries), l.nq, l.dp / 4,
+                                                    reinterpret_cast<uint2 *>(qb.p), dk / 4, qn.p, l.nq, flag.p);
         qsrc = qb.p;
         qnorm = qn.p;
     }
@@ -555,10 +968,13 @@ cudaError_t launch_knn_tc(const KnnLaunch &l, int *used, cudaStream_t st) {
     CUtensorMap mA, mB;
     const int64_t arows = l.self_join ? l.n - l.q0 : l.nq;
     if (!make_map(&mA, qsrc, arows, dk, TC_M) || !make_map(&mB, xb.p, l.n, dk, TC_N)) return cudaSuccess;
+    const int T = (int)((l.nq + TC_UNIT - 1) / TC_UNIT);
+    const int S = knn_splits(T, ntiles, l.nq, KL);
     // the rows' sorted lists live in the output arrays (exact) or in scratch
-    // (candidates); distances are kept even when the caller asked for ids only
-    Scratch<float> d2s;
-    Scratch<int> ids_s;
+    // (candidates, splits); distances are kept even when the caller asked for
+    // ids only
+    Scratch<float> d2s, d2p;
+    Scratch<int> ids_s, ids_p;
     float *d2out = l.d2;
     int *idsout = l.ids;
     if (!exact) {
@@ -569,6 +985,15 @@ cudaError_t launch_knn_tc(const KnnLaunch &l, int *used, cudaStream_t st) {
         if ((e = d2s.alloc((size_t)l.nq * KL)) != cudaSuccess) return e;
         d2out = d2s.p;
     }
+    if (S > 1) {
+        if ((e = ids_p.alloc((size_t)l.nq * S * KL)) != cudaSuccess) return e;
+        if ((e = d2p.alloc((size_t)l.nq * S * KL)) != cudaSuccess) return e;
+    }
+    Scratch<float> vals;
+    Scratch<int> cols;
+    const int64_t grid = std::min<int64_t>((int64_t)T * S, sm_count());
+    if ((e = vals.alloc((size_t)grid * TC_UNIT * TC_RING * 8)) != cudaSuccess) return e;
+    if ((e = cols.alloc((size_t)grid * TC_UNIT * TC_RING)) != cudaSuccess) return e;
     TcArgs a;
     a.qn = qnorm;
     a.xn = xn.p;
@@ -578,46 +1003,82 @@ cudaError_t launch_knn_tc(const KnnLaunch &l, int *used, cudaStream_t st) {
     a.self_join = l.self_join;
     a.KL = KL;
     a.kb = dk / TC_BOXK;
-    a.ids = idsout;
-    a.d2 = d2out;
+    a.ids = S > 1 ? ids_p.p : idsout;
+    a.d2 = S > 1 ? d2p.p : d2out;
     a.err = flag.p + 1;
-    // The base is taken in chunks of ~48 MB of BF16 rows, one launch per chunk
-    // over every query tile, so a chunk stays in L2 while all query tiles pass
+    a.vals = vals.p;
+    a.cols = cols.p;
+    a.T = T;
+    a.thr0 = nullptr;
+    a.minima = nullptr;
+    a.mpad = 0;
+    a.rt0 = 0;
+    a.lsz = nullptr;
+    a.first = a.last = 1;
+    // Pre-pass: `rank` of the sample's 64-column minima have as many distinct
+    // columns at or below them (one more where a row meets itself).  Two
+    // minima per tile, 2.5 ranks' worth of tiles: the bound then admits ~1.1
+    // times the sample's own k nearest, and a larger sample would cost more
+    // tiles than the candidates it saves (k ln 2 per doubling, ~30 warp
+    // instructions each, against ~10 per tile and row).  At most a quarter of
+    // the base, and none when those are too few for a useful bound.
+    const int rank = KL + (l.self_join ? 1 : 0);
+    const int P = (int)std::min<int64_t>(ntiles / 4, (int64_t)rank * 5 / 2);
+    Scratch<float> minima, thr;
+    if (2 * P >= rank + rank / 4) {
+        // up to 1 GB of minima at a time: blocks of row units
+        const int64_t fit = (int64_t(1) << 30) / ((int64_t)2 * P * TC_UNIT * 4);
+        const int TB = (int)std::max<int64_t>(1, std::min<int64_t>(T, fit));
+        TcArgs p = a;
+        p.mpad = (int64_t)TB * TC_UNIT;
+        if ((e = minima.alloc((size_t)2 * P * p.mpad)) != cudaSuccess) return e;
+        if ((e = thr.alloc((size_t)l.nq)) != cudaSuccess) return e;
+        p.minima = minima.p;
+        p.tile0 = 0;
+        p.tile1 = P;
+        p.stride = (int)(ntiles / P);
+        for (int t0 = 0; t0 < T; t0 += TB) {
+            p.rt0 = t0;
+            p.T = std::min(TB, T - t0);
+            p.S = (int)std::max<int64_t>(1, std::min<int64_t>(P / 4, ((int64_t)sm_count() * 4 + p.T - 1) / p.T));
+            if ((e = launch_tc<true>(dk, mA, mB, p, st)) != cudaSuccess) return e;
+            const int64_t r0 = (int64_t)t0 * TC_UNIT, rows = std::min<int64_t>((int64_t)p.T * TC_UNIT, l.nq - r0);
+            const int64_t blocks = std::min<int64_t>((rows + 7) / 8, (int64_t)sm_count() * 16);
+            auto bound = 2 * P <= 512 ? knn_bound_kernel<16> : 2 * P <= 1024 ? knn_bound_kernel<32> : knn_bound_kernel<48>;
+            bound<<<(unsigned)blocks, 256, 0, st>>>(minima.p, 2 * P, p.mpad, rows, rank, thr.p + r0);
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
+        a.thr0 = thr.p;
+    }
+    // An unsplit base is taken in chunks of ~48 MB of BF16 rows, one launch per
+    // chunk over every row unit, so a chunk stays in L2 while all units pass
     // over it (a single sweep per CTA would re-read a base larger than L2 from
     // HBM once per wave of CTAs).  Rows see columns in increasing id across
     // chunks, and their lists carry over through the output arrays and lsz.
     int64_t chunk_tiles = std::max<int64_t>(1, (int64_t(48) << 20) / ((int64_t)TC_N * dk * 2));
     if (const char *ct = getenv("NSG_KNN_CHUNK_TILES"))  // smaller chunks (tests)
         if (atoi(ct) > 0) chunk_tiles = atoi(ct);
+    if (S > 1) chunk_tiles = ntiles;
     const int64_t nchunks = (ntiles + chunk_tiles - 1) / chunk_tiles;
     Scratch<int> lsz;
     if (nchunks > 1 && (e = lsz.alloc((size_t)l.nq)) != cudaSuccess) return e;
     a.lsz = lsz.p;
-    const int64_t grid = (l.nq + TC_M - 1) / TC_M;
+    a.S = S;
+    a.stride = 1;
     for (int64_t c = 0; c < nchunks; ++c) {
-        a.t0 = (int)(c * chunk_tiles);
-        a.t1 = (int)std::min<int64_t>(ntiles, (c + 1) * chunk_tiles);
+        a.tile0 = (int)(c * chunk_tiles);
+        a.tile1 = (int)std::min<int64_t>(ntiles, (c + 1) * chunk_tiles);
         a.first = c == 0;
         a.last = c == nchunks - 1;
-        if (dk == 64) {
-            auto kern = knn_tc_kernel<64>;
-            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<64>::SMEM)) !=
-                cudaSuccess)
-                return e;
-            kern<<<(unsigned)grid, TC_THREADS, TcCfg<64>::SMEM, st>>>(mA, mB, a);
-        } else if (dk == 128) {
-            auto kern = knn_tc_kernel<128>;
-            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<128>::SMEM)) !=
-                cudaSuccess)
-                return e;
-            kern<<<(unsigned)grid, TC_THREADS, TcCfg<128>::SMEM, st>>>(mA, mB, a);
-        } else {
-            auto kern = knn_tc_kernel<0>;
-            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<0>::SMEM)) !=
-                cudaSuccess)
-                return e;
-            kern<<<(unsigned)grid, TC_THREADS, TcCfg<0>::SMEM, st>>>(mA, mB, a);
-        }
+        if ((e = launch_tc<false>(dk, mA, mB, a, st)) != cudaSuccess) return e;
+    }
+    if (S > 1) {
+        const size_t smem = (size_t)8 * 5 * KL * sizeof(uint64_t);
+        if ((e = cudaFuncSetAttribute(knn_merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
+            cudaSuccess)
+            return e;
+        const int64_t blocks = std::min<int64_t>(l.nq, (int64_t)sm_count() * 16);
+        knn_merge_kernel<<<(unsigned)blocks, 256, smem, st>>>(a.ids, a.d2, l.nq, S, KL, idsout, d2out);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     if ((e = cudaMemcpyAsync(h, flag.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
