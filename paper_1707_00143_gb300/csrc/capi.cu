@@ -369,6 +369,15 @@ nsg_status collect_prune_all(const float *bp, int64_t n, int dp, const int *knn,
     DevBuf<int> cid, ccnt;
     DevBuf<float> cd2;
     DevBuf<unsigned long long> nexam;
+    // logs of the searches' keys (2 GiB at most: fewer, larger launches); without
+    // that memory the collect lists are merged as they grow
+    DevBuf<uint64_t> log;
+    const int64_t log_cap = nsg::collect_log_cap(L, K, C);
+    int64_t log_nodes = log_cap ? std::min<int64_t>(chunk, (int64_t)(budget / (8 * log_cap))) : 0;
+    if (log_nodes && log.alloc((size_t)(log_nodes * log_cap)) != cudaSuccess) {
+        cudaGetLastError();
+        log_nodes = 0;
+    }
     NSG_CK(cid.alloc((size_t)chunk * C));
     NSG_CK(cd2.alloc((size_t)chunk * C));
     NSG_CK(ccnt.alloc(chunk));
@@ -397,6 +406,8 @@ nsg_status collect_prune_all(const float *bp, int64_t n, int dp, const int *knn,
         c.cand_d2 = cd2.p;
         c.cand_count = ccnt.p;
         c.status = nullptr;
+        c.log = log.p;
+        c.log_nodes = log_nodes;
         cudaEventRecord(ev[0], st);
         cudaError_t e = nsg::launch_collect(c, st);
         if (e != cudaSuccess) rc = cuda_fail(e, "launch_collect");
@@ -624,7 +635,21 @@ nsg_status nsg_collect(const float *base_dev, int64_t n, int32_t d, const int32_
     c.cand_d2 = cand_d2_dev;
     c.cand_count = cand_count_dev;
     c.status = status_dev;
-    NSG_CK(nsg::launch_collect(c, st));
+    // stream-ordered logs of 256 MiB at most, returned to the device once the
+    // call's work is done; refused, the call runs without
+    const int64_t log_cap = nsg::collect_log_cap(L, K, C);
+    void *log = nullptr;
+    if (log_cap) {
+        c.log_nodes = std::min<int64_t>(nv, (int64_t)((size_t(256) << 20) / (8 * log_cap)));
+        if (cudaMallocAsync(&log, (size_t)(8 * log_cap * c.log_nodes), st) != cudaSuccess) {
+            cudaGetLastError();
+            log = nullptr;
+        }
+        c.log = static_cast<uint64_t *>(log);
+    }
+    const cudaError_t e = nsg::launch_collect(c, st);
+    if (log) cudaFreeAsync(log, st);
+    NSG_CK(e);
     return NSG_OK;
 }
 

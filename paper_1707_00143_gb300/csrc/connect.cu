@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(256) fix_search_kernel(FixArgs a, int round) {
         if (round == 0 || fix_stale(a, f, u)) {
             DistF32<G, V, U> dist{{}, a.base4, a.dp4};
             dist.Q.load_row(a.base4 + (int64_t)u * a.dp4, a.dp4);
-            const SearchOut o = warp_alg1<false>(dist, GraphView{a.adj, a.R, a.deg, a.label, a.flab[f]}, a.nav, a.L,
+            const SearchOut o = warp_alg1<KEYS_POOL>(dist, GraphView{a.adj, a.R, a.deg, a.label, a.flab[f]}, a.nav, a.L,
                                                  s, (uint32_t)a.H - 1, a.hshift, a.max_steps, -1, 0, csize,
                                                  a.xlog + (int64_t)f * a.xcap, a.xcap, nullptr,
                                                  a.xthr + (int64_t)f * a.xcap);

@@ -180,7 +180,12 @@ struct CollectLaunch {
     float *cand_d2;
     int *cand_count;
     int *status;
+    // logs of collect_log_cap keys for log_nodes nodes at a time (nullptr: the
+    // kernel that keeps sorted lists)
+    uint64_t *log = nullptr;
+    int64_t log_nodes = 0;
 };
+int collect_log_cap(int L, int K, int C);  // keys per node, 0: no log form
 cudaError_t launch_collect(const CollectLaunch &a, cudaStream_t st);
 
 // MRNG edge selection for nodes v0..v0+nv-1.

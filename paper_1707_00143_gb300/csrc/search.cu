@@ -1,64 +1,8 @@
-// search.cu -- Alg. 1 for a batch of queries (search on NSG, Section 3.6) and
-// the per-node search-and-collect of Alg. 2 (Section 3.5 iii), one warp per unit.
+// search.cu -- Alg. 1 for a batch of queries (search on NSG, Section 3.6), one
+// warp per unit.
 #include "search_kern.cuh"
 
 namespace nsg {
-
-struct CollectArgs {
-    const float4 *base4;
-    int dp4;
-    const int *knn;
-    int K, W, nav, L, C, H, hshift, max_steps;
-    int64_t v0, nv;
-    int *cand_ids;
-    float *cand_d2;
-    int *cand_count, *status;
-};
-
-template <int G, int V, int U>
-__global__ void __launch_bounds__(256) collect_kernel(CollectArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    const unsigned lane = lane_id();
-    WarpSmem s = carve_warp_smem(smem + warp * warp_smem_bytes(a.L, a.W, a.C, a.H), a.L, a.W, a.C, a.H);
-    const int64_t stride = (int64_t)gridDim.x * wpb;
-    const uint32_t hmask = (uint32_t)a.H - 1;
-    for (int64_t j = (int64_t)blockIdx.x * wpb + warp; j < a.nv; j += stride) {
-        const int v = (int)(a.v0 + j);
-        DistF32<G, V, U> dist{{}, a.base4, a.dp4};
-        dist.Q.load_row(a.base4 + (int64_t)v * a.dp4, a.dp4);
-        int csize = 0;
-        SearchOut o = warp_alg1<true>(dist, GraphRef{a.knn, a.K}, a.nav, a.L, s, hmask, a.hshift,
-                                             a.max_steps, v, a.C, csize);
-        // Alg. 2: v's nearest neighbours in G join the candidates
-        const int *row = a.knn + (int64_t)v * a.K;
-        int m = 0;
-        for (int b = 0; b < a.K; b += 32) {
-            int slot = b + (int)lane;
-            int w = slot < a.K ? __ldg(row + slot) : -1;
-            bool fresh = w >= 0 && visit(s.hash, hmask, a.hshift, w);
-            unsigned bal = __ballot_sync(NSG_FULL, fresh);
-            if (fresh) s.ids[m + __popc(bal & lanemask_lt())] = w;
-            m += __popc(bal);
-        }
-        __syncwarp();
-        if (m > 0) {
-            dist(s.ids, m, s.keys);
-            collect_merge(s, m, v, a.C, csize);
-        }
-        // Alg. 2: sorted candidates, cut to C
-        for (int t = lane; t < a.C; t += 32) {
-            uint64_t e = t < csize ? s.clist[t] : KEY_INF;
-            a.cand_ids[j * a.C + t] = t < csize ? kid(e) : -1;
-            a.cand_d2[j * a.C + t] = t < csize ? kd2(e) : __int_as_float(0x7f800000);
-        }
-        if (lane == 0) {
-            a.cand_count[j] = csize;
-            if (a.status) a.status[j] = o.capped ? -4 : 0;
-        }
-        __syncwarp();
-    }
-}
 
 cudaError_t launch_search(const SearchLaunch &l, cudaStream_t st) {
     if (l.nq <= 0) return cudaSuccess;
@@ -361,40 +305,5 @@ cudaError_t launch_nav_order(const float *queries, int64_t nq, int d, const floa
 int64_t search_pool_slots() { return (int64_t)sm_count() * 32; }
 
 size_t search_warp_smem_bytes(int L, int W, int H) { return warp_smem_bytes(L, W, 0, H, true); }
-
-cudaError_t launch_collect(const CollectLaunch &l, cudaStream_t st) {
-    if (l.nv <= 0) return cudaSuccess;
-    CollectArgs a;
-    a.base4 = reinterpret_cast<const float4 *>(l.base);
-    a.dp4 = l.dp / 4;
-    a.knn = l.knn;
-    a.K = l.K;
-    a.W = round32(l.K);
-    a.nav = l.nav;
-    a.L = l.L;
-    a.C = l.C;
-    a.H = l.hash_slots;
-    a.hshift = 32 - log2i((unsigned)l.hash_slots);
-    a.max_steps = l.max_steps;
-    a.v0 = l.v0;
-    a.nv = l.nv;
-    a.cand_ids = l.cand_ids;
-    a.cand_d2 = l.cand_d2;
-    a.cand_count = l.cand_count;
-    a.status = l.status;
-    size_t per_warp = warp_smem_bytes(a.L, a.W, a.C, a.H);
-    cudaError_t err = cudaSuccess;
-    NSG_DISPATCH_DP4(a.dp4, {
-        auto kern = collect_kernel<G_, V_, U_>;
-        int grid, wpb;
-        size_t smem;
-        err = config(kern, per_warp, 4, l.nv, &grid, &wpb, &smem);
-        if (err == cudaSuccess) {
-            kern<<<grid, wpb * 32, smem, st>>>(a);
-            err = cudaGetLastError();
-        }
-    });
-    return err;
-}
 
 }  // namespace nsg

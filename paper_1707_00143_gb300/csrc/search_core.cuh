@@ -12,8 +12,8 @@
 // The same routine serves
 //   * search on the NSG from the navigating node (Section 3.6),
 //   * search-and-collect on the kNN graph (Alg. 2, Section 3.5 iii): every computed
-//     key except the node itself is also merged into a collect list of the C
-//     smallest keys,
+//     key except the node itself also goes to a collect list of the C smallest
+//     keys, merged at once or logged and selected by a kernel that follows,
 //   * the connectivity pass (Alg. 2, Section 3.5 iv): searches that also log the
 //     ids they expand, on a view of the graph that hides later fix-ups' edges.
 #pragma once
@@ -171,6 +171,79 @@ __device__ __forceinline__ float stop_logit(const StopMLP &m, const float (&f)[N
 __device__ __forceinline__ void collect_merge(WarpSmem &s, int m, int excl, int C, int &csize) {
     warp_merge(s.clist, C, csize, s.keys, m, s.ck, s.cp, s.sk, s.sp, excl);
 }
+
+// Every measured key of a node's search, appended in global memory and cut to
+// the C smallest by collect_select_kernel (collect.cu).
+struct KeyLog {
+    uint64_t *keys;  // [cap], cap >= 2 C + the graph's width
+    int cap, C;
+    int count;
+    uint64_t thr;  // keys from here on are not among the C smallest
+};
+
+// What a full log keeps: its C smallest distinct keys, sorted by a bitonic
+// network whose first step of each merge pairs mirrored positions, so that
+// every comparison puts the smaller key first and positions past the end need
+// no padding.  Out of line: the host sizes the log so that it rarely fills.
+static __device__ __noinline__ int log_compact(uint64_t *a, int n, int C) {
+    const unsigned lane = lane_id();
+    __syncwarp();
+    for (int k = 2; k < 2 * n; k <<= 1) {
+        for (int h = k >> 1; h > 0; h >>= 1) {
+            const bool flip = h == k >> 1;
+            for (int p = lane; ; p += 32) {
+                const int blk = p / h, t = p - blk * h, i = blk * 2 * h + t;
+                if (i >= n) break;
+                const int j = flip ? blk * 2 * h + 2 * h - 1 - t : i + h;
+                if (j < n) {
+                    const uint64_t x = a[i], y = a[j];
+                    if (y < x) {
+                        a[i] = y;
+                        a[j] = x;
+                    }
+                }
+            }
+            __syncwarp();
+        }
+    }
+    int kept = 0;
+    uint64_t before = 0;  // the key just below this chunk
+    for (int b = 0; b < n && kept < C; b += 32) {
+        const int j = b + (int)lane;
+        const uint64_t k = j < n ? a[j] : 0;
+        uint64_t prev = __shfl_up_sync(NSG_FULL, k, 1);
+        if (lane == 0) prev = before;
+        const bool keep = j < n && (j == 0 || k != prev);
+        before = __shfl_sync(NSG_FULL, k, 31);
+        const unsigned bal = __ballot_sync(NSG_FULL, keep);
+        const int o = kept + __popc(bal & lanemask_lt());
+        __syncwarp();
+        if (keep && o < C) a[o] = k;
+        kept += __popc(bal);
+        __syncwarp();
+    }
+    return min(kept, C);
+}
+
+// Appends keys[0..m) minus id `excl` to the log.  Warp-wide.
+__device__ __forceinline__ void log_append(KeyLog &lg, const uint64_t *keys, int m, int excl) {
+    if (lg.count + m > lg.cap) {
+        lg.count = log_compact(lg.keys, lg.count, lg.C);
+        if (lg.count == lg.C) lg.thr = lg.keys[lg.C - 1];
+    }
+    const unsigned lane = lane_id();
+    for (int b = 0; b < m; b += 32) {
+        const int j = b + (int)lane;
+        const uint64_t k = j < m ? keys[j] : ~0ull;
+        const bool keep = j < m && k < lg.thr && kid(k) != excl;
+        const unsigned bal = __ballot_sync(NSG_FULL, keep);
+        if (keep) lg.keys[lg.count + __popc(bal & lanemask_lt())] = k;
+        lg.count += __popc(bal);
+    }
+}
+
+// What a search does with the keys it measures besides the pool.
+enum { KEYS_POOL = 0, KEYS_MERGE = 1, KEYS_LOG = 2 };
 
 // Distances of a query to FP32 rows (the plain form).
 template <int G, int V, int U>
@@ -462,11 +535,11 @@ __device__ SearchOut group_alg1(const D &dist, GraphRef g, int start, int L, War
 // it is the predicted node the prepared row is used, otherwise (rare: see
 // predict_next) the speculative visited-set claims are taken back and the
 // row is read again.  The steps, keys and results are those of the plain loop.
-template <bool COLLECT, bool STOP = false, class Gr, class D>
+template <int COLLECT, bool STOP = false, class Gr, class D>
 __device__ SearchOut warp_alg1(const D &dist, const Gr g, int start, int L, WarpSmem &s, uint32_t hmask,
                                int hshift, int max_steps, int excl, int C, int &csize, int *xlog = nullptr,
                                int xcap = 0, const StopCtx *stop = nullptr, uint64_t *xthr = nullptr,
-                               const InitRand *init = nullptr) {
+                               const InitRand *init = nullptr, KeyLog *klog = nullptr) {
     constexpr int PIPE = NSG_PIPE;
     const unsigned lane = lane_id();
     SearchOut o;
@@ -478,7 +551,8 @@ __device__ SearchOut warp_alg1(const D &dist, const Gr g, int start, int L, Warp
     int since_change = 0, last_m = 0;
     bool last_changed = true;
     init_pool(dist, start, L, s, hmask, hshift, init, o);
-    if (COLLECT && (init == nullptr || init->count <= 0)) collect_merge(s, 1, excl, C, csize);
+    if (COLLECT == KEYS_MERGE && (init == nullptr || init->count <= 0)) collect_merge(s, 1, excl, C, csize);
+    if (COLLECT == KEYS_LOG) log_append(*klog, s.keys, 1, excl);
     int cursor = 0;
     int pre_u = -1;  // node whose row is prepared (PIPE)
     int pre_m = 0;   // PIPE 2: its new neighbours, already in s.ids
@@ -557,7 +631,8 @@ __device__ SearchOut warp_alg1(const D &dist, const Gr g, int start, int L, Warp
         }
         dist(s.ids, m, s.keys);
         o.n_dist += m;
-        if (COLLECT) collect_merge(s, m, excl, C, csize);
+        if (COLLECT == KEYS_MERGE) collect_merge(s, m, excl, C, csize);
+        if (COLLECT == KEYS_LOG) log_append(*klog, s.keys, m, excl);
         if constexpr (PIPE != 0) {
             const uint64_t nx = predict_next(s.pool, o.size, L, i, s.keys, m);
             if (nx != ~0ull && o.n_expand < max_steps) {

@@ -267,7 +267,7 @@ __device__ __forceinline__ void search_body(const SearchArgs &a) {
         const InitRand *initp = a.init_count > 0 ? &ir : nullptr;
         SearchOut o;
         const bool qexact = with_dist<G, V, U, P, ST>(a, qp, &sref, [&](const auto &dist) {
-            o = warp_alg1<false, STOP>(
+            o = warp_alg1<KEYS_POOL, STOP>(
                 dist, GraphRef{a.adj, a.width}, start, Lq, s, (uint32_t)a.H - 1, a.hshift, a.max_steps, -1, 0,
                 csize, nullptr, 0, scp, nullptr, initp);
         });
