@@ -5,7 +5,7 @@
 #include <climits>
 
 #include "kernels.h"
-#include "search_core.cuh"
+#include "lowp.cuh"
 
 namespace nsg {
 
@@ -190,8 +190,7 @@ cudaError_t launch_navigate(const float *base, int64_t n, int d, const int *knn,
 // and the count of candidates examined, equal the one-at-a-time scan.
 // ---------------------------------------------------------------------------
 struct PruneArgs {
-    const float4 *base4;
-    int dp4;
+    ExactRows rows;
     const int *cand_ids;
     const float *cand_d2;
     const int *cand_count;
@@ -216,13 +215,74 @@ __device__ __forceinline__ unsigned batch_mask(const bool (&f)[B]) {
     return m;
 }
 
-template <int G, int V, int U, int B>
+// Rows as the selection holds them, a slice per lane of a G-lane group.
+template <int G_, int V>
+struct PruneF32 {
+    static constexpr int G = G_;
+    struct Reg {
+        float4 v[V];
+    };
+    static __device__ __forceinline__ Reg load(const ExactRows &r, int64_t id, bool valid) {
+        const float4 *row = r.base4 + id * r.dp4;
+        Reg x;
+#pragma unroll
+        for (int w = 0; w < V; ++w) {
+            const int k = w * G + (int)lane_id() % G;
+            x.v[w] = (valid && k < r.dp4) ? __ldg(row + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        return x;
+    }
+    static __device__ __forceinline__ float dist(const Reg &x, const Reg &q) {
+        float s = 0.0f;
+#pragma unroll
+        for (int w = 0; w < V; ++w) s += sq4(x.v[w], q.v[w]);
+        return group_sum<G>(s);
+    }
+};
+
+template <int G_, int VC>
+struct PruneU8 {
+    static constexpr int G = G_;
+    struct Reg {
+        uint4 v[VC];
+    };
+    static __device__ __forceinline__ Reg load(const ExactRows &r, int64_t id, bool valid) {
+        const uint4 *row = r.u8 + id * r.dc;
+        Reg x;
+#pragma unroll
+        for (int w = 0; w < VC; ++w) {
+            const int k = w * G + (int)lane_id() % G;
+            x.v[w] = (valid && k < r.dc) ? __ldg(row + k) : make_uint4(0, 0, 0, 0);
+        }
+        return x;
+    }
+    static __device__ __forceinline__ float dist(const Reg &x, const Reg &q) {
+        unsigned s = 0;
+#pragma unroll
+        for (int w = 0; w < VC; ++w) {
+            unsigned e = __vabsdiffu4(x.v[w].x, q.v[w].x);
+            s = __dp4a(e, e, s);
+            e = __vabsdiffu4(x.v[w].y, q.v[w].y);
+            s = __dp4a(e, e, s);
+            e = __vabsdiffu4(x.v[w].z, q.v[w].z);
+            s = __dp4a(e, e, s);
+            e = __vabsdiffu4(x.v[w].w, q.v[w].w);
+            s = __dp4a(e, e, s);
+        }
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) s += __shfl_xor_sync(NSG_FULL, s, o, G);
+        return (float)s;
+    }
+};
+
+template <class Row, int U, int B>
 __device__ __forceinline__ void prune_body(const PruneArgs &a) {
     extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int G = Row::G;
     constexpr int P = 32 / G, NB = P * B;
     static_assert(NB <= 32, "batch mask holds 32 positions");
     const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-    const int lane = (int)lane_id(), grp = lane / G, sub = lane % G;
+    const int lane = (int)lane_id(), grp = lane / G;
     int *kept = reinterpret_cast<int *>(smem) + (size_t)warp * a.Wr;
     const int64_t stride = (int64_t)gridDim.x * wpb;
     unsigned long long examined = 0;
@@ -240,7 +300,7 @@ __device__ __forceinline__ void prune_body(const PruneArgs &a) {
         }
         __syncwarp();
         while (t < cnt && nk < a.R) {
-            float4 q[B][V];
+            typename Row::Reg q[B];
             float pdv[B];
             bool occ[B];
             int id[B];
@@ -258,12 +318,7 @@ __device__ __forceinline__ void prune_body(const PruneArgs &a) {
                 const bool valid = c < cnt;
                 pdv[b] = valid ? cd[c] : 0.0f;
                 occ[b] = !valid;
-                const float4 *row = a.base4 + (int64_t)(valid ? id[b] : 0) * a.dp4;
-#pragma unroll
-                for (int u = 0; u < V; ++u) {
-                    const int k = u * G + sub;
-                    q[b][u] = (valid && k < a.dp4) ? __ldg(row + k) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
+                q[b] = Row::load(a.rows, valid ? id[b] : 0, valid);
             }
             // against the kept set as it was before the batch
             for (int i0 = 0; i0 < nk; i0 += U) {
@@ -271,25 +326,17 @@ __device__ __forceinline__ void prune_body(const PruneArgs &a) {
 #pragma unroll
                 for (int b = 0; b < B; ++b) all &= occ[b];
                 if (__all_sync(NSG_FULL, all)) break;
-                float4 x[U][V];
+                typename Row::Reg x[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int i = i0 + u;
-                    const float4 *row = a.base4 + (int64_t)(i < nk ? kept[i] : 0) * a.dp4;
-#pragma unroll
-                    for (int w = 0; w < V; ++w) {
-                        const int k = w * G + sub;
-                        x[u][w] = (i < nk && k < a.dp4) ? __ldg(row + k) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
+                    x[u] = Row::load(a.rows, i < nk ? kept[i] : 0, i < nk);
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u)
 #pragma unroll
                     for (int b = 0; b < B; ++b) {
-                        float s = 0.0f;
-#pragma unroll
-                        for (int w = 0; w < V; ++w) s += sq4(x[u][w], q[b][w]);
-                        s = group_sum<G>(s);
+                        const float s = Row::dist(x[u], q[b]);
                         if (i0 + u < nk && s < pdv[b]) occ[b] = true;
                     }
             }
@@ -310,22 +357,10 @@ __device__ __forceinline__ void prune_body(const PruneArgs &a) {
                     break;
                 }
                 if (!live) break;
-                const float4 *row = a.base4 + (int64_t)pj * a.dp4;
-                float4 x[V];
-#pragma unroll
-                for (int w = 0; w < V; ++w) {
-                    const int k = w * G + sub;
-                    x[w] = k < a.dp4 ? __ldg(row + k) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
+                const typename Row::Reg x = Row::load(a.rows, pj, true);
                 bool hit[B];
 #pragma unroll
-                for (int b = 0; b < B; ++b) {
-                    float s = 0.0f;
-#pragma unroll
-                    for (int w = 0; w < V; ++w) s += sq4(x[w], q[b][w]);
-                    s = group_sum<G>(s);
-                    hit[b] = s < pdv[b];
-                }
+                for (int b = 0; b < B; ++b) hit[b] = Row::dist(x, q[b]) < pdv[b];
                 live &= ~batch_mask<G, B>(hit);
             }
             __syncwarp();
@@ -342,31 +377,41 @@ __device__ __forceinline__ void prune_body(const PruneArgs &a) {
 // Rows of up to 4 float4s per lane run 3 blocks per SM (78 registers, no
 // spills; 8 % faster than 2 blocks on 128-value rows); wider rows keep the
 // compiler's own budget (at 3 blocks they spill and run 1.8x slower).
-template <int G, int V, int U, int B>
+template <class Row, int U, int B>
 __global__ void __launch_bounds__(256) prune_kernel(PruneArgs a) {
-    prune_body<G, V, U, B>(a);
+    prune_body<Row, U, B>(a);
 }
-template <int G, int V, int U, int B>
+template <class Row, int U, int B>
 __global__ void __launch_bounds__(256, 3) prune_narrow_kernel(PruneArgs a) {
-    prune_body<G, V, U, B>(a);
+    prune_body<Row, U, B>(a);
 }
-template <int G, int V, int U, int B>
-constexpr auto prune_entry() {
-    if constexpr (V <= 4) return prune_narrow_kernel<G, V, U, B>;
-    else return prune_kernel<G, V, U, B>;
+template <class Row, int U, int B>
+__global__ void __launch_bounds__(256, 3) prune_u8_kernel(PruneArgs a) {
+    prune_body<Row, U, B>(a);
 }
 
-// Candidate rows held per lane group: two while they fit in 32 float4s.
-template <int V>
-struct PruneBatch {
-    static constexpr int value = V <= 8 ? 2 : 1;
-};
+// Candidate rows held per lane group: two while they fit in 32 float4s.  8-bit
+// rows take a quarter of the lanes, loads and arithmetic, so a batch is up to
+// 32 candidates: four per group of four or more lanes.  100,000 SIFT-shaped
+// rows (R = 50, C = 500): FP32 7.17 ms; 8-bit 3.48 ms with one, 2.85 with two,
+// 2.61 with four (4 blocks per SM: 2.92 with two, 2.74 with four; 4 kept rows
+// at a time instead of 2: 3.08).
+template <int G, int V, int U>
+void (*prune_entry(bool u8))(PruneArgs) {
+    if constexpr (V > 4) {  // no 8-bit copy at these widths
+        return prune_kernel<PruneF32<G, V>, U, V <= 8 ? 2 : 1>;
+    } else {
+        using S = Exact8Shape<G, V>;
+        if (u8) return prune_u8_kernel<PruneU8<S::lanes, S::chunks>, U, S::lanes < 4 ? S::lanes : 4>;
+        return prune_narrow_kernel<PruneF32<G, V>, U, 2>;
+    }
+}
 
 cudaError_t launch_prune(const PruneLaunch &l, cudaStream_t st) {
     if (l.nv <= 0) return cudaSuccess;
     PruneArgs a;
-    a.base4 = reinterpret_cast<const float4 *>(l.base);
-    a.dp4 = l.dp / 4;
+    a.rows = ExactRows{reinterpret_cast<const float4 *>(l.base), l.dp / 4, reinterpret_cast<const uint4 *>(l.u8.rows),
+                       l.u8.chunks, l.u8.d, l.u8.lo};
     a.cand_ids = l.cand_ids;
     a.cand_d2 = l.cand_d2;
     a.cand_count = l.cand_count;
@@ -381,8 +426,8 @@ cudaError_t launch_prune(const PruneLaunch &l, cudaStream_t st) {
     const int wpb = 8;
     size_t smem = (size_t)wpb * a.Wr * 4;
     cudaError_t err = cudaSuccess;
-    NSG_DISPATCH_DP4(a.dp4, {
-        auto kern = prune_entry<G_, V_, U_, PruneBatch<V_>::value>();
+    NSG_DISPATCH_DP4(a.rows.dp4, {
+        void (*kern)(PruneArgs) = prune_entry<G_, V_, U_>(a.rows.u8 != nullptr);
         err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (err == cudaSuccess) {
             int per_sm = 0;

@@ -264,43 +264,55 @@ bool nndescent_params_ok(const nsg_nndescent_params &p) {
            p.iters <= 1000 && p.delta >= 0.0f;
 }
 
-// Approximate kNN graph by nn-descent into ids [n][K] (d2 nullable), with
-// scratch allocated for the call.  base [n][dp] padded rows of d values.
 // Integer data of span <= 255 with d * 255^2 < 2^24 (every distance an exact
-// integer below 2^24) get an 8-bit copy x - min for the distances: the same
-// keys as the FP32 rows at a quarter of the bytes gathered.
-nsg_status nndescent_run(const float *base, int64_t n, int dp, int d, int K, const nsg_nndescent_params &p,
-                         int *ids, float *d2, int *iters_run, int64_t *last_updates, cudaStream_t st) {
-    DevBuf<unsigned char> scratch, u8;
-    NSG_CK(scratch.alloc(nsg::nndescent_scratch_bytes(n, K, p.sample, p.reverse)));
-    float lo = 0.0f;
-    bool use_u8 = false;
+// integer below 2^24) gets an 8-bit copy x - min of base [n][dp] for the build's
+// distances: the same keys as the FP32 rows at a quarter of the bytes gathered.
+// Other data, and data whose copy finds no memory: x.rows stays null.
+nsg_status exact8_copy(const float *base, int64_t n, int dp, int d, DevBuf<unsigned char> &buf, nsg::Exact8 &x,
+                       cudaStream_t st) {
+    x = nsg::Exact8{};
     const int dpl = (d + 15) / 16 * 16;
-    if ((int64_t)d * 65025 < (1 << 24)) {
-        DevBuf<unsigned> flags;
-        NSG_CK(flags.alloc(4));
-        unsigned mm[3] = {0xffffffffu, 0u, 0u};
-        NSG_CK(cudaMemcpyAsync(flags.p, mm, sizeof(mm), cudaMemcpyHostToDevice, st));
-        NSG_CK(nsg::launch_minmax(base, n, dp, d, flags.p, st));
-        NSG_CK(cudaMemcpyAsync(mm, flags.p, sizeof(mm), cudaMemcpyDeviceToHost, st));
-        NSG_CK(cudaStreamSynchronize(st));
-        const float mn = nsg::float_from_order_key(mm[0]), mx = nsg::float_from_order_key(mm[1]);
-        if (mm[2] == 0 && (double)mx - (double)mn <= 255.0) {
-            lo = mn;
-            NSG_CK(cudaMemsetAsync(flags.p, 0, sizeof(unsigned), st));
-            NSG_CK(u8.alloc((size_t)n * dpl));
-            NSG_CK(nsg::launch_to_lowp(base, n, dp, d, NSG_PREC_U8, 1.0f, lo, u8.p, dpl,
-                                       reinterpret_cast<int *>(flags.p), st));
-            unsigned inexact = 0;
-            NSG_CK(cudaMemcpyAsync(&inexact, flags.p, sizeof(inexact), cudaMemcpyDeviceToHost, st));
-            NSG_CK(cudaStreamSynchronize(st));
-            use_u8 = inexact == 0;
-        }
+    if ((int64_t)d * 65025 >= (1 << 24)) return NSG_OK;
+    DevBuf<unsigned> flags;
+    NSG_CK(flags.alloc(4));
+    unsigned mm[3] = {0xffffffffu, 0u, 0u};
+    NSG_CK(cudaMemcpyAsync(flags.p, mm, sizeof(mm), cudaMemcpyHostToDevice, st));
+    NSG_CK(nsg::launch_minmax(base, n, dp, d, flags.p, st));
+    NSG_CK(cudaMemcpyAsync(mm, flags.p, sizeof(mm), cudaMemcpyDeviceToHost, st));
+    NSG_CK(cudaStreamSynchronize(st));
+    const float mn = nsg::float_from_order_key(mm[0]), mx = nsg::float_from_order_key(mm[1]);
+    if (mm[2] != 0 || !((double)mx - (double)mn <= 255.0)) return NSG_OK;
+    if (buf.alloc((size_t)n * dpl) != cudaSuccess) {
+        cudaGetLastError();
+        return NSG_OK;
     }
+    NSG_CK(cudaMemsetAsync(flags.p, 0, sizeof(unsigned), st));
+    NSG_CK(nsg::launch_to_lowp(base, n, dp, d, NSG_PREC_U8, 1.0f, mn, buf.p, dpl, reinterpret_cast<int *>(flags.p),
+                               st));
+    unsigned inexact = 0;
+    NSG_CK(cudaMemcpyAsync(&inexact, flags.p, sizeof(inexact), cudaMemcpyDeviceToHost, st));
+    NSG_CK(cudaStreamSynchronize(st));
+    if (inexact == 0) {
+        x.rows = buf.p;
+        x.chunks = dpl / 16;
+        x.d = d;
+        x.lo = mn;
+    }
+    return NSG_OK;
+}
+
+// Approximate kNN graph by nn-descent into ids [n][K] (d2 nullable), with
+// scratch allocated for the call.  base [n][dp] padded rows of d values, u8
+// their exact 8-bit copy if there is one.
+nsg_status nndescent_run(const float *base, int64_t n, int dp, int d, int K, const nsg_nndescent_params &p,
+                         const nsg::Exact8 &u8, int *ids, float *d2, int *iters_run, int64_t *last_updates,
+                         cudaStream_t st) {
+    DevBuf<unsigned char> scratch;
+    NSG_CK(scratch.alloc(nsg::nndescent_scratch_bytes(n, K, p.sample, p.reverse)));
     nsg::NnDescentLaunch l;
-    l.u8 = use_u8 ? u8.p : nullptr;
-    l.u8_chunks = dpl / 16;
-    l.u8_lo = lo;
+    l.u8 = u8.rows;
+    l.u8_chunks = u8.chunks;
+    l.u8_lo = u8.lo;
     l.d = d;
     l.base = base;
     l.n = n;
@@ -360,7 +372,7 @@ nsg_status connect_run(const float *bp, int64_t n, int dp, int *adj, int *deg, i
 
 nsg_status collect_prune_all(const float *bp, int64_t n, int dp, const int *knn, int K, int nav, int L,
                              int R, int C, int *adj, int *deg, float *ms_collect, float *ms_prune,
-                             int64_t *examined, cudaStream_t st) {
+                             int64_t *examined, const nsg::Exact8 &u8, cudaStream_t st) {
     // candidate lists are materialised for a chunk of nodes at a time
     const size_t budget = size_t(2) << 30;
     int64_t chunk = (int64_t)(budget / ((size_t)C * 8 + 8));
@@ -406,6 +418,7 @@ nsg_status collect_prune_all(const float *bp, int64_t n, int dp, const int *knn,
         c.cand_d2 = cd2.p;
         c.cand_count = ccnt.p;
         c.status = nullptr;
+        c.u8 = u8;
         c.log = log.p;
         c.log_nodes = log_nodes;
         cudaEventRecord(ev[0], st);
@@ -426,6 +439,7 @@ nsg_status collect_prune_all(const float *bp, int64_t n, int dp, const int *knn,
         p.adj = adj;
         p.deg = deg;
         p.examined = nexam.p;
+        p.u8 = u8;
         if (rc == NSG_OK) {
             e = nsg::launch_prune(p, st);
             if (e != cudaSuccess) rc = cuda_fail(e, "launch_prune");
@@ -782,10 +796,14 @@ static nsg_status build_index(const float *base_dev, int64_t n, int32_t d, int32
     if (!s && (e = adj.alloc((size_t)n * R)) != cudaSuccess) s = cuda_fail(e, "alloc adj");
     if (!s && (e = deg.alloc((size_t)n)) != cudaSuccess) s = cuda_fail(e, "alloc deg");
     if (!s && (e = knn.alloc((size_t)n * K)) != cudaSuccess) s = cuda_fail(e, "alloc knn");
+    DevBuf<unsigned char> u8buf;
+    nsg::Exact8 u8;
+    if (!s) s = exact8_copy(base.p, n, ix->dp, d, u8buf, u8, st);
     // A1: kNN graph, exact or by nn-descent
     auto t0 = std::chrono::steady_clock::now();
     if (!s && !nnd) s = knn_run(base.p, n, ix->dp, base.p, n, 0, K, 1, knn.p, nullptr, st);
-    if (!s && nnd) s = nndescent_run(base.p, n, ix->dp, d, K, *nnd, knn.p, nullptr, &ix->knn_iters, nullptr, st);
+    if (!s && nnd) s = nndescent_run(base.p, n, ix->dp, d, K, *nnd, u8, knn.p, nullptr, &ix->knn_iters, nullptr,
+                               st);
     if (!s && (e = cudaStreamSynchronize(st)) != cudaSuccess) s = cuda_fail(e, "knn");
     ix->ms[0] = (float)since_ms(t0);
     // A2 + A3: centroid and navigating node
@@ -801,7 +819,7 @@ static nsg_status build_index(const float *base_dev, int64_t n, int32_t d, int32
     // A5 + A6: search-collect-select per node
     if (!s)
         s = collect_prune_all(base.p, n, ix->dp, knn.p, K, ix->nav, L, R, C, adj.p, deg.p, &ix->ms[2],
-                              &ix->ms[3], &ix->prune_examined, st);
+                              &ix->ms[3], &ix->prune_examined, u8, st);
     knn.alloc(0);  // release the kNN graph before the connectivity pass
     // A7: connectivity
     t0 = std::chrono::steady_clock::now();
@@ -857,7 +875,11 @@ nsg_status nsg_knn_nndescent(const float *base_dev, int64_t n, int32_t d, int32_
         if (s) return s;
         int it = 0;
         int64_t upd = 0;
-        s = nndescent_run(view, n, round_up4(d), d, K, *params, knn_ids_dev, knn_d2_dev, &it, &upd, st);
+        DevBuf<unsigned char> u8buf;
+        nsg::Exact8 u8;
+        s = exact8_copy(view, n, round_up4(d), d, u8buf, u8, st);
+        if (s) return s;
+        s = nndescent_run(view, n, round_up4(d), d, K, *params, u8, knn_ids_dev, knn_d2_dev, &it, &upd, st);
         if (s) return s;
         if (iters_run) *iters_run = it;
         if (last_updates) *last_updates = upd;

@@ -6,8 +6,7 @@
 namespace nsg {
 
 struct CollectArgs {
-    const float4 *base4;
-    int dp4;
+    ExactRows rows;
     const int *knn;
     int K, W, nav, L, C, H, hshift, max_steps;
     int64_t v0, nv;
@@ -50,8 +49,8 @@ __global__ void __launch_bounds__(256) collect_kernel(CollectArgs a) {
     const uint32_t hmask = (uint32_t)a.H - 1;
     for (int64_t j = (int64_t)blockIdx.x * wpb + warp; j < a.nv; j += stride) {
         const int v = (int)(a.v0 + j);
-        DistF32<G, V, U> dist{{}, a.base4, a.dp4};
-        dist.Q.load_row(a.base4 + (int64_t)v * a.dp4, a.dp4);
+        DistF32<G, V, U> dist{{}, a.rows.base4, a.rows.dp4};
+        dist.Q.load_row(a.rows.base4 + (int64_t)v * a.rows.dp4, a.rows.dp4);
         int csize = 0;
         SearchOut o = warp_alg1<KEYS_MERGE>(dist, GraphRef{a.knn, a.K}, a.nav, a.L, s, hmask, a.hshift,
                                              a.max_steps, v, a.C, csize);
@@ -78,8 +77,10 @@ __global__ void __launch_bounds__(256) collect_kernel(CollectArgs a) {
 // time) and its list a third of the shared memory: 20 warps per SM, 32 with
 // the log.  Both halves together, FP32 rows: 100,000 SIFT-shaped rows (K =
 // 100, L = 40, C = 500) 18.6 -> 14.0 ms, 150,000 DEEP-shaped (64, 60, 500)
-// 7.2 -> 6.2 ms, 10,000 x 32 (20, 40, 200) 0.57 -> 0.41 ms.
-template <int G, int V, int U>
+// 7.2 -> 6.2 ms, 10,000 x 32 (20, 40, 200) 0.57 -> 0.41 ms.  Integer rows go
+// through their exact 8-bit copy, a quarter of the bytes gathered and of the
+// instructions per row: 14.0 -> 9.0 ms, 0.41 -> 0.37 ms.
+template <int G, int V, int U, bool U8>
 __device__ __forceinline__ void collect_log_body(const CollectArgs &a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
@@ -88,17 +89,19 @@ __device__ __forceinline__ void collect_log_body(const CollectArgs &a) {
     const int64_t stride = (int64_t)gridDim.x * wpb;
     for (int64_t j = (int64_t)blockIdx.x * wpb + warp; j < a.nv; j += stride) {
         const int v = (int)(a.v0 + j);
-        DistF32<G, V, U> dist{{}, a.base4, a.dp4};
-        dist.Q.load_row(a.base4 + (int64_t)v * a.dp4, a.dp4);
         KeyLog lg{a.log + j * a.log_cap, a.log_cap, a.C, 0, ~0ull};
-        int none = 0;
-        SearchOut o = warp_alg1<KEYS_LOG>(dist, GraphRef{a.knn, a.K}, a.nav, a.L, s, (uint32_t)a.H - 1, a.hshift,
-                                          a.max_steps, v, 0, none, nullptr, 0, nullptr, nullptr, nullptr, &lg);
-        const int m = knn_row_keys(a, dist, s, v);
-        if (m > 0) log_append(lg, s.keys, m, v);
+        bool capped = false;
+        with_row_dist<G, V, U, U8>(a.rows, v, [&](const auto &dist) {
+            int none = 0;
+            capped = warp_alg1<KEYS_LOG>(dist, GraphRef{a.knn, a.K}, a.nav, a.L, s, (uint32_t)a.H - 1, a.hshift,
+                                         a.max_steps, v, 0, none, nullptr, 0, nullptr, nullptr, nullptr, &lg)
+                         .capped;
+            const int m = knn_row_keys(a, dist, s, v);
+            if (m > 0) log_append(lg, s.keys, m, v);
+        });
         if (lane == 0) {
             a.cand_count[j] = lg.count;
-            if (a.status) a.status[j] = o.capped ? -4 : 0;
+            if (a.status) a.status[j] = capped ? -4 : 0;
         }
         __syncwarp();
     }
@@ -106,18 +109,18 @@ __device__ __forceinline__ void collect_log_body(const CollectArgs &a) {
 
 // As for the searches: rows of up to 512 values at 64 registers and 32 warps
 // per SM, wider ones on the compiler's own budget.
-template <int G, int V, int U>
+template <int G, int V, int U, bool U8>
 __global__ void __launch_bounds__(256, 4) collect_log_kernel(CollectArgs a) {
-    collect_log_body<G, V, U>(a);
+    collect_log_body<G, V, U, U8>(a);
 }
-template <int G, int V, int U>
+template <int G, int V, int U, bool U8>
 __global__ void __launch_bounds__(256) collect_log_wide_kernel(CollectArgs a) {
-    collect_log_body<G, V, U>(a);
+    collect_log_body<G, V, U, U8>(a);
 }
 template <int G, int V, int U>
-constexpr auto collect_log_entry() {
-    if constexpr (V <= 4) return collect_log_kernel<G, V, U>;
-    else return collect_log_wide_kernel<G, V, U>;
+void (*collect_log_entry(bool u8))(CollectArgs) {
+    if constexpr (V > 4) return collect_log_wide_kernel<G, V, U, false>;  // no 8-bit copy at these widths
+    else return u8 ? collect_log_kernel<G, V, U, true> : collect_log_kernel<G, V, U, false>;
 }
 
 // Search-and-collect, second half: one block per node cuts its log to the C
@@ -126,7 +129,8 @@ constexpr auto collect_log_entry() {
 // bits (their order is the distances' order) find a bound that lets through
 // the C smallest and hardly more; those are sorted in shared memory by the
 // network of log_compact.  Bound by the shared-memory passes of the hash and
-// the sort; the log itself is read up to four times, from L2 after the first.  Each thread owns at most 32 log entries, whose
+// the sort; the log itself is read up to four times, from L2 after the first.
+// Each thread owns at most 32 log entries, whose
 // first-copy flags are one register.
 constexpr int SEL_BINS = 1024;
 constexpr int LOG_CAP_MAX = 16384;
@@ -318,8 +322,8 @@ static cudaError_t launch_select(const CollectArgs &a, cudaStream_t st) {
 cudaError_t launch_collect(const CollectLaunch &l, cudaStream_t st) {
     if (l.nv <= 0) return cudaSuccess;
     CollectArgs a;
-    a.base4 = reinterpret_cast<const float4 *>(l.base);
-    a.dp4 = l.dp / 4;
+    a.rows = ExactRows{reinterpret_cast<const float4 *>(l.base), l.dp / 4, reinterpret_cast<const uint4 *>(l.u8.rows),
+                       l.u8.chunks, l.u8.d, l.u8.lo};
     a.knn = l.knn;
     a.K = l.K;
     a.W = round32(l.K);
@@ -351,8 +355,8 @@ cudaError_t launch_collect(const CollectLaunch &l, cudaStream_t st) {
             a.cand_d2 = l.cand_d2 + j0 * l.C;
             a.cand_count = l.cand_count + j0;
             a.status = l.status != nullptr ? l.status + j0 : nullptr;
-            NSG_DISPATCH_DP4(a.dp4, {
-                auto kern = collect_log_entry<G_, V_, U_>();
+            NSG_DISPATCH_DP4(a.rows.dp4, {
+                auto kern = collect_log_entry<G_, V_, U_>(a.rows.u8 != nullptr);
                 int grid, wpb;
                 size_t smem;
                 err = config(kern, per_warp, 4, a.nv, &grid, &wpb, &smem);
@@ -366,7 +370,7 @@ cudaError_t launch_collect(const CollectLaunch &l, cudaStream_t st) {
         return err;
     }
     const size_t per_warp = warp_smem_bytes(a.L, a.W, a.C, a.H);
-    NSG_DISPATCH_DP4(a.dp4, {
+    NSG_DISPATCH_DP4(a.rows.dp4, {
         auto kern = collect_kernel<G_, V_, U_>;
         int grid, wpb;
         size_t smem;

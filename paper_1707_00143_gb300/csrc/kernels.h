@@ -167,6 +167,14 @@ inline float float_from_order_key(unsigned k) {
 cudaError_t launch_to_lowp(const float *src, int64_t n, int dp, int d, int precision, float scale, float lo,
                            void *dst, int dpl, int *inexact, cudaStream_t st);
 
+// An 8-bit copy of integer rows that gives the FP32 distances (lowp.cuh:
+// ExactRows), or none (rows nullptr).
+struct Exact8 {
+    const void *rows = nullptr;
+    int chunks = 0, d = 0;  // 16-byte chunks per row; values per row
+    float lo = 0.0f;
+};
+
 // Search-and-collect on the kNN graph for nodes v0..v0+nv-1.
 struct CollectLaunch {
     const float *base;  // [n][dp]
@@ -180,6 +188,7 @@ struct CollectLaunch {
     float *cand_d2;
     int *cand_count;
     int *status;
+    Exact8 u8;  // used by the log form
     // logs of collect_log_cap keys for log_nodes nodes at a time (nullptr: the
     // kernel that keeps sorted lists)
     uint64_t *log = nullptr;
@@ -200,6 +209,7 @@ struct PruneLaunch {
     int64_t v0, nv;
     int *adj;
     int *deg;
+    Exact8 u8;
     unsigned long long *examined = nullptr;  // nullable: += candidates examined over all nodes
 };
 cudaError_t launch_prune(const PruneLaunch &a, cudaStream_t st);

@@ -13,7 +13,7 @@
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
 
-#include "common.cuh"
+#include "search_core.cuh"
 
 namespace nsg {
 
@@ -254,5 +254,43 @@ struct DistLp {
         return group_sum<G>(s);
     }
 };
+
+// Rows whose distances the build measures: FP32, and (u8 not null) an 8-bit
+// copy x - lo that holds every value, d * 255^2 < 2^24, so that its integer
+// distances are the FP32 keys.
+struct ExactRows {
+    const float4 *base4;
+    int dp4;
+    const uint4 *u8;
+    int dc, d;
+    float lo;
+};
+
+// Lanes per 8-bit row and 16-byte chunks per lane at the dispatch shape G, V.
+template <int G, int V>
+struct Exact8Shape {
+    static constexpr int VG = V * G;  // float4s a group's registers hold
+    static constexpr int lanes = VG / 8 < 1 ? 1 : (VG / 8 > 32 ? 32 : VG / 8);
+    static constexpr int chunks = VG / (4 * lanes);
+};
+
+// The distance functor for row v as the query: FP32 rows, or the exact 8-bit
+// copy (a quarter of the bytes, the same keys), laid out as the 8-bit search
+// form lays it out (lanes of 2 16-byte chunks, 3 row groups in flight; 8 for
+// rows of 513..1024 values).
+template <int G, int V, int U, bool U8, class F>
+__device__ __forceinline__ void with_row_dist(const ExactRows &r, int64_t v, F &&f) {
+    if constexpr (U8) {
+        using S = Exact8Shape<G, V>;
+        constexpr int R8 = V == 8 ? 8 : (V > 8 ? 2 : 3);
+        DistU8<S::lanes, S::chunks, R8> dist{{}, r.u8, r.dc};
+        dist.Q.load(reinterpret_cast<const float *>(r.base4 + v * r.dp4), r.d, r.lo, 1.0f);
+        f(dist);
+    } else {
+        DistF32<G, V, U> dist{{}, r.base4, r.dp4};
+        dist.Q.load_row(r.base4 + v * r.dp4, r.dp4);
+        f(dist);
+    }
+}
 
 }  // namespace nsg

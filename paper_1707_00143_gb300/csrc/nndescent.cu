@@ -68,8 +68,7 @@ __device__ inline NdSmem nd_carve(unsigned char *p, int K) {
 }
 
 struct NdArgs {
-    const float4 *base4;
-    int dp4;
+    ExactRows rows;
     int64_t n;
     int K, S, Sr;
     uint64_t seed;
@@ -85,33 +84,7 @@ struct NdArgs {
     const int64_t *moff;    // [n + 1]
     int *members;           // (v << 1) | (p in NEW(v))
     unsigned long long *updates;
-    // 8-bit copy (rows of dc 16-byte chunks, x - lo) when it holds every
-    // distance exactly, else nullptr: distances on FP32 rows
-    const uint4 *u8;
-    int dc, d;
-    float lo;
 };
-
-// The distance functor for node v's row as the query: FP32 rows, or the exact
-// 8-bit copy (a quarter of the bytes, the same keys), laid out as the 8-bit
-// search form lays it out (lanes of 2 16-byte chunks, 3 row groups in flight;
-// 8 for rows of 513..1024 values).
-template <int G, int V, int U, bool U8, class F>
-__device__ __forceinline__ void nd_with_dist(const NdArgs &a, int64_t v, F &&f) {
-    if constexpr (U8) {
-        constexpr int VG = V * G;
-        constexpr int G8 = VG / 8 < 1 ? 1 : (VG / 8 > 32 ? 32 : VG / 8);
-        constexpr int VC = VG / (4 * G8);
-        constexpr int R8 = V == 8 ? 8 : (V > 8 ? 2 : 3);
-        DistU8<G8, VC, R8> dist{{}, a.u8, a.dc};
-        dist.Q.load(reinterpret_cast<const float *>(a.base4 + v * a.dp4), a.d, a.lo, 1.0f);
-        f(dist);
-    } else {
-        DistF32<G, V, U> dist{{}, a.base4, a.dp4};
-        dist.Q.load_row(a.base4 + v * a.dp4, a.dp4);
-        f(dist);
-    }
-}
 
 // init: K distinct seeded random neighbours per node, sorted by key.  One warp
 // per node: lane 0 draws, the warp checks each draw against the ids so far.
@@ -138,7 +111,7 @@ __global__ void __launch_bounds__(128) nd_init_kernel(NdArgs a) {
             }
         }
         int size = 0;
-        nd_with_dist<G, V, U, U8>(a, v, [&](const auto &dist) {
+        with_row_dist<G, V, U, U8>(a.rows, v, [&](const auto &dist) {
             for (int c0 = 0; c0 < a.K; c0 += ND_W) {
                 const int cnt = min(ND_W, a.K - c0);
                 for (int j = lane; j < cnt; j += 32) s.ids[j] = got[c0 + j];
@@ -321,7 +294,7 @@ __global__ void __launch_bounds__(128) nd_join_kernel(NdArgs a) {
         if (lane == 0) visit(s.hash, hmask, hshift, (int)p);
         __syncwarp();
         int size = a.K;
-        nd_with_dist<G, V, U, U8>(a, p, [&](const auto &dist) {
+        with_row_dist<G, V, U, U8>(a.rows, p, [&](const auto &dist) {
             int m = 0;
             const int64_t m0 = a.moff[p], m1 = a.moff[p + 1];
             for (int64_t mi = m0; mi < m1; ++mi) {
@@ -482,17 +455,13 @@ cudaError_t launch_nndescent(const NnDescentLaunch &l, cudaStream_t st) {
         return q;
     };
     NdArgs a;
-    a.base4 = reinterpret_cast<const float4 *>(l.base);
-    a.dp4 = l.dp / 4;
+    a.rows = ExactRows{reinterpret_cast<const float4 *>(l.base), l.dp / 4, reinterpret_cast<const uint4 *>(l.u8),
+                       l.u8_chunks, l.d, l.u8_lo};
     a.n = n;
     a.K = K;
     a.S = S;
     a.Sr = Sr;
     a.seed = l.seed;
-    a.u8 = reinterpret_cast<const uint4 *>(l.u8);
-    a.dc = l.u8_chunks;
-    a.d = l.d;
-    a.lo = l.u8_lo;
     a.lists = reinterpret_cast<uint64_t *>(take(8ull * n * K));
     a.newS = reinterpret_cast<uint64_t *>(take(8ull * n * std::max(S, 1)));
     a.oldS = reinterpret_cast<uint64_t *>(take(8ull * n * std::max(S, 1)));
@@ -519,8 +488,8 @@ cudaError_t launch_nndescent(const NnDescentLaunch &l, cudaStream_t st) {
     a.updates = reinterpret_cast<unsigned long long *>(take(8));
     const size_t per_warp = (nd_warp_bytes(K) + 15) & ~size_t(15);
     cudaError_t e = cudaSuccess;
-    const int dp4 = a.dp4;
-    const bool u8 = a.u8 != nullptr;
+    const int dp4 = a.rows.dp4;
+    const bool u8 = a.rows.u8 != nullptr;
     NSG_DISPATCH_DP4(dp4, {
         e = u8 ? warp_launch(nd_init_kernel<G_, V_, U_, true>, a, per_warp, st)
                : warp_launch(nd_init_kernel<G_, V_, U_, false>, a, per_warp, st);
