@@ -10,11 +10,6 @@
 namespace nsg {
 
 __host__ __device__ static inline int round32(int x) { return (x + 31) & ~31; }
-static inline int log2i(unsigned x) {
-    int r = 0;
-    while ((1u << r) < x) ++r;
-    return r;
-}
 
 template <typename T>
 __device__ __forceinline__ T ld_volatile(const T *p) {
@@ -58,105 +53,200 @@ cudaError_t launch_centroid(const float *base, int64_t n, int d, double *partial
 
 // ---------------------------------------------------------------------------
 // Navigating node (Alg. 2; Section 3.5 ii): Alg. 1 on the kNN graph from `start`
-// toward the centroid, one warp.  Distances are FP64 sums over j in order with
+// toward the centroid, one block.  Distances are FP64 sums over j in order with
 // explicitly rounded operations (no FMA), so they do not depend on the
-// compiler.  Lanes compute the distances of the new neighbours; lane 0 keeps
-// the sorted pool (one query: simplicity over speed).
+// compiler.
+//
+// One search is a chain of steps, so a step's latency is what counts.  Up to
+// NAV_ROWS neighbours at a time, the block reads tiles of NAV_TILE values of
+// all their rows (coalesced) and leaves the rounded squares in shared memory;
+// the first warps add a row's squares in order, one row per thread, while the
+// others fill the next tile; and the new keys enter the sorted pool by rank,
+// from one buffer into the other.  Bound by the chain of steps (~60 of ~7 us)
+// and the SM's few FP64 units.  One warp with a lane per row and lane 0
+// inserting took 1.65 ms for 100,000 SIFT-shaped rows (K = 100, L = 40,
+// centroid included; now 0.55), 0.86 ms for DEEP-shaped (now 0.35), 0.57 ms
+// for 10,000 x 32 (now 0.26).
 // ---------------------------------------------------------------------------
+constexpr int NAV_THREADS = 512, NAV_ROWS = 128, NAV_TILE = 64, NAV_PITCH = NAV_TILE + 1;
+
 __device__ __forceinline__ bool dkey_less(double da, int ia, double db, int ib) {
     return da < db || (da == db && ia < ib);
 }
+// the same order on the bits of distances >= +0 that are no NaN
+__device__ __forceinline__ bool bkey_less(uint64_t a, int ia, uint64_t b, int ib) {
+    return a < b || (a == b && ia < ib);
+}
 
-__global__ void navigate_kernel(const float *__restrict__ base, int d, const int *__restrict__ knn,
-                                int K, const double *__restrict__ cg, int start, int L,
-                                uint32_t *visited, int max_steps, int *nav_out, int *status) {
+struct NavShared {
+    int warp_new[NAV_ROWS / 32];
+    int at, u;
+    uint64_t ck[NAV_ROWS];  // the new nodes' distances (bits) and ids
+    int ci[NAV_ROWS];
+};
+
+__host__ __device__ inline size_t nav_smem_bytes(int d, int L) {
+    return 8ull * (d + 2 * NAV_ROWS * NAV_PITCH + 2 * (size_t)L) + 4ull * 2 * (size_t)L;
+}
+
+__global__ void __launch_bounds__(NAV_THREADS) navigate_kernel(const float *__restrict__ base, int d,
+                                                               const int *__restrict__ knn, int K,
+                                                               const double *__restrict__ cg, int start, int L,
+                                                               uint32_t *visited, int max_steps, int *nav_out,
+                                                               int *status) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int Wk = round32(K);
+    __shared__ NavShared sh;
     double *c = reinterpret_cast<double *>(smem);
-    double *pd = c + d;
-    double *cd = pd + (L + 1);
-    int *pid = reinterpret_cast<int *>(cd + Wk);
-    int *pchk = pid + (L + 1);
-    int *cid = pchk + (L + 1);
-    const unsigned lane = threadIdx.x & 31;
-    for (int j = lane; j < d; j += 32) c[j] = cg[j];
-    __syncwarp();
-    auto dist = [&](int id) -> double {
-        const float *x = base + (int64_t)id * d;
-        double s = 0.0;
-        for (int j = 0; j < d; ++j) {
-            double t = __dsub_rn((double)__ldg(x + j), c[j]);
-            s = __dadd_rn(s, __dmul_rn(t, t));
-        }
-        return s;
-    };
-    int size = 1;
-    if (lane == 0) {
+    double *tile = c + d;                                                             // two of NAV_ROWS rows
+    uint64_t *pk = reinterpret_cast<uint64_t *>(tile + 2 * NAV_ROWS * NAV_PITCH);     // two pools of L
+    int *pi = reinterpret_cast<int *>(pk + 2 * (size_t)L);                            // ids, bit 31 = checked
+    const int t = threadIdx.x, lane = t & 31;
+    const int tiles = (d + NAV_TILE - 1) / NAV_TILE;
+    for (int j = t; j < d; j += NAV_THREADS) c[j] = cg[j];
+    if (t == 0) {
         atomicOr(visited + (start >> 5), 1u << (start & 31));
-        pd[0] = dist(start);
-        pid[0] = start;
-        pchk[0] = 0;
+        sh.ci[0] = start;
     }
-    __syncwarp();
-    int steps = 0;
+    __syncthreads();
+    // squares of tile i of the rows sh.ci[0..m) by threads f0..NAV_THREADS-1
+    auto fill = [&](int i, int m, int f0) {
+        double *out = tile + (i & 1) * NAV_ROWS * NAV_PITCH;
+        const int j0 = i * NAV_TILE, w = min(NAV_TILE, d - j0);
+#pragma unroll 4
+        for (int e = t - f0; e < m * NAV_TILE; e += NAV_THREADS - f0) {
+            const int r = e / NAV_TILE, jj = e % NAV_TILE;
+            if (jj < w) {
+                const double x = __dsub_rn((double)__ldg(base + (int64_t)sh.ci[r] * d + j0 + jj), c[j0 + jj]);
+                out[r * NAV_PITCH + jj] = __dmul_rn(x, x);
+            }
+        }
+    };
+    // distances of the rows sh.ci[0..m) into sh.ck; whether one of them is a NaN
+    auto measure = [&](int m) -> bool {
+        double s = 0.0;
+        fill(0, m, 0);
+        __syncthreads();
+        for (int i = 0; i < tiles; ++i) {
+            if (t >= NAV_ROWS) {
+                if (i + 1 < tiles) fill(i + 1, m, NAV_ROWS);
+            } else if (t < m) {
+                const double *row = tile + (i & 1) * NAV_ROWS * NAV_PITCH + t * NAV_PITCH;
+                const int w = min(NAV_TILE, d - i * NAV_TILE);
+#pragma unroll 8
+                for (int jj = 0; jj < w; ++jj) s = __dadd_rn(s, row[jj]);
+            }
+            __syncthreads();
+        }
+        if (t < m) sh.ck[t] = (uint64_t)__double_as_longlong(s);
+        return __syncthreads_or(t < m && s != s) != 0;
+    };
+    // NaN distances have no order: the pool is then kept by insertion, one node after the other
+    bool serial = measure(1);
+    if (t == 0) {
+        pk[0] = sh.ck[0];
+        pi[0] = start;
+    }
+    __syncthreads();
+    int size = 1, cur = 0, steps = 0;
     bool capped = false;
     for (;;) {
-        int i = -1;
-        if (lane == 0)
-            for (int t = 0; t < size; ++t)
-                if (!pchk[t]) {
-                    i = t;
-                    break;
-                }
-        i = __shfl_sync(NSG_FULL, i, 0);
-        if (i < 0) break;
+        int *ids = pi + cur * L;
+        if (t < 32) {  // the first unchecked entry
+            int at = -1;
+            for (int b = 0; b < size && at < 0; b += 32) {
+                const unsigned bal = __ballot_sync(NSG_FULL, b + lane < size && ids[b + lane] >= 0);
+                if (bal) at = b + __ffs(bal) - 1;
+            }
+            if (lane == 0) {
+                sh.at = at;
+                if (at >= 0) sh.u = ids[at];
+            }
+        }
+        __syncthreads();
+        const int at = sh.at, u = sh.u;
+        if (at < 0) break;
         if (steps >= max_steps) {
             capped = true;
             break;
         }
         ++steps;
-        if (lane == 0) pchk[i] = 1;
-        __syncwarp();
-        const int u = pid[i];
-        int m = 0;
-        for (int b = 0; b < K; b += 32) {
-            int slot = b + lane;
-            int w = slot < K ? __ldg(knn + (int64_t)u * K + slot) : -1;
-            bool fresh = false;
-            if (w >= 0) {
-                uint32_t bit = 1u << (w & 31);
-                fresh = !(atomicOr(visited + (w >> 5), bit) & bit);
-            }
-            unsigned bal = __ballot_sync(NSG_FULL, fresh);
-            if (fresh) cid[m + __popc(bal & lanemask_lt())] = w;
-            m += __popc(bal);
-        }
-        __syncwarp();
-        for (int t = lane; t < m; t += 32) cd[t] = dist(cid[t]);
-        __syncwarp();
-        if (lane == 0) {
-            for (int t = 0; t < m; ++t) {
-                double dv = cd[t];
-                int iv = cid[t];
-                if (size == L && !dkey_less(dv, iv, pd[L - 1], pid[L - 1])) continue;
-                int pos = size < L ? size : L - 1;
-                while (pos > 0 && dkey_less(dv, iv, pd[pos - 1], pid[pos - 1])) {
-                    pd[pos] = pd[pos - 1];
-                    pid[pos] = pid[pos - 1];
-                    pchk[pos] = pchk[pos - 1];
-                    --pos;
+        if (t == 0) ids[at] |= INT_MIN;
+        for (int b = 0; b < K; b += NAV_ROWS) {
+            int w = -1, rank = 0;
+            if (t < NAV_ROWS) {
+                if (b + t < K) w = __ldg(knn + (int64_t)u * K + b + t);
+                if (w >= 0) {
+                    const uint32_t bit = 1u << (w & 31);
+                    if (atomicOr(visited + (w >> 5), bit) & bit) w = -1;
                 }
-                pd[pos] = dv;
-                pid[pos] = iv;
-                pchk[pos] = 0;
-                if (size < L) ++size;
+                const unsigned bal = __ballot_sync(NSG_FULL, w >= 0);
+                rank = __popc(bal & lanemask_lt());
+                if (lane == 0) sh.warp_new[t >> 5] = __popc(bal);
             }
+            __syncthreads();
+            int m = 0;
+#pragma unroll
+            for (int x = 0; x < NAV_ROWS / 32; ++x) {
+                if (x < (t >> 5)) rank += sh.warp_new[x];
+                m += sh.warp_new[x];
+            }
+            if (w >= 0) sh.ci[rank] = w;
+            __syncthreads();
+            if (m == 0) continue;
+            if (measure(m)) serial = true;
+            uint64_t *k0 = pk + cur * L;
+            int *i0 = pi + cur * L;
+            if (!serial) {
+                uint64_t *k1 = pk + (cur ^ 1) * L;
+                int *i1 = pi + (cur ^ 1) * L;
+                for (int x = t; x < NAV_ROWS + size; x += NAV_THREADS) {
+                    const bool fresh = x < NAV_ROWS;
+                    if (fresh && x >= m) continue;
+                    const uint64_t k = fresh ? sh.ck[x] : k0[x - NAV_ROWS];
+                    const int tag = fresh ? sh.ci[x] : i0[x - NAV_ROWS], id = tag & INT_MAX;
+                    int pos = x - NAV_ROWS;  // pool entries smaller than it
+                    if (fresh) {
+                        int lo = 0, hi = size;
+                        while (lo < hi) {
+                            const int mid = (lo + hi) >> 1;
+                            if (bkey_less(k0[mid], i0[mid] & INT_MAX, k, id)) lo = mid + 1;
+                            else hi = mid;
+                        }
+                        pos = lo;
+                    }
+                    for (int y = 0; y < m; ++y) pos += bkey_less(sh.ck[y], sh.ci[y], k, id);
+                    if (pos < L) {
+                        k1[pos] = k;
+                        i1[pos] = tag;
+                    }
+                }
+                cur ^= 1;
+            } else if (t == 0) {
+                int sz = size;
+                for (int x = 0; x < m; ++x) {
+                    const double dv = __longlong_as_double((long long)sh.ck[x]);
+                    const int iv = sh.ci[x];
+                    auto before = [&](int p) {
+                        return dkey_less(dv, iv, __longlong_as_double((long long)k0[p]), i0[p] & INT_MAX);
+                    };
+                    if (sz == L && !before(L - 1)) continue;
+                    int pos = sz < L ? sz : L - 1;
+                    while (pos > 0 && before(pos - 1)) {
+                        k0[pos] = k0[pos - 1];
+                        i0[pos] = i0[pos - 1];
+                        --pos;
+                    }
+                    k0[pos] = sh.ck[x];
+                    i0[pos] = iv;
+                    if (sz < L) ++sz;
+                }
+            }
+            size = min(L, size + m);
+            __syncthreads();
         }
-        size = __shfl_sync(NSG_FULL, size, 0);
-        __syncwarp();
     }
-    if (lane == 0) {
-        *nav_out = pid[0];
+    if (t == 0) {
+        *nav_out = pi[cur * L] & INT_MAX;
         *status = capped ? -4 : 0;
     }
 }
@@ -165,13 +255,12 @@ cudaError_t launch_navigate(const float *base, int64_t n, int d, const int *knn,
                             const double *c, int start, int L, uint32_t *visited_bits,
                             int max_steps, int *nav_out, int *status, cudaStream_t st) {
     (void)n;
-    int Wk = round32(K);
-    size_t smem = 8ull * (d + (L + 1) + Wk) + 4ull * (2 * (L + 1) + Wk);
+    const size_t smem = nav_smem_bytes(d, L);
     cudaError_t e = cudaFuncSetAttribute(navigate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    navigate_kernel<<<1, 32, smem, st>>>(base, d, knn, K, c, start, L, visited_bits, max_steps,
-                                         nav_out, status);
+    navigate_kernel<<<1, NAV_THREADS, smem, st>>>(base, d, knn, K, c, start, L, visited_bits, max_steps,
+                                                  nav_out, status);
     return cudaGetLastError();
 }
 
