@@ -41,27 +41,28 @@ __device__ __forceinline__ uint64_t nd_splitmix64(uint64_t x) {
     return z ^ (z >> 31);
 }
 
-// Per-warp shared memory: list [K], first [K] (the list at the iteration's
-// start), batch keys / merge scratch [ND_W], ids / positions [ND_W], hash.
+// Per-warp shared memory: list [K], first [K] (not in the join), batch keys /
+// merge scratch [ND_W], ids / positions [ND_W], hash.
 struct NdSmem {
     uint64_t *list, *first, *keys, *ck, *sk;
     int *ids, *cp, *sp;
     uint32_t *hash;
 };
 
-__host__ __device__ inline size_t nd_warp_bytes(int K) {
-    return 8ull * (2 * K + 3 * ND_W) + 4ull * (3 * ND_W + ND_HASH);
+__host__ __device__ inline size_t nd_warp_bytes(int K, bool join = false) {
+    return ((join ? 8ull * (K + 2 * ND_W) : 8ull * (2 * K + 3 * ND_W)) + 4ull * (3 * ND_W + ND_HASH) + 15) & ~size_t(15);
 }
 
-__device__ inline NdSmem nd_carve(unsigned char *p, int K) {
+// The join's merges consume their keys, so the sorted keys take their space.
+__device__ inline NdSmem nd_carve(unsigned char *p, int K, bool join = false) {
     NdSmem s;
     s.hash = reinterpret_cast<uint32_t *>(p);
     s.list = reinterpret_cast<uint64_t *>(s.hash + ND_HASH);
     s.first = s.list + K;
-    s.keys = s.first + K;
+    s.keys = join ? s.first : s.first + K;
     s.ck = s.keys + ND_W;
-    s.sk = s.ck + ND_W;
-    s.ids = reinterpret_cast<int *>(s.sk + ND_W);
+    s.sk = join ? s.keys : s.ck + ND_W;
+    s.ids = reinterpret_cast<int *>(s.ck + (join ? 1 : 2) * ND_W);
     s.cp = s.ids + ND_W;
     s.sp = s.cp + ND_W;
     return s;
@@ -93,7 +94,7 @@ __global__ void __launch_bounds__(128) nd_init_kernel(NdArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const unsigned lane = lane_id();
-    NdSmem s = nd_carve(smem + warp * ((nd_warp_bytes(a.K) + 15) & ~size_t(15)), a.K);
+    NdSmem s = nd_carve(smem + warp * nd_warp_bytes(a.K), a.K);
     int *got = reinterpret_cast<int *>(s.first);  // K ids (the first-list space is free here)
     for (int64_t v = (int64_t)blockIdx.x * wpb + warp; v < a.n; v += (int64_t)gridDim.x * wpb) {
         int m = 0;
@@ -200,7 +201,7 @@ __global__ void __launch_bounds__(128) nd_sets_kernel(NdArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const unsigned lane = lane_id();
-    NdSmem s = nd_carve(smem + warp * ((nd_warp_bytes(a.K) + 15) & ~size_t(15)), a.K);
+    NdSmem s = nd_carve(smem + warp * nd_warp_bytes(a.K), a.K);
     const int W2 = a.S + a.Sr;
     int *rn = reinterpret_cast<int *>(s.first);  // Sr ids each
     int *ro = rn + a.Sr;
@@ -273,12 +274,18 @@ __global__ void nd_member_fill_kernel(NdArgs a) {
 // The offers to p (NEW(v) u OLD(v) for members v with p in NEW(v), NEW(v)
 // for the others), the ones the visited set has not seen measured, and p's
 // list cut to its K smallest keys of itself and them.
+//
+// Bound by the latency of its gathers at 28 warps per SM (7 blocks, 72
+// registers; held to 64 registers for 8 blocks it spills, 28.5 -> 33.8 ms of
+// kNN stage): reading the members one after the other, three dependent loads
+// each, took the stage of 150,000 DEEP-shaped rows (K = 64, 6 iterations) 31.2
+// ms, with them read ahead it takes 28.5 ms.
 template <int G, int V, int U, bool U8>
-__global__ void __launch_bounds__(128) nd_join_kernel(NdArgs a) {
+__global__ void __launch_bounds__(128, V <= 4 ? 7 : 1) nd_join_kernel(NdArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const unsigned lane = lane_id();
-    NdSmem s = nd_carve(smem + warp * ((nd_warp_bytes(a.K) + 15) & ~size_t(15)), a.K);
+    NdSmem s = nd_carve(smem + warp * nd_warp_bytes(a.K, true), a.K, true);
     const uint32_t hmask = ND_HASH - 1;
     const int hshift = 32 - 10;  // log2(ND_HASH)
     const int W2 = a.S + a.Sr;
@@ -287,7 +294,6 @@ __global__ void __launch_bounds__(128) nd_join_kernel(NdArgs a) {
         for (int j = lane; j < a.K; j += 32) {
             const uint64_t e = a.lists[p * a.K + j];
             s.list[j] = e;
-            s.first[j] = kval(e);
             visit(s.hash, hmask, hshift, kid(e));  // the list's own ids need no offer
         }
         __syncwarp();
@@ -297,27 +303,50 @@ __global__ void __launch_bounds__(128) nd_join_kernel(NdArgs a) {
         with_row_dist<G, V, U, U8>(a.rows, p, [&](const auto &dist) {
             int m = 0;
             const int64_t m0 = a.moff[p], m1 = a.moff[p + 1];
-            for (int64_t mi = m0; mi < m1; ++mi) {
-                const int tag = a.members[mi];
-                const int64_t v = tag >> 1;
-                const int cn = a.cNEW[v], co = (tag & 1) ? a.cOLD[v] : 0;
-                for (int b = 0; b < cn + co; b += 32) {
+            // 32 members' tags and counts at a time, one per lane, and the next
+            // member's first 64 offers read before the current one's are
+            // visited: one round trip per member instead of three in a row
+            for (int64_t g0 = m0; g0 < m1; g0 += 32) {
+                const int members = m1 - g0 < 32 ? (int)(m1 - g0) : 32;
+                int64_t row = 0;
+                int cn = 0, tot = 0;
+                if ((int)lane < members) {
+                    const int tag = a.members[g0 + lane];
+                    const int v = tag >> 1;
+                    row = (int64_t)v * W2;
+                    cn = a.cNEW[v];
+                    tot = cn + ((tag & 1) ? a.cOLD[v] : 0);
+                }
+                auto offer = [&](int i, int b) -> int {
+                    const int64_t r = __shfl_sync(NSG_FULL, row, i);
+                    const int c = __shfl_sync(NSG_FULL, cn, i), t = __shfl_sync(NSG_FULL, tot, i);
                     const int j = b + (int)lane;
-                    const int x = j < cn ? a.NEWs[v * W2 + j] : (j < cn + co ? a.OLDs[v * W2 + j - cn] : -1);
-                    // p itself is among its own offers (p is in NEW(v)); the visited set
-                    // may have forgotten it, so it is excluded by id
-                    const bool fresh = x >= 0 && x != (int)p && visit(s.hash, hmask, hshift, x);
-                    const unsigned bal = __ballot_sync(NSG_FULL, fresh);
-                    const int cnt = __popc(bal);
-                    if (m + cnt > ND_W) {  // flush the batch first
-                        __syncwarp();
-                        dist(s.ids, m, s.keys);
-                        warp_merge(s.list, a.K, size, s.keys, m, s.ck, s.cp, s.sk, s.sp);
-                        m = 0;
+                    return j < c ? __ldg(a.NEWs + r + j) : (j < t ? __ldg(a.OLDs + r + j - c) : -1);
+                };
+                int x0 = offer(0, 0), x1 = offer(0, 32);
+                for (int i = 0; i < members; ++i) {
+                    const int y0 = x0, y1 = x1, t = __shfl_sync(NSG_FULL, tot, i);
+                    if (i + 1 < members) {
+                        x0 = offer(i + 1, 0);
+                        x1 = offer(i + 1, 32);
                     }
-                    if (fresh) s.ids[m + __popc(bal & lanemask_lt())] = x;
-                    m += cnt;
-                    __syncwarp();
+                    for (int b = 0; b < t; b += 32) {
+                        const int x = b == 0 ? y0 : b == 32 ? y1 : offer(i, b);
+                        // p itself is among its own offers (p is in NEW(v)); the visited set
+                        // may have forgotten it, so it is excluded by id
+                        const bool fresh = x >= 0 && x != (int)p && visit(s.hash, hmask, hshift, x);
+                        const unsigned bal = __ballot_sync(NSG_FULL, fresh);
+                        const int cnt = __popc(bal);
+                        if (m + cnt > ND_W) {  // flush the batch first
+                            __syncwarp();
+                            dist(s.ids, m, s.keys);
+                            warp_merge(s.list, a.K, size, s.keys, m, s.ck, s.cp, s.sk, s.sp);
+                            m = 0;
+                        }
+                        if (fresh) s.ids[m + __popc(bal & lanemask_lt())] = x;
+                        m += cnt;
+                        __syncwarp();
+                    }
                 }
             }
             if (m > 0) {
@@ -325,17 +354,21 @@ __global__ void __launch_bounds__(128) nd_join_kernel(NdArgs a) {
                 warp_merge(s.list, a.K, size, s.keys, m, s.ck, s.cp, s.sk, s.sp);
             }
         });
-        // entries that were not in the list at the iteration's start
+        // entries that were not in the list at the iteration's start (read again
+        // into the visited set's space: K keys, 2 K <= ND_HASH)
+        uint64_t *first = reinterpret_cast<uint64_t *>(s.hash);
+        for (int j = lane; j < a.K; j += 32) first[j] = kval(a.lists[p * a.K + j]);
+        __syncwarp();
         int changed = 0;
         for (int j = lane; j < a.K; j += 32) {
             const uint64_t k = kval(s.list[j]);
             int lo = 0, hi = a.K;
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
-                if (s.first[mid] < k) lo = mid + 1;
+                if (first[mid] < k) lo = mid + 1;
                 else hi = mid;
             }
-            changed += !(lo < a.K && s.first[lo] == k);
+            changed += !(lo < a.K && first[lo] == k);
             a.lists[p * a.K + j] = s.list[j];
         }
 #pragma unroll
@@ -486,7 +519,7 @@ cudaError_t launch_nndescent(const NnDescentLaunch &l, cudaStream_t st) {
     const int64_t nb = (n + SCAN_T * SCAN_PER - 1) / (SCAN_T * SCAN_PER);
     int64_t *bsum = reinterpret_cast<int64_t *>(take(8ull * nb));
     a.updates = reinterpret_cast<unsigned long long *>(take(8));
-    const size_t per_warp = (nd_warp_bytes(K) + 15) & ~size_t(15);
+    const size_t per_warp = nd_warp_bytes(K), join_warp = nd_warp_bytes(K, true);
     cudaError_t e = cudaSuccess;
     const int dp4 = a.rows.dp4;
     const bool u8 = a.rows.u8 != nullptr;
@@ -514,8 +547,8 @@ cudaError_t launch_nndescent(const NnDescentLaunch &l, cudaStream_t st) {
         if ((e = cudaMemsetAsync(a.mcnt, 0, 4ull * n, st)) != cudaSuccess) return e;
         nd_member_fill_kernel<<<grid_for(n * std::max(W2, 1), 256), 256, 0, st>>>(a);
         NSG_DISPATCH_DP4(dp4, {
-            e = u8 ? warp_launch(nd_join_kernel<G_, V_, U_, true>, a, per_warp, st)
-                   : warp_launch(nd_join_kernel<G_, V_, U_, false>, a, per_warp, st);
+            e = u8 ? warp_launch(nd_join_kernel<G_, V_, U_, true>, a, join_warp, st)
+                   : warp_launch(nd_join_kernel<G_, V_, U_, false>, a, join_warp, st);
         });
         if (e != cudaSuccess) return e;
         if ((e = cudaMemcpyAsync(&upd, a.updates, 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
