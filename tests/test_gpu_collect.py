@@ -22,8 +22,9 @@ N = 6000
     (20, 256, 200, 30, 511),   # 256 threads per node
     (32, 256, 30, 60, 4096),   # 512 threads; fewer keys than the list holds
     (600, 16, 64, 60, 300),    # wide rows
-    (32, 256, 128, 128, 300),  # the longest log
-    (32, 256, 129, 128, 300),  # merged lists
+    (32, 256, 128, 128, 300),  # log of 8,192
+    (32, 256, 256, 128, 300),  # the longest log
+    (32, 256, 257, 128, 300),  # merged lists
 ])
 def test_collect_equals_oracle(nsg, d, span, K, L, C):
     rng = np.random.default_rng(1000 * K + L)
