@@ -39,6 +39,9 @@ struct nsg_index {
     float lowp_lo[4] = {0, 0, 0, 0};        // U8 offset
     int lowp_exact[4] = {0, 0, 0, 0};       // every value (U8: every distance) survived
     void *lowp_map[4] = {nullptr, nullptr, nullptr, nullptr};  // device tensor maps for staged four-row gathers
+    // integer rows: 8-bit copy whose distances are the FP32 ones (exact8.rows null: none)
+    void *exact8_buf = nullptr;
+    nsg::Exact8 exact8;
     int max_degree = 0;
     double avg_degree = 0.0;
     int64_t n_fixup = 0;
@@ -497,6 +500,7 @@ void destroy(nsg_index *ix) {
     if (ix->deg) cudaFree(ix->deg);
     if (ix->flag) cudaFree(ix->flag);
     if (ix->work) cudaFree(ix->work);
+    if (ix->exact8_buf) cudaFree(ix->exact8_buf);
     for (void *p : ix->lowp)
         if (p) cudaFree(p);
     for (void *p : ix->lowp_map)
@@ -511,6 +515,21 @@ void destroy(nsg_index *ix) {
     if (ix->part_d2) cudaFree(ix->part_d2);
     if (ix->gpool) cudaFree(ix->gpool);
     delete ix;
+}
+
+// The index keeps the exact 8-bit copy of its rows, if they have one.
+void keep_exact8(nsg_index *ix, DevBuf<unsigned char> &buf, const nsg::Exact8 &x) {
+    if (x.rows) {
+        ix->exact8 = x;
+        ix->exact8_buf = buf.release();
+    }
+}
+nsg_status make_exact8(nsg_index *ix, cudaStream_t st) {
+    DevBuf<unsigned char> buf;
+    nsg::Exact8 x;
+    if (nsg_status s = exact8_copy(ix->base, ix->n, ix->dp, ix->d, buf, x, st)) return s;
+    keep_exact8(ix, buf, x);
+    return NSG_OK;
 }
 
 double since_ms(std::chrono::steady_clock::time_point t0) {
@@ -767,6 +786,7 @@ nsg_status nsg_build_naive(const float *base_dev, int64_t n, int32_t d, int32_t 
     ix->adj = adj.release();
     ix->deg = deg.release();
     s = finish_index(ix, st);
+    if (!s) s = make_exact8(ix, st);
     ix->ms[5] = (float)since_ms(t_all);
     if (s) {
         destroy(ix);
@@ -838,6 +858,7 @@ static nsg_status build_index(const float *base_dev, int64_t n, int32_t d, int32
     ix->base = base.release();
     ix->adj = adj.release();
     ix->deg = deg.release();
+    keep_exact8(ix, u8buf, u8);
     s = finish_index(ix, st);
     ix->ms[5] = (float)since_ms(t_all);
     if (s) {
@@ -946,6 +967,7 @@ nsg_status nsg_index_from_graph(const float *base_dev, int64_t n, int32_t d, con
         ix->adj = adj.release();
         ix->deg = deg.release();
         s = finish_index(ix, st);
+        if (!s) s = make_exact8(ix, st);
         if (s) {
             destroy(ix);
             return s;
@@ -1035,6 +1057,7 @@ nsg_status nsg_build_partitioned(const float *base_dev, int64_t n, int32_t d, co
         ix->n_fixup_searches = researched;
         ix->prune_examined = examined;
         s = finish_index(ix, st);
+        if (!s) s = make_exact8(ix, st);
         if (s) return s;
         ix->ms[5] = (float)since_ms(t_all);
         *out = hold.release();
@@ -1045,6 +1068,15 @@ nsg_status nsg_build_partitioned(const float *base_dev, int64_t n, int32_t d, co
 namespace {
 
 // Validated launch description for nsg_search_ex / nsg_search_trace.
+// The plain form on integer rows takes its keys from the index's 8-bit copy.
+void use_exact8(const nsg_index *idx, nsg::SearchLaunch &l) {
+    if (!idx->exact8.rows) return;
+    l.exact8 = true;
+    l.lowp = idx->exact8.rows;
+    l.lowp_chunks = idx->exact8.chunks;
+    l.lowp_lo = idx->exact8.lo;
+}
+
 nsg_status make_search(const nsg_index *idx, const float *queries_dev, int64_t nq, int32_t k, int32_t L,
                        const nsg_search_params *params, int32_t *ids_dev, float *d2_dev, int32_t *n_expand_dev,
                        int32_t *n_dist_dev, int32_t *status_dev, nsg::SearchLaunch &l) {
@@ -1096,6 +1128,7 @@ nsg_status make_search(const nsg_index *idx, const float *queries_dev, int64_t n
     const bool staged = idx->dp > 512 && (p.stage_rows > 0 || (p.stage_rows == 0 && p.precision == NSG_PREC_F32));
     l.hash_slots = p.hash_slots > 0 ? p.hash_slots
                                     : default_search_hash(L, idx->R, nq, l.warps_per_query, staged || p.stop_model);
+    if (p.precision == NSG_PREC_F32) use_exact8(idx, l);
     if (p.precision != NSG_PREC_F32) {
         l.precision = p.precision;
         l.lowp = idx->lowp[p.precision];
@@ -1662,6 +1695,7 @@ nsg_status nsg_search(const nsg_index *idx, const float *queries_dev, int64_t nq
     l.warps_per_query = nsg::search_auto_wpq(nq, idx->dp, NSG_PREC_F32, L);
     l.hash_slots = default_search_hash(L, idx->R, nq, l.warps_per_query, idx->dp > 512);
     l.pool_global = L > 1024;
+    use_exact8(idx, l);
     NSG_CK(cudaMemsetAsync(idx->flag, 0, sizeof(int), st));
     if (nsg_status ls = launch_dynamic(idx, l, st)) return ls;
     int h = 0;
@@ -1700,6 +1734,7 @@ nsg_status nsg_index_info(const nsg_index *idx, nsg_index_info_t *info) {
     info->prune_examined = idx->prune_examined;
     for (int p = 1; p <= 3; ++p)
         if (idx->lowp[p]) info->device_bytes += (int64_t)idx->n * idx->lowp_dpl[p] * (p == 1 ? 2 : 1);
+    if (idx->exact8.rows) info->device_bytes += (int64_t)idx->n * idx->exact8.chunks * 16;
     info->ms_knn = idx->ms[0];
     info->ms_centroid_nav = idx->ms[1];
     info->ms_collect = idx->ms[2];

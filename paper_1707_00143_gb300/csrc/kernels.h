@@ -35,6 +35,7 @@ struct SearchLaunch {
     int *any_capped;  // device flag, nullable
     // precision forms: traversal on a BF16 / FP8 copy, FP32 re-rank of the pool
     int precision = 0;  // 0 FP32, 1 BF16, 2 FP8-e4m3, 3 U8
+    bool exact8 = false;  // FP32 form: lowp is the index's exact 8-bit copy
     const void *lowp = nullptr;
     int lowp_chunks = 0;  // 16-byte chunks per low-precision row
     float lowp_scale = 1.0f;

@@ -72,6 +72,7 @@ cudaError_t launch_search(const SearchLaunch &l, cudaStream_t st) {
         return a.gpool != nullptr ? launch_search_staged_global(a, l, pw, wpq, st)
                                   : launch_search_staged(a, l, pw, wpq, st);
     }
+    if (l.exact8 && !stop && l.precision == PREC_F32) return launch_search_int8(a, l, per_warp, wpq, st);
     if (a.gpool != nullptr) return launch_search_global(a, l, per_warp, per_cta, stop, wpq, st);
     return launch_search_args<false>(a, l, per_warp, per_cta, stop, wpq, st);
 }

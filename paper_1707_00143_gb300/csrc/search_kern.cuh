@@ -131,6 +131,23 @@ __device__ __forceinline__ bool with_dist(const SearchArgs &a, const float *qp, 
         dist.Q.load(qp, a.d, a.dp4);
         run_dist<ST>(dist, sr, nullptr, f);
         return true;
+    } else if constexpr (P == PREC_F32_INT8) {
+        using S = Exact8Shape<G, V>;
+        DistU8<S::lanes, S::chunks, NSG_U8ROWS> d8{{}, a.lowp, a.dc};
+        // integers that the copy's map keeps: their distances are exact in both forms
+        bool whole = true;
+        for (int j = lane_id(); j < a.d; j += 32) {
+            const float v = __ldg(qp + j);
+            whole &= rintf(v) == v;
+        }
+        if (d8.Q.load(qp, a.d, a.lo, 1.0f) && __all_sync(NSG_FULL, whole)) {
+            f(d8);
+        } else {
+            DistF32<G, V, U> dist{{}, a.base4, a.dp4};
+            dist.Q.load(qp, a.d, a.dp4);
+            f(dist);
+        }
+        return true;
     } else if constexpr (P == PREC_U8) {
         // an 8-bit row is a quarter of the FP32 row: G8 lanes of up to
         // NSG_U8CHUNKS 16-byte chunks each, 32 / G8 rows per pass
@@ -169,7 +186,7 @@ __device__ __forceinline__ void finish_query(const SearchArgs &a, WarpSmem &s, c
     const unsigned lane = lane_id();
     const uint64_t *res = s.pool;
     int rsize = o.size;
-    if constexpr (P != PREC_F32) if (rerank) {
+    if constexpr (P != PREC_F32 && P != PREC_F32_INT8) if (rerank) {
         uint64_t *cl = a.C > 0 ? s.clist : reinterpret_cast<uint64_t *>(s.hash);
         // the re-rank gathers all L pool rows at once: more rows in flight
         // than the traversal for rows of 513..1024 values
@@ -386,6 +403,19 @@ static void (*search_entry(bool stop, int wpq))(SearchArgs) {
     }
 }
 
+// The plain form on integer rows with an exact 8-bit copy (rows of up to 258
+// values, no stop model).
+template <int G, int V, int U, bool GP>
+static void (*int8_entry(int wpq))(SearchArgs) {
+    if constexpr (V <= 4) {
+        if (wpq == 2) return search_group_kernel<G, V, U, PREC_F32_INT8, 2, GP>;
+        if (wpq == 4) return search_group_kernel<G, V, U, PREC_F32_INT8, 4, GP>;
+        return search_kernel<G, V, U, PREC_F32_INT8, GP>;
+    } else {
+        return nullptr;
+    }
+}
+
 template <int G, int V, int U, int P, bool GP>
 static void (*staged_entry(int wpq))(SearchArgs) {
     if (wpq == 2) return search_group_staged_kernel<G, V, U, P, 2, GP>;
@@ -419,14 +449,16 @@ static cudaError_t config(K kernel, size_t smem_per_warp, int want_wpb, int64_t 
 // Launch of the search kernels for the launch description `a`: pools in
 // shared memory (GP false) or in the global slots a.gpool (GP true, at most
 // gpool_slots resident warps or groups); ST: the staged-gather kernels (rows
-// of more than 512 values, no stop model).
-template <bool GP, bool ST = false>
+// of more than 512 values, no stop model); INT8: the plain form on integer rows.
+template <bool GP, bool ST = false, bool INT8 = false>
 cudaError_t launch_search_args(const SearchArgs &a, const SearchLaunch &l, size_t per_warp, size_t per_cta,
                                bool stop, int wpq, cudaStream_t st) {
     cudaError_t err = cudaSuccess;
     NSG_DISPATCH_DP4(a.dp4, {
         void (*kern)(SearchArgs) = nullptr;
-        if constexpr (ST) {
+        if constexpr (INT8) {
+            kern = int8_entry<G_, V_, U_, GP>(wpq);
+        } else if constexpr (ST) {
             if constexpr (V_ >= 8)
                 if (!stop)
                     kern = l.precision == PREC_BF16  ? staged_entry<G_, V_, U_, PREC_BF16, GP>(wpq)
@@ -457,9 +489,10 @@ cudaError_t launch_search_args(const SearchArgs &a, const SearchLaunch &l, size_
     return err;
 }
 
-// The global-memory and staged instantiations live in translation units of
-// their own (search_global.cu, search_staged.cu, search_staged_global.cu) so
-// they compile in parallel.
+// The global-memory, staged and integer-row instantiations live in translation
+// units of their own (search_global.cu, search_staged.cu,
+// search_staged_global.cu, search_int8.cu) so they compile in parallel.
+cudaError_t launch_search_int8(const SearchArgs &a, const SearchLaunch &l, size_t per_warp, int wpq, cudaStream_t st);
 cudaError_t launch_search_global(const SearchArgs &a, const SearchLaunch &l, size_t per_warp, size_t per_cta,
                                  bool stop, int wpq, cudaStream_t st);
 cudaError_t launch_search_staged(const SearchArgs &a, const SearchLaunch &l, size_t per_warp, int wpq,
