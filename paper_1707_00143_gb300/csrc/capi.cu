@@ -353,7 +353,8 @@ nsg_status navigate_run(const float *base, int64_t n, int d, const int *knn, int
 }
 
 nsg_status connect_run(const float *bp, int64_t n, int dp, int *adj, int *deg, int R, int nav, int L,
-                       int *n_added, cudaStream_t st, int *n_research = nullptr) {
+                       int *n_added, cudaStream_t st, int *n_research = nullptr,
+                       const nsg::Exact8 &u8 = nsg::Exact8{}) {
     nsg::ConnectLaunch c;
     c.base = bp;
     c.n = n;
@@ -364,6 +365,7 @@ nsg_status connect_run(const float *bp, int64_t n, int dp, int *adj, int *deg, i
     c.nav = nav;
     c.L = L;
     c.hash_slots = default_hash(L, R);
+    c.u8 = u8;
     c.max_steps = nsg::default_steps(L);
     int h[4] = {0, 0, 0, 0};
     NSG_CK(nsg::run_connect(c, h, st));
@@ -847,7 +849,7 @@ static nsg_status build_index(const float *base_dev, int64_t n, int32_t d, int32
     // A7: connectivity
     t0 = std::chrono::steady_clock::now();
     int added = 0, research = 0;
-    if (!s) s = connect_run(base.p, n, ix->dp, adj.p, deg.p, R, ix->nav, L, &added, st, &research);
+    if (!s) s = connect_run(base.p, n, ix->dp, adj.p, deg.p, R, ix->nav, L, &added, st, &research, u8);
     ix->ms[4] = (float)since_ms(t0);
     ix->n_fixup = added;
     ix->n_fixup_searches = research;

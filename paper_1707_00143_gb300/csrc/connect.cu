@@ -41,12 +41,14 @@
 // repeated a stale search alone.  Measured (whole build, before -> after):
 // 10,000 x 32 16.9 -> 5.4 ms, 100,000 x 128 115.6 -> 58.9 ms, 150,000 x 96 on
 // an nn-descent graph 106.4 -> 51.8 ms (the pass itself 66 -> 4, 65 -> 5 and
-// 68 -> 8 ms).
+// 68 -> 8 ms).  With the exact 8-bit copy of integer rows (one round of gathers
+// per expansion instead of three or four) and the largest visited set that
+// fits, the pass takes 2.8, 3.2 and 6.2 ms of 2.9, 3.9 and 6.4 before.
 #include <climits>
 #include <vector>
 
 #include "kernels.h"
-#include "search_core.cuh"
+#include "lowp.cuh"
 
 #ifndef NSG_CONNECT_U_WIDE8
 #define NSG_CONNECT_U_WIDE8 4  // rows in flight per warp, 513..1024-value rows
@@ -159,6 +161,7 @@ __global__ void __launch_bounds__(1024) gather_unreached_kernel(const uint32_t *
 }
 
 struct FixArgs {
+    ExactRows rows;  // base4, dp4 and the exact 8-bit copy, if any
     const float4 *base4;
     int dp4;
     int64_t n;
@@ -342,7 +345,7 @@ __device__ __forceinline__ int fix_select(const FixArgs &a, int f, const uint64_
     return -1;
 }
 
-template <int G, int V, int U>
+template <int G, int V, int U, bool U8>
 __global__ void __launch_bounds__(256) fix_search_kernel(FixArgs a, int round) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
@@ -356,12 +359,13 @@ __global__ void __launch_bounds__(256) fix_search_kernel(FixArgs a, int round) {
         uint64_t *pool = a.pools + (int64_t)f * a.L;
         int size;
         if (round == 0 || fix_stale(a, f, u)) {
-            DistF32<G, V, U> dist{{}, a.base4, a.dp4};
-            dist.Q.load_row(a.base4 + (int64_t)u * a.dp4, a.dp4);
-            const SearchOut o = warp_alg1<KEYS_POOL>(dist, GraphView{a.adj, a.R, a.deg, a.label, a.flab[f]}, a.nav, a.L,
-                                                 s, (uint32_t)a.H - 1, a.hshift, a.max_steps, -1, 0, csize,
-                                                 a.xlog + (int64_t)f * a.xcap, a.xcap, nullptr,
-                                                 a.xthr + (int64_t)f * a.xcap);
+            SearchOut o;
+            with_row_dist<G, V, U, U8>(a.rows, u, [&](const auto &dist) {
+                o = warp_alg1<KEYS_POOL>(dist, GraphView{a.adj, a.R, a.deg, a.label, a.flab[f]}, a.nav, a.L, s,
+                                         (uint32_t)a.H - 1, a.hshift, a.max_steps, -1, 0, csize,
+                                         a.xlog + (int64_t)f * a.xcap, a.xcap, nullptr,
+                                         a.xthr + (int64_t)f * a.xcap);
+            });
             size = o.size;
             for (int t = lane; t < size; t += 32) pool[t] = s.pool[t];
             if (lane == 0) {
@@ -564,6 +568,7 @@ cudaError_t run_connect(const ConnectLaunch &l, int out_host[4], cudaStream_t st
     FixArgs a;
     a.base4 = reinterpret_cast<const float4 *>(l.base);
     a.dp4 = l.dp / 4;
+    a.rows = ExactRows{a.base4, a.dp4, reinterpret_cast<const uint4 *>(l.u8.rows), l.u8.chunks, l.u8.d, l.u8.lo};
     a.n = n;
     a.adj = l.adj;
     a.deg = l.deg;
@@ -571,8 +576,6 @@ cudaError_t run_connect(const ConnectLaunch &l, int out_host[4], cudaStream_t st
     a.W = round32c(l.R);
     a.nav = l.nav;
     a.L = l.L;
-    a.H = l.hash_slots;
-    a.hshift = 32 - log2c((unsigned)l.hash_slots);
     a.max_steps = l.max_steps;
     a.reached = reinterpret_cast<uint32_t *>(at(o_reached));
     a.stamp = reinterpret_cast<int *>(at(o_stamp));
@@ -625,7 +628,7 @@ cudaError_t run_connect(const ConnectLaunch &l, int out_host[4], cudaStream_t st
         if ((e = cudaMemcpyAsync(lev, &nf, sizeof(int), cudaMemcpyHostToDevice, st))) return e;
     }
     const int wpb = 4;
-    const size_t per_warp = warp_smem_bytes(l.L, a.W, 0, a.H, true), psmem = 16 * (size_t)BMAX;
+    const size_t psmem = 16 * (size_t)BMAX;
     if ((e = cudaFuncSetAttribute(fix_propose_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem)) ||
         (e = list_next()) || (e = cudaStreamSynchronize(st)))
         return e;
@@ -641,7 +644,21 @@ cudaError_t run_connect(const ConnectLaunch &l, int out_host[4], cudaStream_t st
             // not the occupancy, sets the time: 513..1024-value rows keep more
             // rows in flight than the search kernels do
             constexpr int UC = V_ == 8 ? NSG_CONNECT_U_WIDE8 : U_;
-            auto search = fix_search_kernel<G_, V_, UC>;
+            void (*search)(FixArgs, int) = fix_search_kernel<G_, V_, UC, false>;
+            if constexpr (V_ <= 4)
+                if (a.rows.u8 != nullptr) search = fix_search_kernel<G_, V_, UC, true>;
+            // a batch has few searches: the largest visited set (little measured
+            // twice) that lets all of them run at once; with 512 slots the pass
+            // takes 3.20 ms instead of 3.16 (SIFT-shaped 100,000), 6.37 instead of
+            // 6.19 (DEEP-shaped 150,000)
+            const int64_t blocks = ((h.cnt + wpb - 1) / wpb + sm_count() - 1) / sm_count();  // per SM
+            a.H = l.hash_slots;
+            for (int slots = 4096; slots > a.H; slots >>= 1)
+                if (blocks * (wpb * warp_smem_bytes(l.L, a.W, 0, slots, true) + 1024) <= smem_per_sm() &&
+                    wpb * warp_smem_bytes(l.L, a.W, 0, slots, true) <= smem_optin())
+                    a.H = slots;
+            a.hshift = 32 - log2c((unsigned)a.H);
+            const size_t per_warp = warp_smem_bytes(l.L, a.W, 0, a.H, true);
             e = cudaFuncSetAttribute(search, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(per_warp * wpb));
             for (int r = 0; r < CONNECT_ROUNDS && !e; ++r) {
                 search<<<(h.cnt + wpb - 1) / wpb, wpb * 32, per_warp * wpb, st>>>(a, r);

@@ -237,6 +237,7 @@ struct ConnectLaunch {
     int *adj;  // [n][R], edited in place
     int *deg;
     int R, nav, L;
+    Exact8 u8;
     int hash_slots, max_steps;
 };
 // Whole connectivity pass (reach from nav, then batches of fix-ups).  out = {edges added, status, any search capped, re-searches}.
