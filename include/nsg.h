@@ -135,7 +135,7 @@ typedef struct {
     int32_t max_degree;    /* largest out-degree present */
     double avg_degree;     /* mean out-degree (AOD of Table 2) */
     int64_t n_fixup_edges; /* edges added by the connectivity pass */
-    int64_t device_bytes;  /* device memory held by the index */
+    int64_t device_bytes;  /* device memory held by the index (integer rows: with their 8-bit copy) */
     int32_t has_bf16;      /* BF16 copy: 0 none, 1 lossy, 2 every value exact */
     int32_t has_fp8;       /* FP8-e4m3 copy: 0 none, 1 lossy, 2 every value exact */
     float fp8_scale;       /* x_fp8 = x * fp8_scale (0 when absent) */
