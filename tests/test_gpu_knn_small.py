@@ -9,8 +9,8 @@ import oracle
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n, nq, d, k", [(7167, 33, 32, 10), (7168, 33, 32, 10), (7300, 32, 20, 1), (129, 300, 128, 100),
-                                         (9000, 2049, 48, 100), (9000, 2048, 48, 100), (11000, 4097, 16, 10),
+@pytest.mark.parametrize("n, nq, d, k", [(8447, 33, 32, 10), (8448, 33, 32, 10), (8500, 32, 20, 1), (129, 300, 128, 100),
+                                         (9000, 1025, 48, 100), (9000, 1024, 48, 100), (11000, 4097, 16, 10),
                                          (16385, 4097, 16, 3)])
 def test_query_equals_oracle(nsg, n, nq, d, k):
     rng = np.random.default_rng(n + nq)
