@@ -87,6 +87,14 @@ bool knn_force_scan() {
     return e && std::strcmp(e, "scan") == 0;
 }
 
+// Search-and-collect (tests; read at every call): NSG_COLLECT_ENGINE=merge keeps
+// sorted lists instead of logs; NSG_COLLECT_LOG="size,cap" sets the keys of the
+// log and of a node's share in the first slice.
+bool collect_force(const char *engine) {
+    const char *e = std::getenv("NSG_COLLECT_ENGINE");
+    return e && std::strcmp(e, engine) == 0;
+}
+
 nsg_status cuda_fail(cudaError_t e, const char *what) {
     std::snprintf(g_err, sizeof(g_err), "%s: %s", what, cudaGetErrorString(e));
     return NSG_ECUDA;
@@ -399,6 +407,24 @@ nsg_status connect_run(const float *bp, int64_t n, int dp, int *adj, int *deg, i
     return h[2] ? NSG_ESTEPCAP : NSG_OK;
 }
 
+// Logs of the searches' keys for nv nodes.  Without that memory log.keys stays
+// null: the collect lists are merged as they grow.
+void make_collect_log(int L, int K, int64_t nv, DevBuf<uint64_t> &buf, nsg::CollectLog &log) {
+    log.size = nsg::collect_log_keys(L, K, nv);
+    if (!log.size) return;
+    if (const char *e = std::getenv("NSG_COLLECT_LOG")) {
+        char *end = nullptr;
+        log.size = std::max<int64_t>(std::strtoll(e, &end, 10), 1);
+        if (*end == ',') log.first_cap = std::atoi(end + 1);
+    }
+    if (buf.alloc((size_t)log.size + 1) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    log.keys = buf.p;
+    log.seen = reinterpret_cast<int *>(buf.p + log.size);
+}
+
 nsg_status collect_prune_all(const float *bp, int64_t n, int dp, const int *knn, int K, int nav, int L,
                              int R, int C, int *adj, int *deg, float *ms_collect, float *ms_prune,
                              int64_t *examined, const nsg::Exact8 &u8, cudaStream_t st) {
@@ -410,18 +436,9 @@ nsg_status collect_prune_all(const float *bp, int64_t n, int dp, const int *knn,
     DevBuf<int> cid, ccnt;
     DevBuf<float> cd2;
     DevBuf<unsigned long long> nexam;
-    // logs of the searches' keys; without that memory the collect lists are
-    // merged as they grow.  512 MiB: allocating and freeing costs 0.8 us per MiB,
-    // smaller logs leave more launches with a last wave (100,000 SIFT-shaped
-    // rows, whole build: 256 MiB 24.4, 512 24.4, 1,024 24.6, 2,048 25.4 ms)
-    const size_t log_budget = size_t(512) << 20;
-    DevBuf<uint64_t> log;
-    const int64_t log_cap = nsg::collect_log_cap(L, K, C);
-    int64_t log_nodes = log_cap ? std::min<int64_t>(chunk, (int64_t)(log_budget / (8 * log_cap))) : 0;
-    if (log_nodes && log.alloc((size_t)(log_nodes * log_cap)) != cudaSuccess) {
-        cudaGetLastError();
-        log_nodes = 0;
-    }
+    DevBuf<uint64_t> logbuf;
+    nsg::CollectLog log;
+    if (!collect_force("merge")) make_collect_log(L, K, chunk, logbuf, log);
     NSG_CK(cid.alloc((size_t)chunk * C));
     NSG_CK(cd2.alloc((size_t)chunk * C));
     NSG_CK(ccnt.alloc(chunk));
@@ -451,10 +468,8 @@ nsg_status collect_prune_all(const float *bp, int64_t n, int dp, const int *knn,
         c.cand_count = ccnt.p;
         c.status = nullptr;
         c.u8 = u8;
-        c.log = log.p;
-        c.log_nodes = log_nodes;
         cudaEventRecord(ev[0], st);
-        cudaError_t e = nsg::launch_collect(c, st);
+        cudaError_t e = log.keys ? nsg::run_collect_log(c, log, st) : nsg::launch_collect(c, st);
         if (e != cudaSuccess) rc = cuda_fail(e, "launch_collect");
         cudaEventRecord(ev[1], st);
         nsg::PruneLaunch p;
@@ -697,21 +712,11 @@ nsg_status nsg_collect(const float *base_dev, int64_t n, int32_t d, const int32_
     c.cand_d2 = cand_d2_dev;
     c.cand_count = cand_count_dev;
     c.status = status_dev;
-    // stream-ordered logs of 256 MiB at most, returned to the device once the
-    // call's work is done; refused, the call runs without
-    const int64_t log_cap = nsg::collect_log_cap(L, K, C);
-    void *log = nullptr;
-    if (log_cap) {
-        c.log_nodes = std::min<int64_t>(nv, (int64_t)((size_t(256) << 20) / (8 * log_cap)));
-        if (cudaMallocAsync(&log, (size_t)(8 * log_cap * c.log_nodes), st) != cudaSuccess) {
-            cudaGetLastError();
-            log = nullptr;
-        }
-        c.log = static_cast<uint64_t *>(log);
-    }
-    const cudaError_t e = nsg::launch_collect(c, st);
-    if (log) cudaFreeAsync(log, st);
-    NSG_CK(e);
+    DevBuf<uint64_t> buf;
+    nsg::CollectLog log;
+    if (!collect_force("merge")) make_collect_log(L, K, nv, buf, log);
+    NSG_CK(log.keys ? nsg::run_collect_log(c, log, st) : nsg::launch_collect(c, st));
+    if (log.keys) NSG_CK(cudaStreamSynchronize(st));  // the logs are freed on return
     return NSG_OK;
 }
 

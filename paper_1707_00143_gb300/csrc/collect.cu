@@ -15,6 +15,9 @@ struct CollectArgs {
     int *cand_count, *status;
     uint64_t *log;  // [nv][log_cap] measured keys, cand_count their numbers
     int log_cap;
+    int *seen;    // longest log (one that filled counts as twice what it holds), logs that filled
+    int sel_cap;  // keys the selection has room for: no log is longer
+    bool left;    // merged lists only for the nodes whose logs filled (cand_count -1)
 };
 
 // v's nearest neighbours in the kNN graph that its search has not seen (Alg.
@@ -37,10 +40,10 @@ __device__ __forceinline__ int knn_row_keys(const CollectArgs &a, const D &dist,
     return m;
 }
 
-// Search-and-collect with the collect list kept sorted as the search goes: the
-// general form, for searches that measure more keys than a log holds.
+// Search-and-collect with the collect list kept sorted as the search goes: for
+// searches that measure more keys than a log holds.
 template <int G, int V, int U>
-__global__ void __launch_bounds__(256) collect_kernel(CollectArgs a) {
+__device__ __forceinline__ void collect_body(const CollectArgs &a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const unsigned lane = lane_id();
@@ -48,6 +51,7 @@ __global__ void __launch_bounds__(256) collect_kernel(CollectArgs a) {
     const int64_t stride = (int64_t)gridDim.x * wpb;
     const uint32_t hmask = (uint32_t)a.H - 1;
     for (int64_t j = (int64_t)blockIdx.x * wpb + warp; j < a.nv; j += stride) {
+        if (a.left && a.cand_count[j] >= 0) continue;
         const int v = (int)(a.v0 + j);
         DistF32<G, V, U> dist{{}, a.rows.base4, a.rows.dp4};
         dist.Q.load_row(a.rows.base4 + (int64_t)v * a.rows.dp4, a.rows.dp4);
@@ -71,11 +75,29 @@ __global__ void __launch_bounds__(256) collect_kernel(CollectArgs a) {
     }
 }
 
+// 20 warps per SM by the lists' shared memory: rows of up to 512 values on 80
+// registers without spills (the compiler's own choice is 64 with some: 612 -> 705
+// ms for 1,000,000 uniform rows of 128 values, K = 100, L = 60), wider ones on
+// the compiler's own budget.
+template <int G, int V, int U>
+__global__ void __launch_bounds__(256, 3) collect_kernel(CollectArgs a) {
+    collect_body<G, V, U>(a);
+}
+template <int G, int V, int U>
+__global__ void __launch_bounds__(256) collect_wide_kernel(CollectArgs a) {
+    collect_body<G, V, U>(a);
+}
+template <int G, int V, int U>
+void (*collect_entry())(CollectArgs) {
+    if constexpr (V > 4) return collect_wide_kernel<G, V, U>;
+    else return collect_kernel<G, V, U>;
+}
+
 // Search-and-collect, first half: the keys are only appended to the node's log
 // in global memory.  Merging every expansion's keys into a sorted list of C in
 // shared memory was most of a search's instructions (moving up to C keys each
-// time) and its list a third of the shared memory: 20 warps per SM, 32 with
-// the log.  Both halves together, FP32 rows: 100,000 SIFT-shaped rows (K =
+// time) and its list a third of the shared memory: 20 warps per SM, 24 to 32
+// with the log.  Both halves together, FP32 rows: 100,000 SIFT-shaped rows (K =
 // 100, L = 40, C = 500) 18.6 -> 14.0 ms, 150,000 DEEP-shaped (64, 60, 500)
 // 7.2 -> 6.2 ms, 10,000 x 32 (20, 40, 200) 0.57 -> 0.41 ms.  Integer rows go
 // through their exact 8-bit copy, a quarter of the bytes gathered and of the
@@ -87,23 +109,30 @@ __device__ __forceinline__ void collect_log_body(const CollectArgs &a) {
     const unsigned lane = lane_id();
     WarpSmem s = carve_warp_smem(smem + warp * warp_smem_bytes(a.L, a.W, 0, a.H, true), a.L, a.W, 0, a.H, true);
     const int64_t stride = (int64_t)gridDim.x * wpb;
+    int longest = 0, filled = 0;
     for (int64_t j = (int64_t)blockIdx.x * wpb + warp; j < a.nv; j += stride) {
         const int v = (int)(a.v0 + j);
-        KeyLog lg{a.log + j * a.log_cap, a.log_cap, a.C, 0, ~0ull};
+        KeyLog lg{a.log + j * a.log_cap, a.log_cap, 0, false};
         bool capped = false;
         with_row_dist<G, V, U, U8>(a.rows, v, [&](const auto &dist) {
             int none = 0;
             capped = warp_alg1<KEYS_LOG>(dist, GraphRef{a.knn, a.K}, a.nav, a.L, s, (uint32_t)a.H - 1, a.hshift,
                                          a.max_steps, v, 0, none, nullptr, 0, nullptr, nullptr, nullptr, &lg)
                          .capped;
-            const int m = knn_row_keys(a, dist, s, v);
+            const int m = lg.full ? 0 : knn_row_keys(a, dist, s, v);
             if (m > 0) log_append(lg, s.keys, m, v);
         });
+        longest = max(longest, lg.full ? 2 * a.log_cap : lg.count);
+        filled += lg.full;
         if (lane == 0) {
-            a.cand_count[j] = lg.count;
+            a.cand_count[j] = lg.full ? -1 : lg.count;
             if (a.status) a.status[j] = capped ? -4 : 0;
         }
         __syncwarp();
+    }
+    if (lane == 0 && longest > 0) {
+        atomicMax(a.seen, longest);
+        if (filled) atomicAdd(a.seen + 1, filled);
     }
 }
 
@@ -124,16 +153,19 @@ void (*collect_log_entry(bool u8))(CollectArgs) {
 }
 
 // Search-and-collect, second half: one block per node cuts its log to the C
-// smallest distinct keys, sorted.  Duplicates (nodes the visited set forgot)
+// smallest distinct keys, sorted; nodes whose logs filled are left alone.  Duplicates (nodes the visited set forgot)
 // go through an exact hash of the ids; two 1024-bin passes over the distance
 // bits (their order is the distances' order) find a bound that lets through
-// the C smallest and hardly more; those are sorted in shared memory by the
-// network of log_compact.  Bound by the shared-memory passes of the hash and
+// the C smallest and hardly more; those are sorted in shared memory by a bitonic
+// network whose first step of each merge pairs mirrored positions, so that
+// every comparison puts the smaller key first and positions past the end need
+// no padding.  Bound by the shared-memory passes of the hash and
 // the sort; the log itself is read up to four times, from L2 after the first.
 // Each thread owns at most 32 log entries, whose
 // first-copy flags are one register.
 constexpr int SEL_BINS = 1024;
 constexpr int LOG_CAP_MAX = 16384;
+constexpr int LOG_LONG = 6400;  // run_collect_log
 
 template <int NT>
 struct SelectShared {
@@ -207,15 +239,16 @@ __global__ void __launch_bounds__(NT) collect_select_kernel(CollectArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ SelectShared<NT> sh;
     uint32_t *hash = reinterpret_cast<uint32_t *>(smem);  // then the keys to sort
-    uint64_t *keys = reinterpret_cast<uint64_t *>(smem);  // [log_cap]
+    uint64_t *keys = reinterpret_cast<uint64_t *>(smem);  // [sel_cap]
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t j = blockIdx.x;
     const uint64_t *log = a.log + j * a.log_cap;
     const int n = a.cand_count[j];
+    if (n < 0) return;
     // table of more than n slots: the largest power of two that the keys' space
-    // holds is more than log_cap
+    // holds is more than sel_cap
     int hb = 6;
-    while ((1 << hb) < 2 * n && (2 << hb) <= 2 * a.log_cap) ++hb;
+    while ((1 << hb) < 2 * n && (2 << hb) <= 2 * a.sel_cap) ++hb;
     const uint32_t hmask = (1u << hb) - 1;
     for (int i = t; i <= (int)hmask; i += NT) hash[i] = HASH_EMPTY;
     for (int i = t; i < SEL_BINS; i += NT) sh.hist[i] = 0;
@@ -294,20 +327,28 @@ __global__ void __launch_bounds__(NT) collect_select_kernel(CollectArgs a) {
     if (t == 0) a.cand_count[j] = cnt;
 }
 
-// Log entries per node.  A search of pool L expands little more than L nodes
-// and finds less than half of their K neighbours new (512 visited slots, most
-// of any node: 1,643 keys of L K = 4,000 on 100,000 SIFT-shaped rows, 288 of
-// 3,840 DEEP-shaped, 376 of 800 on 10,000 x 32); a log that fills all the same
-// is compacted in place, so it holds two lists and a row.
-// 0: such a log would pass the selection's limit, the lists are merged instead.
-int collect_log_cap(int L, int K, int C) {
-    const int64_t cap = std::max<int64_t>(std::max<int64_t>((int64_t)L * K / 2, 2 * (int64_t)C + K), 1024);
-    return cap <= LOG_CAP_MAX ? (int)((cap + 31) & ~31) : 0;
+// Whether logs are tried, and the keys a log is given before any was seen: a
+// search of pool L measured 0.03 to 2.1 times L K keys.
+static bool log_form(int L, int K) { return (int64_t)L * K <= 2 * LOG_CAP_MAX; }
+static int first_log_cap(int L, int K) {
+    return (int)std::min<int64_t>(std::max<int64_t>(3 * (int64_t)L * K, 1024), LOG_CAP_MAX);
+}
+// Nodes searched before the logs' length is known: a wave.
+static int64_t first_nodes() { return (int64_t)sm_count() * 32; }
+
+// The keys of a log for the search of nv nodes, 0: no log form.  512 MiB at
+// most: allocating and freeing costs 0.8 us per MiB.
+int64_t collect_log_keys(int L, int K, int64_t nv) {
+    if (!log_form(L, K) || nv < 1) return 0;
+    const int64_t budget = (int64_t)((size_t(512) << 20) / 8);
+    const int64_t first = std::min(nv, first_nodes()) * first_log_cap(L, K);
+    const int64_t rest = nv * std::max<int64_t>((int64_t)L * K / 2, 1024);
+    return std::min(budget, std::max(first, rest));
 }
 
 template <int NT>
 static cudaError_t launch_select_nt(const CollectArgs &a, cudaStream_t st) {
-    const size_t smem = 8 * (size_t)a.log_cap;
+    const size_t smem = 8 * (size_t)a.sel_cap;
     cudaError_t e = cudaFuncSetAttribute(collect_select_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
@@ -315,14 +356,18 @@ static cudaError_t launch_select_nt(const CollectArgs &a, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-static cudaError_t launch_select(const CollectArgs &a, cudaStream_t st) {
-    return a.log_cap <= 32 * 128   ? launch_select_nt<128>(a, st)
-           : a.log_cap <= 32 * 256 ? launch_select_nt<256>(a, st)
+// `longest`: of the logs.  The keys' space is also the hash table's: half of
+// the power of two that leaves the table at most 70 % full.
+static cudaError_t launch_select(CollectArgs a, int longest, cudaStream_t st) {
+    int half = 32;
+    while (2 * half * 7 < longest * 10) half *= 2;
+    a.sel_cap = std::min(std::max((longest + 31) & ~31, half), LOG_CAP_MAX);
+    return a.sel_cap <= 32 * 128   ? launch_select_nt<128>(a, st)
+           : a.sel_cap <= 32 * 256 ? launch_select_nt<256>(a, st)
                                    : launch_select_nt<512>(a, st);
 }
 
-cudaError_t launch_collect(const CollectLaunch &l, cudaStream_t st) {
-    if (l.nv <= 0) return cudaSuccess;
+static CollectArgs collect_args(const CollectLaunch &l) {
     CollectArgs a;
     a.rows = ExactRows{reinterpret_cast<const float4 *>(l.base), l.dp / 4, reinterpret_cast<const uint4 *>(l.u8.rows),
                        l.u8.chunks, l.u8.d, l.u8.lo};
@@ -341,41 +386,21 @@ cudaError_t launch_collect(const CollectLaunch &l, cudaStream_t st) {
     a.cand_d2 = l.cand_d2;
     a.cand_count = l.cand_count;
     a.status = l.status;
-    cudaError_t err = cudaSuccess;
-    a.log = l.log;
-    a.log_cap = collect_log_cap(l.L, l.K, l.C);
-    if (a.log != nullptr && a.log_cap > 0 && l.log_nodes > 0) {
-        // the visited set takes 1024 slots while 24 warps per SM still fit: the
-        // 512 that fit 32 warps beside rows of 100 neighbours measure 62 % more
-        // nodes (100,000 SIFT-shaped rows: 1,460 keys per node, collect 8.7 ms;
-        // 1024 slots 900 keys, 7.3 ms; 2048 on 20 warps 7.3, on 16 8.3 ms)
-        if (a.H < 1024 && 6 * (4 * warp_smem_bytes(a.L, a.W, 0, 1024, true) + 1024) <= smem_per_sm()) a.H = 1024;
-        a.hshift = 32 - log2i((unsigned)a.H);
-        const size_t per_warp = warp_smem_bytes(a.L, a.W, 0, a.H, true);
-        for (int64_t j0 = 0; j0 < l.nv && err == cudaSuccess; j0 += l.log_nodes) {
-            a.v0 = l.v0 + j0;
-            a.nv = std::min<int64_t>(l.log_nodes, l.nv - j0);
-            a.cand_ids = l.cand_ids + j0 * l.C;
-            a.cand_d2 = l.cand_d2 + j0 * l.C;
-            a.cand_count = l.cand_count + j0;
-            a.status = l.status != nullptr ? l.status + j0 : nullptr;
-            NSG_DISPATCH_DP4(a.rows.dp4, {
-                auto kern = collect_log_entry<G_, V_, U_>(a.rows.u8 != nullptr);
-                int grid, wpb;
-                size_t smem;
-                err = config(kern, per_warp, 4, a.nv, &grid, &wpb, &smem);
-                if (err == cudaSuccess) {
-                    kern<<<grid, wpb * 32, smem, st>>>(a);
-                    err = cudaGetLastError();
-                }
-            });
-            if (err == cudaSuccess) err = launch_select(a, st);
-        }
-        return err;
-    }
+    a.log = nullptr;
+    a.log_cap = a.sel_cap = 0;
+    a.seen = nullptr;
+    a.left = false;
+    return a;
+}
+
+static cudaError_t launch_merge(const CollectLaunch &l, bool left, cudaStream_t st) {
+    if (l.nv <= 0) return cudaSuccess;
+    CollectArgs a = collect_args(l);
+    a.left = left;
     const size_t per_warp = warp_smem_bytes(a.L, a.W, a.C, a.H);
+    cudaError_t err = cudaSuccess;
     NSG_DISPATCH_DP4(a.rows.dp4, {
-        auto kern = collect_kernel<G_, V_, U_>;
+        auto kern = collect_entry<G_, V_, U_>();
         int grid, wpb;
         size_t smem;
         err = config(kern, per_warp, 4, l.nv, &grid, &wpb, &smem);
@@ -384,6 +409,86 @@ cudaError_t launch_collect(const CollectLaunch &l, cudaStream_t st) {
             err = cudaGetLastError();
         }
     });
+    return err;
+}
+
+cudaError_t launch_collect(const CollectLaunch &l, cudaStream_t st) { return launch_merge(l, false, st); }
+
+// The nodes j0 .. j0 + nv - 1 of a launch.
+static CollectLaunch part_of(const CollectLaunch &l, int64_t j0, int64_t nv) {
+    CollectLaunch p = l;
+    p.v0 = l.v0 + j0;
+    p.nv = nv;
+    p.cand_ids = l.cand_ids + j0 * l.C;
+    p.cand_d2 = l.cand_d2 + j0 * l.C;
+    p.cand_count = l.cand_count + j0;
+    p.status = l.status != nullptr ? l.status + j0 : nullptr;
+    return p;
+}
+
+// How many keys a search measures depends on the rows and their number (0.04 L K
+// for 100,000 DEEP-shaped rows, K = 64, L = 60, 0.24 for a million; 0.26 and
+// 0.73 for as many SIFT-shaped, 100 and 40; 1.2 for uniform ones) and hardly on
+// the node.  So every slice of nodes is given logs by the longest of the slice
+// before it (a quarter more), the first, a part of a wave, long ones; and the
+// selection gets the shared memory that the slice's longest log needs.  The
+// host reads that number between the two: ~15 us a slice.  A node whose log
+// fills is searched again with a merged list.  What a log costs grows with every
+// key, a merged list's cost only with the keys that enter: FP32 searches that
+// pass LOG_LONG keys are merged (uniform rows of 128 values, K = 100, L = 60,
+// 1,000,000: 1,105 ms logged, 612 merged; 30,000, 6,600 keys: equal), 8-bit ones
+// as long as logs hold them are not (300,000 such rows: 103 ms logged, 156
+// merged on FP32 rows).  Merged lists alone -> logs: 1,000,000 SIFT-shaped rows
+// 295 -> 138 ms, 10,000,000 DEEP-shaped 2,614 -> 2,040 (with logs of L K / 2 that
+// were compacted when full: 293 and 3,220).
+cudaError_t run_collect_log(const CollectLaunch &l, CollectLog &log, cudaStream_t st) {
+    CollectArgs a = collect_args(l);
+    a.log = log.keys;
+    a.seen = log.seen;
+    // the visited set takes 1024 slots while 24 warps per SM still fit: the
+    // 512 that fit 32 warps beside rows of 100 neighbours measure 62 % more
+    // nodes (100,000 SIFT-shaped rows: 1,460 keys per node, collect 8.7 ms;
+    // 1024 slots 900 keys, 7.3 ms; 2048 on 20 warps 7.3, on 16 8.3 ms; a
+    // million: 256, 174 and 162 ms; 10 million DEEP-shaped 2,810 and 2,160)
+    if (a.H < 1024 && 6 * (4 * warp_smem_bytes(a.L, a.W, 0, 1024, true) + 1024) <= smem_per_sm()) a.H = 1024;
+    a.hshift = 32 - log2i((unsigned)a.H);
+    const size_t per_warp = warp_smem_bytes(a.L, a.W, 0, a.H, true);
+    cudaError_t err = cudaSuccess;
+    for (int64_t j0 = 0; j0 < l.nv;) {
+        a.log_cap = log.cap > 0 ? log.cap : log.first_cap > 0 ? log.first_cap : first_log_cap(l.L, l.K);
+        a.log_cap = std::min(a.log_cap, LOG_CAP_MAX);
+        int64_t nodes = std::min(l.nv - j0, log.size / a.log_cap);
+        if (log.cap == 0) nodes = std::min(nodes, first_nodes());
+        if (log.merge || nodes < 1) return launch_merge(part_of(l, j0, l.nv - j0), false, st);
+        const CollectLaunch slice = part_of(l, j0, nodes);
+        a.v0 = slice.v0;
+        a.nv = slice.nv;
+        a.cand_ids = slice.cand_ids;
+        a.cand_d2 = slice.cand_d2;
+        a.cand_count = slice.cand_count;
+        a.status = slice.status;
+        if ((err = cudaMemsetAsync(a.seen, 0, 2 * sizeof(int), st)) != cudaSuccess) return err;
+        NSG_DISPATCH_DP4(a.rows.dp4, {
+            auto kern = collect_log_entry<G_, V_, U_>(a.rows.u8 != nullptr);
+            int grid, wpb;
+            size_t smem;
+            err = config(kern, per_warp, 4, a.nv, &grid, &wpb, &smem);
+            if (err == cudaSuccess) {
+                kern<<<grid, wpb * 32, smem, st>>>(a);
+                err = cudaGetLastError();
+            }
+        });
+        int seen[2] = {0, 0};
+        if (err == cudaSuccess) err = cudaMemcpyAsync(seen, a.seen, sizeof(seen), cudaMemcpyDeviceToHost, st);
+        if (err == cudaSuccess) err = cudaStreamSynchronize(st);
+        if (err == cudaSuccess) err = launch_select(a, std::min(seen[0], a.log_cap), st);
+        if (err == cudaSuccess && seen[1] > 0) err = launch_merge(slice, true, st);
+        if (err != cudaSuccess) return err;
+        log.merge = (seen[1] == 0 || a.log_cap == LOG_CAP_MAX) &&
+                    seen[0] > (a.rows.u8 != nullptr ? LOG_CAP_MAX : LOG_LONG);
+        log.cap = std::min(std::max((seen[0] + seen[0] / 4 + l.K + 31) & ~31, 1024), LOG_CAP_MAX);
+        j0 += nodes;
+    }
     return err;
 }
 

@@ -190,13 +190,21 @@ struct CollectLaunch {
     int *cand_count;
     int *status;
     Exact8 u8;  // used by the log form
-    // logs of collect_log_cap keys for log_nodes nodes at a time (nullptr: the
-    // kernel that keeps sorted lists)
-    uint64_t *log = nullptr;
-    int64_t log_nodes = 0;
 };
-int collect_log_cap(int L, int K, int C);  // keys per node, 0: no log form
+// Sorted lists kept as the searches go.
 cudaError_t launch_collect(const CollectLaunch &a, cudaStream_t st);
+// The same through logs of all measured keys, on exact 8-bit rows where there
+// are some.  Synchronises the stream.
+struct CollectLog {
+    uint64_t *keys = nullptr;  // [size]
+    int64_t size = 0;
+    int *seen = nullptr;  // device, 2 ints
+    int first_cap = 0;    // keys per node of the first slice (0: the library's choice)
+    int cap = 0;          // keys per node of the next one, from the logs so far
+    bool merge = false;   // the searches are too long for logs
+};
+int64_t collect_log_keys(int L, int K, int64_t nv);  // keys for nv nodes, 0: no log form
+cudaError_t run_collect_log(const CollectLaunch &a, CollectLog &log, cudaStream_t st);
 
 // MRNG edge selection for nodes v0..v0+nv-1.
 struct PruneLaunch {

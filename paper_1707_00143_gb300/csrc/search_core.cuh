@@ -173,69 +173,26 @@ __device__ __forceinline__ void collect_merge(WarpSmem &s, int m, int excl, int 
 }
 
 // Every measured key of a node's search, appended in global memory and cut to
-// the C smallest by collect_select_kernel (collect.cu).
+// the C smallest by collect_select_kernel (collect.cu).  A search whose keys do
+// not fit ends there.
 struct KeyLog {
-    uint64_t *keys;  // [cap], cap >= 2 C + the graph's width
-    int cap, C;
+    uint64_t *keys;  // [cap]
+    int cap;
     int count;
-    uint64_t thr;  // keys from here on are not among the C smallest
+    bool full;
 };
-
-// What a full log keeps: its C smallest distinct keys, sorted by a bitonic
-// network whose first step of each merge pairs mirrored positions, so that
-// every comparison puts the smaller key first and positions past the end need
-// no padding.  Out of line: the host sizes the log so that it rarely fills.
-static __device__ __noinline__ int log_compact(uint64_t *a, int n, int C) {
-    const unsigned lane = lane_id();
-    __syncwarp();
-    for (int k = 2; k < 2 * n; k <<= 1) {
-        for (int h = k >> 1; h > 0; h >>= 1) {
-            const bool flip = h == k >> 1;
-            for (int p = lane; ; p += 32) {
-                const int blk = p / h, t = p - blk * h, i = blk * 2 * h + t;
-                if (i >= n) break;
-                const int j = flip ? blk * 2 * h + 2 * h - 1 - t : i + h;
-                if (j < n) {
-                    const uint64_t x = a[i], y = a[j];
-                    if (y < x) {
-                        a[i] = y;
-                        a[j] = x;
-                    }
-                }
-            }
-            __syncwarp();
-        }
-    }
-    int kept = 0;
-    uint64_t before = 0;  // the key just below this chunk
-    for (int b = 0; b < n && kept < C; b += 32) {
-        const int j = b + (int)lane;
-        const uint64_t k = j < n ? a[j] : 0;
-        uint64_t prev = __shfl_up_sync(NSG_FULL, k, 1);
-        if (lane == 0) prev = before;
-        const bool keep = j < n && (j == 0 || k != prev);
-        before = __shfl_sync(NSG_FULL, k, 31);
-        const unsigned bal = __ballot_sync(NSG_FULL, keep);
-        const int o = kept + __popc(bal & lanemask_lt());
-        __syncwarp();
-        if (keep && o < C) a[o] = k;
-        kept += __popc(bal);
-        __syncwarp();
-    }
-    return min(kept, C);
-}
 
 // Appends keys[0..m) minus id `excl` to the log.  Warp-wide.
 __device__ __forceinline__ void log_append(KeyLog &lg, const uint64_t *keys, int m, int excl) {
     if (lg.count + m > lg.cap) {
-        lg.count = log_compact(lg.keys, lg.count, lg.C);
-        if (lg.count == lg.C) lg.thr = lg.keys[lg.C - 1];
+        lg.full = true;
+        return;
     }
     const unsigned lane = lane_id();
     for (int b = 0; b < m; b += 32) {
         const int j = b + (int)lane;
         const uint64_t k = j < m ? keys[j] : ~0ull;
-        const bool keep = j < m && k < lg.thr && kid(k) != excl;
+        const bool keep = j < m && kid(k) != excl;
         const unsigned bal = __ballot_sync(NSG_FULL, keep);
         if (keep) lg.keys[lg.count + __popc(bal & lanemask_lt())] = k;
         lg.count += __popc(bal);
@@ -632,7 +589,10 @@ __device__ SearchOut warp_alg1(const D &dist, const Gr g, int start, int L, Warp
         dist(s.ids, m, s.keys);
         o.n_dist += m;
         if (COLLECT == KEYS_MERGE) collect_merge(s, m, excl, C, csize);
-        if (COLLECT == KEYS_LOG) log_append(*klog, s.keys, m, excl);
+        if (COLLECT == KEYS_LOG) {
+            log_append(*klog, s.keys, m, excl);
+            if (klog->full) break;
+        }
         if constexpr (PIPE != 0) {
             const uint64_t nx = predict_next(s.pool, o.size, L, i, s.keys, m);
             if (nx != ~0ull && o.n_expand < max_steps) {
