@@ -2,7 +2,9 @@
 fill, slices of a few nodes, searches longer than any log (merged lists take over), against the lists that
 are merged as the searches go, bit for bit.  And logs are not slower than those lists where searches
 measure most of what they meet (uniform rows: ~0.6 L K keys each; logs of half L K filled twice and took 2.2 times
-as long)."""
+as long).  The call for some nodes only keeps to the lists: it would pay for the logs each time."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -47,3 +49,25 @@ def test_build_log_no_slower_than_merged_lists(nsg, monkeypatch):
         return min(nsg.nsg_build(base, 100, 60, 50, 500).info()["ms_collect"] for _ in range(4))
 
     assert ms("log") < 1.15 * ms("merge")
+
+
+def test_collect_call_pays_for_no_logs(nsg, monkeypatch):
+    rng = np.random.default_rng(5)
+    base = torch.from_numpy(rng.standard_normal((20000, 96)).astype(np.float32)).cuda()
+    blocks = rng.integers(0, 25, (20000, 20)) + np.arange(20000)[:, None] // 25 * 25  # short searches
+    knn = torch.from_numpy(blocks.astype(np.int32)).cuda()
+
+    def seconds(engine):
+        if engine:
+            monkeypatch.setenv("NSG_COLLECT_ENGINE", engine)
+        best = 1e9
+        for _ in range(8):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            nsg.nsg_collect(base, knn, 17, 500, 500, v0=0, nv=5000)
+            torch.cuda.synchronize()
+            best = min(best, time.perf_counter() - t0)
+        return best
+
+    default = seconds("")
+    assert default < 1.3 * seconds("merge")
