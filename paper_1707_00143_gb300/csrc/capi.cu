@@ -30,7 +30,7 @@ struct nsg_index {
     int *flag = nullptr;    // [4] device scratch for nsg_search's cap check
     // work counters of the search launches (warps draw queries from one),
     // used round-robin so concurrent calls on other streams take other slots
-    int *work = nullptr;    // [kWorkSlots]
+    int *work = nullptr;    // [kWorkSlots][WORK_INTS]
     mutable std::atomic<unsigned> work_next{0};
     // low-precision copies, indexed by nsg_precision (1 = BF16, 2 = FP8-e4m3, 3 = U8)
     void *lowp[4] = {nullptr, nullptr, nullptr, nullptr};  // by nsg_precision
@@ -527,7 +527,7 @@ nsg_status finish_index_body(nsg_index *ix, cudaStream_t st) {
     ix->max_degree = mx;
     ix->avg_degree = ix->n ? (double)sum / (double)ix->n : 0.0;
     NSG_CK(cudaMalloc(reinterpret_cast<void **>(&ix->flag), 4 * sizeof(int)));
-    NSG_CK(cudaMalloc(reinterpret_cast<void **>(&ix->work), kWorkSlots * sizeof(int)));
+    NSG_CK(cudaMalloc(reinterpret_cast<void **>(&ix->work), kWorkSlots * nsg::WORK_INTS * sizeof(int)));
     return NSG_OK;
 }
 
@@ -1238,8 +1238,8 @@ cudaMemPool_t scratch_pool() {
 
 nsg_status launch_dynamic(const nsg_index *idx, nsg::SearchLaunch l, cudaStream_t st) {
     if (nsg_status s = ensure_gpool(idx, l, st)) return s;
-    int *ctr = idx->work + (idx->work_next.fetch_add(1, std::memory_order_relaxed) % kWorkSlots);
-    NSG_CK(cudaMemsetAsync(ctr, 0, sizeof(int), st));
+    int *ctr = idx->work + (idx->work_next.fetch_add(1, std::memory_order_relaxed) % kWorkSlots) * nsg::WORK_INTS;
+    NSG_CK(cudaMemsetAsync(ctr, 0, nsg::WORK_INTS * sizeof(int), st));
     l.work = ctr;
     // queries farthest from the navigating node drawn first (the launch's tail
     // is then made of short searches) when the batch has more warps' worth of
@@ -1381,7 +1381,7 @@ nsg_status nsg_search_host(const nsg_index *idx, const float *queries_host, int6
 struct nsg_plan {
     nsg::SearchLaunch l;
     int *order = nullptr;  // visiting order (longest pool first)
-    int *work = nullptr;   // device work counter
+    int *work = nullptr;   // device work counters
     uint64_t *gpool = nullptr;  // global-memory pool slots (the graph keeps the address)
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -1416,7 +1416,7 @@ nsg_status batched_setup_body(const nsg_index *idx, const float *queries_dev, in
     for (int64_t i = 0; i < nq; ++i) ord[i] = (int)i;
     std::stable_sort(ord.begin(), ord.end(), [&](int a, int b) { return hL[a] > hL[b]; });
     NSG_CK(order.alloc((size_t)nq));
-    NSG_CK(work.alloc(1));
+    NSG_CK(work.alloc(nsg::WORK_INTS));
     NSG_CK(cudaMemcpyAsync(order.p, ord.data(), sizeof(int) * nq, cudaMemcpyHostToDevice, st));
     NSG_CK(cudaStreamSynchronize(st));
     l.kv = k_dev;
@@ -1437,7 +1437,7 @@ nsg_status batched_setup(const nsg_index *idx, const float *queries_dev, int64_t
 }
 
 nsg_status batched_run(const nsg::SearchLaunch &l, cudaStream_t st) {
-    NSG_CK(cudaMemsetAsync(l.work, 0, sizeof(int), st));
+    NSG_CK(cudaMemsetAsync(l.work, 0, nsg::WORK_INTS * sizeof(int), st));
     NSG_CK(nsg::launch_search(l, st));
     return NSG_OK;
 }

@@ -16,6 +16,9 @@ constexpr int MAX_DP4_HOST = 512;  // largest supported row: 2048 floats
 inline int default_steps(int L) { return 16 * L + 4096; }
 
 // Search on a fixed-width graph (Alg. 1 from `start`), one warp per query.
+// SearchLaunch::work: queries drawn; on integer rows also whether one of them
+// needs the FP32 rows (search_int8.cu).
+constexpr int WORK_LEFT = 1, WORK_INTS = 2;
 struct SearchLaunch {
     const float *base;  // [n][dp] padded, 16-byte aligned
     int64_t n;
@@ -49,7 +52,7 @@ struct SearchLaunch {
     unsigned char *trace_flag = nullptr;   // [nq][trace_cap]
     int trace_cap = 0;
     // batched uneven queries: per-query k / L (k, L are then the maxima),
-    // visiting order, device work counter (reset before each launch)
+    // visiting order, device work counters [WORK_INTS] (zeroed before each launch)
     const int *kv = nullptr, *Lv = nullptr, *order = nullptr;
     int *work = nullptr;
     // random initial pool of init_count seeded draws (0: start at `start`)

@@ -17,9 +17,19 @@
 
 namespace nsg {
 
-// PREC_F32_INT8 (inside the library): the plain form on integer rows, whose
-// FP32 keys come from the exact 8-bit copy for every query that it holds too.
-enum { PREC_F32 = 0, PREC_BF16 = 1, PREC_FP8 = 2, PREC_U8 = 3, PREC_F32_INT8 = 4 };
+// Inside the library, the plain form on integer rows, whose FP32 keys come from
+// the exact 8-bit copy for queries that it holds too: PREC_F32_EITHER looks at
+// every query, PREC_F32_INT8 takes batches that it holds throughout,
+// PREC_F32_REST the others, on the FP32 rows.
+enum {
+    PREC_F32 = 0,
+    PREC_BF16 = 1,
+    PREC_FP8 = 2,
+    PREC_U8 = 3,
+    PREC_F32_EITHER = 4,
+    PREC_F32_INT8 = 5,
+    PREC_F32_REST = 6
+};
 
 // ---------------------------------------------------------------------------
 // 8-bit integer form: x_u8 = clamp(rint((x - lo) * s), 0, 255), the query

@@ -45,6 +45,7 @@ cudaError_t launch_search(const SearchLaunch &l, cudaStream_t st) {
     a.Lv = l.Lv;
     a.order = l.order;
     a.work = l.work;
+    a.left = nullptr;
     a.init_count = l.init_count;
     a.init_seed = l.init_seed;
     a.n = (int)l.n;
@@ -72,7 +73,7 @@ cudaError_t launch_search(const SearchLaunch &l, cudaStream_t st) {
         return a.gpool != nullptr ? launch_search_staged_global(a, l, pw, wpq, st)
                                   : launch_search_staged(a, l, pw, wpq, st);
     }
-    if (l.exact8 && !stop && l.precision == PREC_F32) return launch_search_int8(a, l, per_warp, wpq, st);
+    if (l.exact8 && l.work != nullptr && !stop && l.precision == PREC_F32) return launch_search_int8(a, l, per_warp, wpq, st);
     if (a.gpool != nullptr) return launch_search_global(a, l, per_warp, per_cta, stop, wpq, st);
     return launch_search_args<false>(a, l, per_warp, per_cta, stop, wpq, st);
 }

@@ -81,6 +81,7 @@ struct SearchArgs {
     // persistent warps draw from (nullptr: static grid-stride assignment)
     const int *kv, *Lv, *order;
     int *work;
+    const int *left;  // integer rows: whether a query of the batch needs the FP32 rows
     // random initial pool (count 0: start at `start`), base rows n
     int init_count;
     uint64_t init_seed;
@@ -126,12 +127,18 @@ __device__ __forceinline__ void run_dist(const D &dist, const StageRef *sr, cons
 // sizes it for at least one traversal row).
 template <int G, int V, int U, int P, bool ST = false, class F>
 __device__ __forceinline__ bool with_dist(const SearchArgs &a, const float *qp, const StageRef *sr, F &&f) {
-    if constexpr (P == PREC_F32) {
+    if constexpr (P == PREC_F32 || P == PREC_F32_REST) {
         DistF32<G, V, U> dist{{}, a.base4, a.dp4};
         dist.Q.load(qp, a.d, a.dp4);
         run_dist<ST>(dist, sr, nullptr, f);
         return true;
     } else if constexpr (P == PREC_F32_INT8) {
+        using S = Exact8Shape<G, V>;
+        DistU8<S::lanes, S::chunks, NSG_U8ROWS> dist{{}, a.lowp, a.dc};
+        dist.Q.load(qp, a.d, a.lo, 1.0f);
+        f(dist);
+        return true;
+    } else if constexpr (P == PREC_F32_EITHER) {
         using S = Exact8Shape<G, V>;
         DistU8<S::lanes, S::chunks, NSG_U8ROWS> d8{{}, a.lowp, a.dc};
         // integers that the copy's map keeps: their distances are exact in both forms
@@ -186,7 +193,7 @@ __device__ __forceinline__ void finish_query(const SearchArgs &a, WarpSmem &s, c
     const unsigned lane = lane_id();
     const uint64_t *res = s.pool;
     int rsize = o.size;
-    if constexpr (P != PREC_F32 && P != PREC_F32_INT8) if (rerank) {
+    if constexpr (P == PREC_BF16 || P == PREC_FP8 || P == PREC_U8) if (rerank) {
         uint64_t *cl = a.C > 0 ? s.clist : reinterpret_cast<uint64_t *>(s.hash);
         // the re-rank gathers all L pool rows at once: more rows in flight
         // than the traversal for rows of 513..1024 values
@@ -255,6 +262,8 @@ __device__ __forceinline__ void search_body(const SearchArgs &a) {
         for (int t = threadIdx.x; t < NSG_STOP_PARAMS; t += blockDim.x) dst[t] = __half2float(a.stop_model[t]);
         __syncthreads();
     }
+    if constexpr (P == PREC_F32_INT8 || P == PREC_F32_REST)
+        if ((*a.left == 0) != (P == PREC_F32_INT8)) return;  // the other kernel's batch
     int csize = 0;
     const int64_t stride = (int64_t)gridDim.x * wpb;
     int64_t t = (int64_t)blockIdx.x * wpb + warp;
@@ -318,6 +327,8 @@ __device__ __forceinline__ void search_group_body(const SearchArgs &a) {
         sref = stage_init(smem + off + warp * stage_bytes(a.stage_nb, a.stage_rb), a.stage_nb, a.stage_rb,
                           a.any_capped);
     }
+    if constexpr (P == PREC_F32_INT8 || P == PREC_F32_REST)
+        if ((*a.left == 0) != (P == PREC_F32_INT8)) return;  // the other kernel's batch
     const int bar_id = 1 + g;
     const int64_t stride = (int64_t)gridDim.x * gpb;
     int64_t tstat = (int64_t)blockIdx.x * gpb + g;
@@ -404,13 +415,13 @@ static void (*search_entry(bool stop, int wpq))(SearchArgs) {
 }
 
 // The plain form on integer rows with an exact 8-bit copy (rows of up to 258
-// values, no stop model).
-template <int G, int V, int U, bool GP>
+// values, no stop model): P is one of its three precisions.
+template <int G, int V, int U, int P, bool GP>
 static void (*int8_entry(int wpq))(SearchArgs) {
     if constexpr (V <= 4) {
-        if (wpq == 2) return search_group_kernel<G, V, U, PREC_F32_INT8, 2, GP>;
-        if (wpq == 4) return search_group_kernel<G, V, U, PREC_F32_INT8, 4, GP>;
-        return search_kernel<G, V, U, PREC_F32_INT8, GP>;
+        if (wpq == 2) return search_group_kernel<G, V, U, P, 2, GP>;
+        if (wpq == 4) return search_group_kernel<G, V, U, P, 4, GP>;
+        return search_kernel<G, V, U, P, GP>;
     } else {
         return nullptr;
     }
@@ -449,15 +460,16 @@ static cudaError_t config(K kernel, size_t smem_per_warp, int want_wpb, int64_t 
 // Launch of the search kernels for the launch description `a`: pools in
 // shared memory (GP false) or in the global slots a.gpool (GP true, at most
 // gpool_slots resident warps or groups); ST: the staged-gather kernels (rows
-// of more than 512 values, no stop model); INT8: the plain form on integer rows.
-template <bool GP, bool ST = false, bool INT8 = false>
+// of more than 512 values, no stop model); INT8: its precision in the plain form on
+// integer rows.
+template <bool GP, bool ST = false, int INT8 = 0>
 cudaError_t launch_search_args(const SearchArgs &a, const SearchLaunch &l, size_t per_warp, size_t per_cta,
                                bool stop, int wpq, cudaStream_t st) {
     cudaError_t err = cudaSuccess;
     NSG_DISPATCH_DP4(a.dp4, {
         void (*kern)(SearchArgs) = nullptr;
-        if constexpr (INT8) {
-            kern = int8_entry<G_, V_, U_, GP>(wpq);
+        if constexpr (INT8 != 0) {
+            kern = int8_entry<G_, V_, U_, INT8, GP>(wpq);
         } else if constexpr (ST) {
             if constexpr (V_ >= 8)
                 if (!stop)
