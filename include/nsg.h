@@ -164,7 +164,8 @@ const char *nsg_last_cuda_error(void);
  *   base_dev [n][d] f32; knn_ids_dev [n][K] i32 out; knn_d2_dev [n][K] f32 out
  *   (nullable).  Requires 1 <= K < n, d >= 1.  Uses tensor cores where the
  *   data allows an exact answer, else an exact FP32 scan.  Allocates scratch.
- *   Environment: NSG_KNN_ENGINE=scan forces the FP32 scan;
+ *   Environment: NSG_KNN_ENGINE=scan forces the FP32 scan, =units or =small
+ *   one of the two tensor-core kernels (the sizes choose otherwise);
  *   NSG_KNN_CHUNK_TILES=t sets the tensor-core form's base chunk (t tiles of
  *   128 rows per launch; default ~48 MB of BF16 rows); the chunk size does
  *   not change results.

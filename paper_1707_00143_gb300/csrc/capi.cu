@@ -81,7 +81,8 @@ namespace {
 
 thread_local char g_err[512] = "";
 // kNN engine: tensor cores when the answer is exact, else the CUDA-core scan;
-// NSG_KNN_ENGINE=scan forces the CUDA-core scan (read at every call).
+// NSG_KNN_ENGINE=scan forces the CUDA-core scan, =units and =small one of the
+// tensor-core kernels where they apply (read at every call).
 bool knn_force_scan() {
     const char *e = std::getenv("NSG_KNN_ENGINE");
     return e && std::strcmp(e, "scan") == 0;
@@ -252,27 +253,6 @@ nsg_status padded_view(const float *src, int64_t n, int d, DevBuf<float> &tmp, c
     return s;
 }
 
-// Few base tiles: the kernel whose scanning warps merge themselves
-// (knn_tc_small.cu).  knn_tc.cu's pre-pass needs ~320 base rows per list entry;
-// without it nearly every column of a short base is a candidate, and the row
-// units' merges (256 rows a unit, split when they are few) take longer than one
-// CTA per 128 rows, but for few queries or a grid that fills the SMs about once.
-// With it the lines are those where launches and splits stop paying.  The
-// entries counted are those of data that needs a re-rank (k and its margin),
-// which is known only later.  Large kernel's speed over the small one's: 6,000
-// x 96 floats, 8,000 queries, k = 1 0.64; 12,000 x 96, k = 10, 1,500 queries 0.84,
-// 8,000 0.71, 40 1.05; 30,000 x 96, k = 100, 8,000 queries 0.73, 300 1.4; kNN graph
-// of 18,000 x 96, K = 100 0.58, of 26,000 1.13, 40,000 0.64, 60,000 2.1; with the
-// pre-pass (integer rows) 8,000 x 128, k = 10, one query 0.72, 1,500 1.2, 10,000
-// 0.91; 18,000 x 128, K = 20 graph 0.92, 26,000 1.8.
-bool knn_small(int64_t n, int64_t nq, int k) {
-    if (n < 8448) return true;
-    const int64_t units = (nq + 255) / 256, sms = nsg::sm_count();
-    const int64_t entries = k + (k / 2 > 32 ? k / 2 : 32);
-    if (n < 320 * entries) return nq > 1024 && !(n >= 20480 && units > sms / 2 && units <= sms);
-    return (n < 16384 && nq > 4096) || (n < 20480 && nq > 12288) || (n < 10240 && nq <= 32);
-}
-
 nsg_status knn_run(const float *bp, int64_t n, int dp, const float *qp, int64_t nq, int64_t q0, int k,
                    int self_join, int *ids, float *d2, cudaStream_t st) {
     nsg::KnnLaunch l;
@@ -287,10 +267,7 @@ nsg_status knn_run(const float *bp, int64_t n, int dp, const float *qp, int64_t 
     l.ids = ids;
     l.d2 = d2;
     int used = 0;
-    if (!knn_force_scan()) {
-        if (knn_small(n, nq, k)) NSG_CK(nsg::launch_knn_tc_small(l, &used, st));
-        else NSG_CK(nsg::launch_knn_tc(l, &used, st));
-    }
+    if (!knn_force_scan()) NSG_CK(nsg::launch_knn_tc(l, &used, st));
     if (!used) NSG_CK(nsg::launch_knn_direct(l, st));
     return NSG_OK;
 }

@@ -279,7 +279,6 @@ cudaError_t launch_knn_direct(const KnnLaunch &a, cudaStream_t st);
 // answer (integer values 0..255, d <= 128, k <= 256): *used = 1 when it ran,
 // 0 when it does not apply (nothing written).  Synchronises the stream.
 cudaError_t launch_knn_tc(const KnnLaunch &a, int *used, cudaStream_t st);
-cudaError_t launch_knn_tc_small(const KnnLaunch &a, int *used, cudaStream_t st);  // few base tiles (knn_tc_small.cu)
 
 // Exact FP32 re-rank: for query i, the k smallest (d2, id) among the KL
 // candidate ids cand[i][..] (-1 = none) into a.ids / a.d2.

@@ -47,13 +47,15 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
+#include <cstring>
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
 #include "common.cuh"
-#include "kernels.h"
+#include "knn_rule.h"
+#include "knn_tc.cuh"
 #include "tc_ptx.cuh"
 
 namespace nsg {
@@ -862,28 +864,19 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
-// 2-D tensor map over a [rows][dk] bf16 matrix, box = 64 (K) x box_rows, 128B swizzle.
-bool make_map(CUtensorMap *map, const void *ptr, int64_t rows, int dk, int box_rows) {
+// 2-D tensor map over a [rows][dk] bf16 matrix, box = 64 (K) x 128 rows, 128B swizzle.
+bool make_map(CUtensorMap *map, const void *ptr, int64_t rows, int dk) {
     auto fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {(cuuint64_t)dk, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)dk * 2};
-    cuuint32_t box[2] = {(cuuint32_t)TC_BOXK, (cuuint32_t)box_rows};
+    cuuint32_t box[2] = {(cuuint32_t)TC_BOXK, (cuuint32_t)TC_N};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
-
-template <typename T>
-struct Scratch {
-    T *p = nullptr;
-    ~Scratch() {
-        if (p) cudaFree(p);
-    }
-    cudaError_t alloc(size_t n) { return cudaMalloc(reinterpret_cast<void **>(&p), n * sizeof(T) + 16); }
-};
 
 // Work split of one selection over `ntiles` base tiles: as few splits as
 // finish the (row unit, split) pairs in about the least number of waves; a
@@ -923,89 +916,34 @@ cudaError_t launch_tc(int dk, const CUtensorMap &mA, const CUtensorMap &mB, cons
 
 }  // namespace
 
-// Tensor-core kNN when the data allows an exact answer (integer 0..255,
-// d <= 128, k <= 256); *used = 0 when it does not apply (nothing written).
-cudaError_t launch_knn_tc(const KnnLaunch &l, int *used, cudaStream_t st) {
-    *used = 0;
-    if (l.nq <= 0 || l.k > TC_MAXK || l.dp > 1024 || !encode_fn()) return cudaSuccess;
-    const int dk = l.dp <= 64 ? 64 : (l.dp <= 128 ? 128 : (l.dp + 63) / 64 * 64);
-    const int64_t ntiles = (l.n + TC_N - 1) / TC_N;
-    if (ntiles > INT32_MAX / TC_N) return cudaSuccess;
-    const int64_t npad = ntiles * TC_N;
-    Scratch<__nv_bfloat16> xb, qb;
-    Scratch<float> xn, qn;
-    Scratch<int> flag;
-    cudaError_t e;
-    if ((e = xb.alloc((size_t)l.n * dk)) != cudaSuccess) return e;
-    if ((e = xn.alloc((size_t)npad)) != cudaSuccess) return e;
-    if ((e = flag.alloc(2)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(flag.p, 0, 2 * sizeof(int), st)) != cudaSuccess) return e;
-    const int grid_rows = sm_count() * 8;
-    bf16_rows_kernel<<<grid_rows, 256, 0, st>>>(reinterpret_cast<const float4 *>(l.base), l.n, l.dp / 4,
-                                                reinterpret_cast<uint2 *>(xb.p), dk / 4, xn.p, npad, flag.p);
-    const __nv_bfloat16 *qsrc = xb.p + (l.self_join ? l.q0 * dk : 0);
-    const float *qnorm = xn.p + (l.self_join ? l.q0 : 0);
-    if (!l.self_join) {
-        if ((e = qb.alloc((size_t)l.nq * dk)) != cudaSuccess) return e;
-        if ((e = qn.alloc((size_t)l.nq)) != cudaSuccess) return e;
-        bf16_rows_kernel<<<grid_rows, 256, 0, st>>>(reinterpret_cast<const float4 *>(l.queries), l.nq, l.dp / 4,
-                                                    reinterpret_cast<uint2 *>(qb.p), dk / 4, qn.p, l.nq, flag.p);
-        qsrc = qb.p;
-        qnorm = qn.p;
-    }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    int h[2] = {0, 0};
-    if ((e = cudaMemcpyAsync(h, flag.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-    // Integer data 0..255 with d <= 128: the GEMM-form distances are exact and
-    // the k best lists are the answer.  Otherwise (float data, or wider rows
-    // whose integer sums may pass 2^24) the GEMM keeps the KL = k + margin best
-    // candidates by its BF16 distance and an exact FP32 re-rank picks the k.
-    const bool exact = !h[0] && dk <= 128;
-    const int KL = exact ? l.k : (l.k + (l.k / 2 > 32 ? l.k / 2 : 32) < TC_MAXK ? l.k + (l.k / 2 > 32 ? l.k / 2 : 32)
-                                                                                 : TC_MAXK);
-    if (!exact && KL < l.k + 16) return cudaSuccess;  // no room for a margin: exact scan instead
-    CUtensorMap mA, mB;
-    const int64_t arows = l.self_join ? l.n - l.q0 : l.nq;
-    if (!make_map(&mA, qsrc, arows, dk, TC_M) || !make_map(&mB, xb.p, l.n, dk, TC_N)) return cudaSuccess;
+// The KL best per query row into ids / d2 [nq][KL]: by work units of 256 rows.
+static cudaError_t select_units(const KnnLaunch &l, const KnnOperands &o, int *idsout, float *d2out, cudaStream_t st) {
+    const int KL = o.KL;
+    const int64_t ntiles = o.ntiles;
     const int T = (int)((l.nq + TC_UNIT - 1) / TC_UNIT);
     const int S = knn_splits(T, ntiles, l.nq, KL);
-    // the rows' sorted lists live in the output arrays (exact) or in scratch
-    // (candidates, splits); distances are kept even when the caller asked for
-    // ids only
-    Scratch<float> d2s, d2p;
-    Scratch<int> ids_s, ids_p;
-    float *d2out = l.d2;
-    int *idsout = l.ids;
-    if (!exact) {
-        if ((e = ids_s.alloc((size_t)l.nq * KL)) != cudaSuccess) return e;
-        idsout = ids_s.p;
-    }
-    if (!exact || !d2out) {
-        if ((e = d2s.alloc((size_t)l.nq * KL)) != cudaSuccess) return e;
-        d2out = d2s.p;
-    }
+    cudaError_t e;
+    KnnScratch<float> d2p, vals;
+    KnnScratch<int> ids_p, cols;
     if (S > 1) {
         if ((e = ids_p.alloc((size_t)l.nq * S * KL)) != cudaSuccess) return e;
         if ((e = d2p.alloc((size_t)l.nq * S * KL)) != cudaSuccess) return e;
     }
-    Scratch<float> vals;
-    Scratch<int> cols;
     const int64_t grid = std::min<int64_t>((int64_t)T * S, sm_count());
     if ((e = vals.alloc((size_t)grid * TC_UNIT * TC_RING * 8)) != cudaSuccess) return e;
     if ((e = cols.alloc((size_t)grid * TC_UNIT * TC_RING)) != cudaSuccess) return e;
     TcArgs a;
-    a.qn = qnorm;
-    a.xn = xn.p;
+    a.qn = o.qn;
+    a.xn = o.xn;
     a.m = l.nq;
     a.n = l.n;
     a.q0 = l.q0;
     a.self_join = l.self_join;
     a.KL = KL;
-    a.kb = dk / TC_BOXK;
+    a.kb = o.dk / TC_BOXK;
     a.ids = S > 1 ? ids_p.p : idsout;
     a.d2 = S > 1 ? d2p.p : d2out;
-    a.err = flag.p + 1;
+    a.err = o.err;
     a.vals = vals.p;
     a.cols = cols.p;
     a.T = T;
@@ -1016,16 +954,11 @@ cudaError_t launch_knn_tc(const KnnLaunch &l, int *used, cudaStream_t st) {
     a.lsz = nullptr;
     a.first = a.last = 1;
     // Pre-pass: `rank` of the sample's 64-column minima have as many distinct
-    // columns at or below them (one more where a row meets itself).  Two
-    // minima per tile, 2.5 ranks' worth of tiles: the bound then admits ~1.1
-    // times the sample's own k nearest, and a larger sample would cost more
-    // tiles than the candidates it saves (k ln 2 per doubling, ~30 warp
-    // instructions each, against ~10 per tile and row).  At most a quarter of
-    // the base, and none when those are too few for a useful bound.
+    // columns at or below them (one more where a row meets itself).
     const int rank = KL + (l.self_join ? 1 : 0);
-    const int P = (int)std::min<int64_t>(ntiles / 4, (int64_t)rank * 5 / 2);
-    Scratch<float> minima, thr;
-    if (2 * P >= rank + rank / 4) {
+    const int P = knn_sample_tiles(ntiles, rank);
+    KnnScratch<float> minima, thr;
+    if (P > 0) {
         // up to 1 GB of minima at a time: blocks of row units
         const int64_t fit = (int64_t(1) << 30) / ((int64_t)2 * P * TC_UNIT * 4);
         const int TB = (int)std::max<int64_t>(1, std::min<int64_t>(T, fit));
@@ -1041,7 +974,7 @@ cudaError_t launch_knn_tc(const KnnLaunch &l, int *used, cudaStream_t st) {
             p.rt0 = t0;
             p.T = std::min(TB, T - t0);
             p.S = (int)std::max<int64_t>(1, std::min<int64_t>(P / 4, ((int64_t)sm_count() * 4 + p.T - 1) / p.T));
-            if ((e = launch_tc<true>(dk, mA, mB, p, st)) != cudaSuccess) return e;
+            if ((e = launch_tc<true>(o.dk, o.mq, o.mx, p, st)) != cudaSuccess) return e;
             const int64_t r0 = (int64_t)t0 * TC_UNIT, rows = std::min<int64_t>((int64_t)p.T * TC_UNIT, l.nq - r0);
             const int64_t blocks = std::min<int64_t>((rows + 7) / 8, (int64_t)sm_count() * 16);
             auto bound = 2 * P <= 512 ? knn_bound_kernel<16> : 2 * P <= 1024 ? knn_bound_kernel<32> : knn_bound_kernel<48>;
@@ -1050,27 +983,20 @@ cudaError_t launch_knn_tc(const KnnLaunch &l, int *used, cudaStream_t st) {
         }
         a.thr0 = thr.p;
     }
-    // An unsplit base is taken in chunks of ~48 MB of BF16 rows, one launch per
-    // chunk over every row unit, so a chunk stays in L2 while all units pass
-    // over it (a single sweep per CTA would re-read a base larger than L2 from
-    // HBM once per wave of CTAs).  Rows see columns in increasing id across
-    // chunks, and their lists carry over through the output arrays and lsz.
-    int64_t chunk_tiles = std::max<int64_t>(1, (int64_t(48) << 20) / ((int64_t)TC_N * dk * 2));
-    if (const char *ct = getenv("NSG_KNN_CHUNK_TILES"))  // smaller chunks (tests)
-        if (atoi(ct) > 0) chunk_tiles = atoi(ct);
-    if (S > 1) chunk_tiles = ntiles;
-    const int64_t nchunks = (ntiles + chunk_tiles - 1) / chunk_tiles;
-    Scratch<int> lsz;
+    // an unsplit base is taken in chunks: rows see columns in increasing id
+    // across them, and their lists carry over through the output arrays and lsz
+    const int64_t chunk = S > 1 ? ntiles : knn_chunk_tiles(o.dk), nchunks = (ntiles + chunk - 1) / chunk;
+    KnnScratch<int> lsz;
     if (nchunks > 1 && (e = lsz.alloc((size_t)l.nq)) != cudaSuccess) return e;
     a.lsz = lsz.p;
     a.S = S;
     a.stride = 1;
     for (int64_t c = 0; c < nchunks; ++c) {
-        a.tile0 = (int)(c * chunk_tiles);
-        a.tile1 = (int)std::min<int64_t>(ntiles, (c + 1) * chunk_tiles);
+        a.tile0 = (int)(c * chunk);
+        a.tile1 = (int)std::min<int64_t>(ntiles, (c + 1) * chunk);
         a.first = c == 0;
         a.last = c == nchunks - 1;
-        if ((e = launch_tc<false>(dk, mA, mB, a, st)) != cudaSuccess) return e;
+        if ((e = launch_tc<false>(o.dk, o.mq, o.mx, a, st)) != cudaSuccess) return e;
     }
     if (S > 1) {
         const size_t smem = (size_t)8 * 5 * KL * sizeof(uint64_t);
@@ -1081,11 +1007,94 @@ cudaError_t launch_knn_tc(const KnnLaunch &l, int *used, cudaStream_t st) {
         knn_merge_kernel<<<(unsigned)blocks, 256, smem, st>>>(a.ids, a.d2, l.nq, S, KL, idsout, d2out);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if ((e = cudaMemcpyAsync(h, flag.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+    return knn_finish(o, st);  // scratch is freed on return
+}
+
+cudaError_t knn_finish(const KnnOperands &o, cudaStream_t st) {
+    int failed = 0;
+    cudaError_t e = cudaMemcpyAsync(&failed, o.err, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    return e == cudaSuccess && failed ? cudaErrorLaunchTimeout : e;
+}
+
+int64_t knn_chunk_tiles(int dk) {
+    if (const char *ct = getenv("NSG_KNN_CHUNK_TILES"))
+        if (atoi(ct) > 0) return atoi(ct);
+    return std::max<int64_t>(1, (int64_t(48) << 20) / ((int64_t)TC_N * dk * 2));
+}
+
+// Tensor-core kNN when the data allows an exact answer (integer 0..255,
+// d <= 128, k <= 256); *used = 0 when it does not apply (nothing written).
+cudaError_t launch_knn_tc(const KnnLaunch &l, int *used, cudaStream_t st) {
+    *used = 0;
+    if (l.nq <= 0 || l.k > TC_MAXK || l.dp > 1024 || !encode_fn()) return cudaSuccess;
+    const int dk = l.dp <= 64 ? 64 : (l.dp <= 128 ? 128 : (l.dp + 63) / 64 * 64);
+    const int64_t ntiles = (l.n + TC_N - 1) / TC_N;
+    if (ntiles > INT32_MAX / TC_N) return cudaSuccess;
+    const int64_t npad = ntiles * TC_N;
+    KnnScratch<__nv_bfloat16> xb, qb;
+    KnnScratch<float> xn, qn;
+    KnnScratch<int> flag;
+    cudaError_t e;
+    if ((e = xb.alloc((size_t)l.n * dk)) != cudaSuccess) return e;
+    if ((e = xn.alloc((size_t)npad)) != cudaSuccess) return e;
+    if ((e = flag.alloc(2)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(flag.p, 0, 2 * sizeof(int), st)) != cudaSuccess) return e;
+    const int grid_rows = sm_count() * 8;
+    bf16_rows_kernel<<<grid_rows, 256, 0, st>>>(reinterpret_cast<const float4 *>(l.base), l.n, l.dp / 4,
+                                                reinterpret_cast<uint2 *>(xb.p), dk / 4, xn.p, npad, flag.p);
+    KnnOperands o;
+    o.xn = xn.p;
+    const __nv_bfloat16 *qsrc = xb.p + (l.self_join ? l.q0 * dk : 0);
+    o.qn = xn.p + (l.self_join ? l.q0 : 0);
+    o.dk = dk;
+    o.ntiles = ntiles;
+    o.err = flag.p + 1;
+    if (!l.self_join) {
+        if ((e = qb.alloc((size_t)l.nq * dk)) != cudaSuccess) return e;
+        if ((e = qn.alloc((size_t)l.nq)) != cudaSuccess) return e;
+        bf16_rows_kernel<<<grid_rows, 256, 0, st>>>(reinterpret_cast<const float4 *>(l.queries), l.nq, l.dp / 4,
+                                                    reinterpret_cast<uint2 *>(qb.p), dk / 4, qn.p, l.nq, flag.p);
+        qsrc = qb.p;
+        o.qn = qn.p;
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    int other = 0;
+    if ((e = cudaMemcpyAsync(&other, flag.p, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-    if (h[1]) return cudaErrorLaunchTimeout;  // a pipeline wait gave up (bounded waits)
+    // Integer data 0..255 with d <= 128: the GEMM-form distances are exact and
+    // the k best lists are the answer.  Otherwise (float data, or wider rows
+    // whose integer sums may pass 2^24) the GEMM keeps the KL = k + margin best
+    // candidates by its BF16 distance and an exact FP32 re-rank picks the k.
+    const bool exact = !other && dk <= 128;
+    o.KL = exact ? l.k : std::min(l.k + std::max(l.k / 2, 32), TC_MAXK);
+    if (!exact && o.KL < l.k + 16) return cudaSuccess;  // no room for a margin: exact scan instead
+    if (!make_map(&o.mq, qsrc, l.self_join ? l.n - l.q0 : l.nq, dk) || !make_map(&o.mx, xb.p, l.n, dk))
+        return cudaSuccess;
+    // the rows' sorted lists live in the output arrays (exact) or in scratch
+    // (candidates); distances are kept even when the caller asked for ids only
+    KnnScratch<float> d2s;
+    KnnScratch<int> ids_s;
+    float *d2out = l.d2;
+    int *idsout = l.ids;
     if (!exact) {
-        if ((e = launch_knn_rerank(l, idsout, KL, st)) != cudaSuccess) return e;
+        if ((e = ids_s.alloc((size_t)l.nq * o.KL)) != cudaSuccess) return e;
+        idsout = ids_s.p;
+    }
+    if (!exact || !d2out) {
+        if ((e = d2s.alloc((size_t)l.nq * o.KL)) != cudaSuccess) return e;
+        d2out = d2s.p;
+    }
+    const bool bounded = knn_sample_tiles(ntiles, o.KL + (l.self_join ? 1 : 0)) > 0;
+    bool small = knn_small(l.n, l.nq, o.KL, bounded, sm_count());
+    if (const char *env = getenv("NSG_KNN_ENGINE")) {  // one of the kernels (tests)
+        if (strcmp(env, "small") == 0) small = true;
+        else if (strcmp(env, "units") == 0) small = false;
+    }
+    e = small ? knn_select_small(l, o, idsout, d2out, st) : select_units(l, o, idsout, d2out, st);
+    if (e != cudaSuccess) return e;
+    if (!exact) {
+        if ((e = launch_knn_rerank(l, idsout, o.KL, st)) != cudaSuccess) return e;
         if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;  // scratch is freed on return
     }
     *used = 1;

@@ -3,7 +3,7 @@
 // by themselves.  With few tiles most columns are candidates, so merging is
 // the work and there is little scan to hide it behind; the pre-pass, the rings
 // and the splits' lists then cost more than they save.  The rule that
-// chooses is knn_small (capi.cu), with both sides' times.
+// chooses is in knn_rule.h, with both sides' times.
 //
 // CTA = 6 warps: warp 0 issues TMA (the 128 x d query tile once, then a ring
 // of base tiles), warp 1 owns TMEM and issues the MMAs into two accumulator
@@ -12,18 +12,13 @@
 // |x_j|^2 - 2 q.x_j < (current k-th distance) - |q|^2; the common case costs
 // one FMA and one min per element (a group of 16 columns is tested through its
 // minimum).  Columns arrive in increasing id, so a strict comparison on the
-// distance alone implements the (distance, id) order.  Buffers of 16+ keys are
+// distance alone implements the (distance, id) order.  Buffers of 48+ keys are
 // merged warp-cooperatively into the row's sorted list, which lives in the
 // output arrays.
 #include <algorithm>
-#include <cstdlib>
-
-#include <cuda.h>
-#include <cudaTypedefs.h>
-#include <cuda_bf16.h>
 
 #include "common.cuh"
-#include "kernels.h"
+#include "knn_tc.cuh"
 #include "tc_ptx.cuh"
 
 namespace nsg {
@@ -178,7 +173,7 @@ __device__ __noinline__ void merge_row(int src, int row_local, int64_t row_g, in
 
 template <int DK>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-    knn_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcArgs a) {
+    knn_tc_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, TcArgs a) {
     using Cfg = TcCfg<DK>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>(
@@ -444,185 +439,48 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
 }
 
-// Row-wise BF16 copy with K padded to DK, squared norms of the rounded values,
-// and a flag raised when a value is not an integer in 0..255.
-__global__ void bf16_rows_kernel(const float *__restrict__ src, int64_t rows, int dp, __nv_bfloat16 *dst,
-                                 int dk, float *norms, int64_t rows_pad, int *nonint) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    const unsigned lane = lane_id();
-    for (int64_t r = warp; r < rows_pad; r += nw) {
-        float acc = 0.0f;
-        bool bad = false;
-        for (int c = lane; c < dk; c += 32) {
-            float v = (r < rows && c < dp) ? src[r * dp + c] : 0.0f;
-            __nv_bfloat16 h = __float2bfloat16_rn(v);
-            float hv = __bfloat162float(h);
-            acc += hv * hv;
-            bad |= !(v >= 0.0f && v <= 255.0f && v == rintf(v));
-            if (r < rows) dst[r * dk + c] = h;
-        }
-        acc = group_sum<32>(acc);
-        if (lane == 0) norms[r] = r < rows ? acc : 0.0f;
-        if (__any_sync(NSG_FULL, bad) && lane == 0 && r < rows) atomicOr(nonint, 1);
-    }
+template <int DK>
+cudaError_t launch(const CUtensorMap &mA, const CUtensorMap &mB, const TcArgs &a, cudaStream_t st) {
+    auto kern = knn_tc_small_kernel<DK>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<DK>::SMEM);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)((a.m + TC_M - 1) / TC_M), TC_THREADS, TcCfg<DK>::SMEM, st>>>(mA, mB, a);
+    return cudaGetLastError();
 }
-
-PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
-    return fn;
-}
-
-// 2-D tensor map over a [rows][dk] bf16 matrix, box = 64 (K) x box_rows, 128B swizzle.
-bool make_map(CUtensorMap *map, const void *ptr, int64_t rows, int dk, int box_rows) {
-    auto fn = encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)dk, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)dk * 2};
-    cuuint32_t box[2] = {(cuuint32_t)TC_BOXK, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
-}
-
-template <typename T>
-struct Scratch {
-    T *p = nullptr;
-    ~Scratch() {
-        if (p) cudaFree(p);
-    }
-    cudaError_t alloc(size_t n) { return cudaMalloc(reinterpret_cast<void **>(&p), n * sizeof(T) + 16); }
-};
 
 }  // namespace
 
-// Tensor-core kNN when the data allows an exact answer (integer 0..255,
-// d <= 128, k <= 256); *used = 0 when it does not apply (nothing written).
-cudaError_t launch_knn_tc_small(const KnnLaunch &l, int *used, cudaStream_t st) {
-    *used = 0;
-    if (l.nq <= 0 || l.k > TC_MAXK || l.dp > 1024 || !encode_fn()) return cudaSuccess;
-    const int dk = l.dp <= 64 ? 64 : (l.dp <= 128 ? 128 : (l.dp + 63) / 64 * 64);
-    const int64_t ntiles = (l.n + TC_N - 1) / TC_N;
-    if (ntiles > INT32_MAX / TC_N) return cudaSuccess;
-    const int64_t npad = ntiles * TC_N;
-    Scratch<__nv_bfloat16> xb, qb;
-    Scratch<float> xn, qn;
-    Scratch<int> flag;
-    cudaError_t e;
-    if ((e = xb.alloc((size_t)l.n * dk)) != cudaSuccess) return e;
-    if ((e = xn.alloc((size_t)npad)) != cudaSuccess) return e;
-    if ((e = flag.alloc(2)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(flag.p, 0, 2 * sizeof(int), st)) != cudaSuccess) return e;
-    const int grid_rows = sm_count() * 8;
-    bf16_rows_kernel<<<grid_rows, 256, 0, st>>>(l.base, l.n, l.dp, xb.p, dk, xn.p, npad, flag.p);
-    const __nv_bfloat16 *qsrc = xb.p + (l.self_join ? l.q0 * dk : 0);
-    const float *qnorm = xn.p + (l.self_join ? l.q0 : 0);
-    if (!l.self_join) {
-        if ((e = qb.alloc((size_t)l.nq * dk)) != cudaSuccess) return e;
-        if ((e = qn.alloc((size_t)l.nq)) != cudaSuccess) return e;
-        bf16_rows_kernel<<<grid_rows, 256, 0, st>>>(l.queries, l.nq, l.dp, qb.p, dk, qn.p, l.nq, flag.p);
-        qsrc = qb.p;
-        qnorm = qn.p;
-    }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    int h[2] = {0, 0};
-    if ((e = cudaMemcpyAsync(h, flag.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-    // Integer data 0..255 with d <= 128: the GEMM-form distances are exact and
-    // the k best lists are the answer.  Otherwise (float data, or wider rows
-    // whose integer sums may pass 2^24) the GEMM keeps the KL = k + margin best
-    // candidates by its BF16 distance and an exact FP32 re-rank picks the k.
-    const bool exact = !h[0] && dk <= 128;
-    const int KL = exact ? l.k : (l.k + (l.k / 2 > 32 ? l.k / 2 : 32) < TC_MAXK ? l.k + (l.k / 2 > 32 ? l.k / 2 : 32)
-                                                                                 : TC_MAXK);
-    if (!exact && KL < l.k + 16) return cudaSuccess;  // no room for a margin: exact scan instead
-    CUtensorMap mA, mB;
-    const int64_t arows = l.self_join ? l.n - l.q0 : l.nq;
-    if (!make_map(&mA, qsrc, arows, dk, TC_M) || !make_map(&mB, xb.p, l.n, dk, TC_N)) return cudaSuccess;
-    // the rows' sorted lists live in the output arrays (exact) or in scratch
-    // (candidates); distances are kept even when the caller asked for ids only
-    Scratch<float> d2s;
-    Scratch<int> ids_s;
-    float *d2out = l.d2;
-    int *idsout = l.ids;
-    if (!exact) {
-        if ((e = ids_s.alloc((size_t)l.nq * KL)) != cudaSuccess) return e;
-        idsout = ids_s.p;
-    }
-    if (!exact || !d2out) {
-        if ((e = d2s.alloc((size_t)l.nq * KL)) != cudaSuccess) return e;
-        d2out = d2s.p;
-    }
+cudaError_t knn_select_small(const KnnLaunch &l, const KnnOperands &o, int *ids, float *d2, cudaStream_t st) {
     TcArgs a;
-    a.qn = qnorm;
-    a.xn = xn.p;
+    a.qn = o.qn;
+    a.xn = o.xn;
     a.m = l.nq;
     a.n = l.n;
     a.q0 = l.q0;
     a.self_join = l.self_join;
-    a.KL = KL;
-    a.kb = dk / TC_BOXK;
-    a.ids = idsout;
-    a.d2 = d2out;
-    a.err = flag.p + 1;
-    // The base is taken in chunks of ~48 MB of BF16 rows, one launch per chunk
-    // over every query tile, so a chunk stays in L2 while all query tiles pass
-    // over it (a single sweep per CTA would re-read a base larger than L2 from
-    // HBM once per wave of CTAs).  Rows see columns in increasing id across
-    // chunks, and their lists carry over through the output arrays and lsz.
-    int64_t chunk_tiles = std::max<int64_t>(1, (int64_t(48) << 20) / ((int64_t)TC_N * dk * 2));
-    if (const char *ct = getenv("NSG_KNN_CHUNK_TILES"))  // smaller chunks (tests)
-        if (atoi(ct) > 0) chunk_tiles = atoi(ct);
-    const int64_t nchunks = (ntiles + chunk_tiles - 1) / chunk_tiles;
-    Scratch<int> lsz;
+    a.KL = o.KL;
+    a.kb = o.dk / TC_BOXK;
+    a.ids = ids;
+    a.d2 = d2;
+    a.err = o.err;
+    // rows see columns in increasing id across chunks, and their lists carry over
+    // through the output arrays and lsz
+    const int64_t chunk = knn_chunk_tiles(o.dk), nchunks = (o.ntiles + chunk - 1) / chunk;
+    cudaError_t e;
+    KnnScratch<int> lsz;
     if (nchunks > 1 && (e = lsz.alloc((size_t)l.nq)) != cudaSuccess) return e;
     a.lsz = lsz.p;
-    const int64_t grid = (l.nq + TC_M - 1) / TC_M;
     for (int64_t c = 0; c < nchunks; ++c) {
-        a.t0 = (int)(c * chunk_tiles);
-        a.t1 = (int)std::min<int64_t>(ntiles, (c + 1) * chunk_tiles);
+        a.t0 = (int)(c * chunk);
+        a.t1 = (int)std::min<int64_t>(o.ntiles, (c + 1) * chunk);
         a.first = c == 0;
         a.last = c == nchunks - 1;
-        if (dk == 64) {
-            auto kern = knn_tc_kernel<64>;
-            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<64>::SMEM)) !=
-                cudaSuccess)
-                return e;
-            kern<<<(unsigned)grid, TC_THREADS, TcCfg<64>::SMEM, st>>>(mA, mB, a);
-        } else if (dk == 128) {
-            auto kern = knn_tc_kernel<128>;
-            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<128>::SMEM)) !=
-                cudaSuccess)
-                return e;
-            kern<<<(unsigned)grid, TC_THREADS, TcCfg<128>::SMEM, st>>>(mA, mB, a);
-        } else {
-            auto kern = knn_tc_kernel<0>;
-            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<0>::SMEM)) !=
-                cudaSuccess)
-                return e;
-            kern<<<(unsigned)grid, TC_THREADS, TcCfg<0>::SMEM, st>>>(mA, mB, a);
-        }
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = o.dk == 64 ? launch<64>(o.mq, o.mx, a, st)
+            : o.dk == 128 ? launch<128>(o.mq, o.mx, a, st)
+                          : launch<0>(o.mq, o.mx, a, st);
+        if (e != cudaSuccess) return e;
     }
-    if ((e = cudaMemcpyAsync(h, flag.p, 2 * sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-    if (h[1]) return cudaErrorLaunchTimeout;  // a pipeline wait gave up (bounded waits)
-    if (!exact) {
-        if ((e = launch_knn_rerank(l, idsout, KL, st)) != cudaSuccess) return e;
-        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;  // scratch is freed on return
-    }
-    *used = 1;
-    return cudaSuccess;
+    return knn_finish(o, st);  // lsz is freed on return
 }
 
 }  // namespace nsg
