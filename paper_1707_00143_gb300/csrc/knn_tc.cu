@@ -321,13 +321,20 @@ __device__ __forceinline__ int unit_groups(const TcArgs &a, int rt) {
 
 // A row's bound on |x|^2 - 2 q.x and its list's size when a unit begins: the
 // k-th key carried over from earlier chunks once the list holds k, before that
-// the pre-pass's; a row past the end takes nothing.
+// the pre-pass's; a row past the end takes nothing.  Keys are rounded sums with
+// |q|^2 and equal ones go by id, so the pre-pass's bound is widened by what that
+// rounding can make equal, and a norm past FP32's range (every key infinite)
+// leaves it out.
 __device__ __forceinline__ float first_bound(const TcArgs &a, int64_t row, int64_t list, int *lsize) {
     *lsize = 0;
-    if (row >= a.m) return __int_as_float(0xff800000);
+    const float inf = __int_as_float(0x7f800000);
+    if (row >= a.m) return -inf;
     if (!a.first) *lsize = a.lsz[row];
-    if (*lsize == a.KL) return a.d2[list + a.KL - 1] - a.qn[row];
-    return a.thr0 ? a.thr0[row] : __int_as_float(0x7f800000);
+    const float q2 = a.qn[row];
+    if (*lsize == a.KL) return a.d2[list + a.KL - 1] - q2;
+    if (a.thr0 == nullptr || !(q2 < inf)) return inf;
+    const float t = a.thr0[row];
+    return t + (q2 + fabsf(t)) * (1.0f / (1 << 22));
 }
 
 // MINS: the pre-pass (minima of every sample tile's two 64-column groups),

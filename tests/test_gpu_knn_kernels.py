@@ -74,3 +74,20 @@ def test_both_kernels_agree_on_a_large_float_base(nsg, monkeypatch):
         monkeypatch.setenv("NSG_KNN_ENGINE", e)
         out.append(nsg.nsg_knn_query(T(base), T(q), 50))
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("scale", [1.0, 4096.0, 1e6, 3e19])
+def test_far_queries(nsg, monkeypatch, scale):
+    """Queries so far away that FP32 distances tie by the hundred (or, past FP32's range, all do): ties go by
+    id in both kernels, whatever bounds the pre-pass of one of them."""
+    n, d = 30000, 96
+    base, q = datagen.uniform_float(n, d, seed=5), datagen.uniform_float(400, d, seed=6)
+    q = (q * np.float32(scale)).astype(np.float32)
+    out = []
+    for e in ("units", "small"):
+        monkeypatch.setenv("NSG_KNN_ENGINE", e)
+        out.append([t.cpu().numpy() for t in nsg.nsg_knn_query(T(base), T(q), 10)])
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+    if scale > 1e19:
+        assert np.isinf(out[0][1]).all()
+        assert np.array_equal(out[0][0], np.tile(np.arange(10), (400, 1)))
