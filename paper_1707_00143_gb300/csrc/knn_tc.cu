@@ -1098,7 +1098,14 @@ cudaError_t launch_knn_tc(const KnnLaunch &l, int *used, cudaStream_t st) {
         if (strcmp(env, "small") == 0) small = true;
         else if (strcmp(env, "units") == 0) small = false;
     }
-    e = small ? knn_select_small(l, o, idsout, d2out, st) : select_units(l, o, idsout, d2out, st);
+    if (!small) {
+        e = select_units(l, o, idsout, d2out, st);
+        if (e == cudaErrorMemoryAllocation) {  // up to 1 GB of minima, splits' lists, rings: do without
+            cudaGetLastError();
+            small = true;
+        }
+    }
+    if (small) e = knn_select_small(l, o, idsout, d2out, st);
     if (e != cudaSuccess) return e;
     if (!exact) {
         if ((e = launch_knn_rerank(l, idsout, o.KL, st)) != cudaSuccess) return e;
