@@ -280,12 +280,17 @@ bool nndescent_params_ok(const nsg_nndescent_params &p) {
 // Integer data of span <= 255 with d * 255^2 < 2^24 (every distance an exact
 // integer below 2^24) gets an 8-bit copy x - min of base [n][dp] for the build's
 // distances: the same keys as the FP32 rows at a quarter of the bytes gathered.
-// Other data, and data whose copy finds no memory: x.rows stays null.
+// Other data, and data whose copy would not leave `reserve` bytes of memory for
+// what cannot be done without: x.rows stays null.
+constexpr size_t kExact8Reserve = size_t(256) << 20;  // searches' scratch, other copies
 nsg_status exact8_copy(const float *base, int64_t n, int dp, int d, DevBuf<unsigned char> &buf, nsg::Exact8 &x,
-                       cudaStream_t st) {
+                       cudaStream_t st, size_t reserve = kExact8Reserve) {
     x = nsg::Exact8{};
     const int dpl = (d + 15) / 16 * 16;
     if ((int64_t)d * 65025 >= (1 << 24)) return NSG_OK;
+    size_t free = 0, total = 0;
+    NSG_CK(cudaMemGetInfo(&free, &total));
+    if (free < (size_t)n * dpl + reserve) return NSG_OK;
     DevBuf<unsigned> flags;
     NSG_CK(flags.alloc(4));
     unsigned mm[3] = {0xffffffffu, 0u, 0u};
@@ -403,24 +408,26 @@ void make_collect_log(int L, int K, int64_t nv, DevBuf<uint64_t> &buf, nsg::Coll
     log.seen = reinterpret_cast<int *>(buf.p + log.size);
 }
 
+// Nodes whose candidate lists are materialised at a time (2 GiB of them).
+int64_t collect_chunk(int64_t n, int C) {
+    return std::max<int64_t>(1, std::min<int64_t>(n, (int64_t)((size_t(2) << 30) / ((size_t)C * 8 + 8))));
+}
+
 nsg_status collect_prune_all(const float *bp, int64_t n, int dp, const int *knn, int K, int nav, int L,
                              int R, int C, int *adj, int *deg, float *ms_collect, float *ms_prune,
                              int64_t *examined, const nsg::Exact8 &u8, cudaStream_t st) {
-    // candidate lists are materialised for a chunk of nodes at a time
-    const size_t budget = size_t(2) << 30;
-    int64_t chunk = (int64_t)(budget / ((size_t)C * 8 + 8));
-    if (chunk > n) chunk = n;
-    if (chunk < 1) chunk = 1;
+    const int64_t chunk = collect_chunk(n, C);
     DevBuf<int> cid, ccnt;
     DevBuf<float> cd2;
     DevBuf<unsigned long long> nexam;
-    DevBuf<uint64_t> logbuf;
-    nsg::CollectLog log;
-    if (!collect_force("merge")) make_collect_log(L, K, chunk, logbuf, log);
     NSG_CK(cid.alloc((size_t)chunk * C));
     NSG_CK(cd2.alloc((size_t)chunk * C));
     NSG_CK(ccnt.alloc(chunk));
     NSG_CK(nexam.alloc(1));
+    // last: the build goes on without logs, but not without the lists
+    DevBuf<uint64_t> logbuf;
+    nsg::CollectLog log;
+    if (!collect_force("merge")) make_collect_log(L, K, chunk, logbuf, log);
     NSG_CK(cudaMemsetAsync(nexam.p, 0, sizeof(unsigned long long), st));
     cudaEvent_t ev[3];
     for (auto &e : ev) NSG_CK(cudaEventCreate(&e));
@@ -832,10 +839,14 @@ static nsg_status build_index(const float *base_dev, int64_t n, int32_t d, int32
     if (!s && (e = knn.alloc((size_t)n * K)) != cudaSuccess) s = cuda_fail(e, "alloc knn");
     DevBuf<unsigned char> u8buf;
     nsg::Exact8 u8;
-    if (!s) s = exact8_copy(base.p, n, ix->dp, d, u8buf, u8, st);
     // A1: kNN graph, exact or by nn-descent
     auto t0 = std::chrono::steady_clock::now();
     if (!s && !nnd) s = knn_run(base.p, n, ix->dp, base.p, n, 0, K, 1, knn.p, nullptr, st);
+    // what the stages to come cannot do without: candidate lists, the connectivity
+    // pass's arrays (28 bytes per row and up to 512 MB of pools), nn-descent's
+    size_t reserve = std::max((size_t)collect_chunk(n, C) * ((size_t)C * 8 + 8), 28 * (size_t)n + (size_t(512) << 20));
+    if (nnd) reserve = std::max(reserve, nsg::nndescent_scratch_bytes(n, K, nnd->sample, nnd->reverse));
+    if (!s) s = exact8_copy(base.p, n, ix->dp, d, u8buf, u8, st, reserve + kExact8Reserve);
     if (!s && nnd) s = nndescent_run(base.p, n, ix->dp, d, K, *nnd, u8, knn.p, nullptr, &ix->knn_iters, nullptr,
                                st);
     if (!s && (e = cudaStreamSynchronize(st)) != cudaSuccess) s = cuda_fail(e, "knn");

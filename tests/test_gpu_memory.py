@@ -34,3 +34,20 @@ def test_knn_query_without_scratch(nsg):
     with Taken(160 << 20):
         got = nsg.nsg_knn_query(base, q, 100)
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+def test_build_without_logs_and_copy(nsg):
+    torch.manual_seed(2)
+    base = torch.randint(0, 256, (66_000, 16), device="cuda").float()
+    args = (30, 40, 16, 4096)  # candidate lists of 2 GiB
+    want = nsg.nsg_build(base, *args)
+    adj, deg = want.graph()
+    info = want.info()
+    want.free()
+    # the lists, ~30 MB of base, graphs and counters, and less than the 256 MB that the copy leaves free
+    with Taken((2 << 30) + (200 << 20)):
+        idx = nsg.nsg_build(base, *args)
+        assert idx.info()["nav"] == info["nav"]
+        assert idx.info()["device_bytes"] == info["device_bytes"] - 66_000 * 16  # without the 8-bit copy
+    a, d = idx.graph()
+    assert torch.equal(a, adj) and torch.equal(d, deg)
