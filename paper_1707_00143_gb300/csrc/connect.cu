@@ -311,7 +311,7 @@ __device__ __forceinline__ bool fix_stale(const FixArgs &a, int f, int u) {
                 const float lim = __shfl_sync(NSG_FULL, bar, src);
                 float d2 = 0.0f;
                 for (int c = (int)lane; c < a.dp4; c += 32) d2 += sq4(__ldg(xu + c), __ldg(xw + c));
-                if (group_sum<32>(d2) <= lim) return true;
+                if (!(group_sum<32>(d2) > lim)) return true;  // a NaN on either side: searched again
             }
         }
     }
