@@ -19,7 +19,8 @@
 //            graph with the proposals of earlier fix-ups (GraphView hides the
 //            later ones) -- in the first round for all, then only where a changed
 //            proposal could have changed it -- and picks its s with the degrees
-//            that view gives; then one CTA collects the proposals, sorts them by
+//            that view gives; then one CTA finds sources for those whose pools
+//            have no room, collects the proposals, sorts them by
 //            (source, fix-up) and writes them past the rows' degrees.  Fix-up 0
 //            depends on nothing, and once the fix-ups before f stand still, f is
 //            final after one more round: whatever precedes the first proposal
@@ -91,6 +92,7 @@ struct FixState {
     int added, status, capped, redone;  // totals of the pass
     int B;                              // ids the next list takes
     int stamp;                          // last label level run
+    int room;                           // every id below it is full
     int lev[LABEL_LEVELS + 1];          // queue sizes of this batch's label levels
 };
 
@@ -178,7 +180,8 @@ struct FixArgs {
     uint64_t *pools, *xthr;   // [B][L] final pools; [B][xcap] entry bar at each expansion
     int *xlog, *xcnt, *psize; // [B][xcap] expanded nodes; expansions (INT_MAX: the search hit its cap)
     int xcap;
-    int *snew, *scur;         // [B] proposed source (-1: no pool entry has room), this and the last round
+    int *snew, *scur;         // [B] proposed source (-1: nothing has room), this and the last round
+    int *used;                // [n] proposals that take a source's slots, 0 between uses
     int *slot, *hold;         // [B] adjacency slot a proposal occupies (-1: none) and what it held
     uint64_t *ent;            // [2 * B]
 };
@@ -391,13 +394,71 @@ __device__ __forceinline__ void withdraw(const FixArgs &a, int F, int from, int 
     for (int p = threadIdx.x; p < nent; p += blockDim.x) a.head[ent_src(a.ent[p])] = make_int2(0, 0);
 }
 
+// Sources for the fix-ups whose pools have no room: in order, the smallest id
+// that is reached when the fix-ups before are made and has a slot that their
+// proposals leave.  Block-wide; list [F] in shared memory.  Taken one per batch, at its
+// end, they had cost a batch each (20,000 x 16 uniform rows, K = R = 5: the pass 132
+// ms; 20,000 x 1,500, R = 24: 894 ms).
+__device__ __forceinline__ void fix_fallback(const FixArgs &a, int F, int *list, int *warp_sum, int *found) {
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    int cnt = 0;
+    for (int b = 0; b < F; b += nt) {
+        const int f = b + tid;
+        const bool is = f < F && a.snew[f] < 0;
+        const unsigned bal = __ballot_sync(NSG_FULL, is);
+        if (lane == 0) warp_sum[warp] = __popc(bal);
+        __syncthreads();
+        int before = cnt;
+        for (int k = 0; k < (nt >> 5); ++k) {
+            if (k < warp) before += warp_sum[k];
+            cnt += warp_sum[k];
+        }
+        if (is) list[before + __popc(bal & lanemask_lt())] = f;
+        __syncthreads();
+    }
+    if (cnt == 0) return;
+    int prev = 0, room = a.st->room;
+    for (int i = 0; i < cnt; ++i) {
+        const int f = list[i], lim = a.flab[f];
+        for (int g = prev + tid; g < f; g += nt)
+            if (ldv(a.snew + g) >= 0) atomicAdd(a.used + ldv(a.snew + g), 1);
+        prev = f;
+        int sel = INT_MAX;
+        bool full = true;  // every id so far
+        for (int64_t w0 = room; w0 < a.n && sel == INT_MAX; w0 += nt) {
+            if (tid == 0) found[0] = found[1] = INT_MAX;
+            __syncthreads();
+            const int64_t x = w0 + tid;
+            if (x < a.n && a.deg[x] < a.R) {
+                atomicMin(found, (int)x);
+                if (a.deg[x] + ldv(a.used + x) < a.R && (bit_is_set(a.reached, x) || a.label[x] < lim))
+                    atomicMin(found + 1, (int)x);
+            }
+            __syncthreads();
+            const int first = found[0];
+            sel = found[1];
+            __syncthreads();
+            if (full) room = first == INT_MAX ? (int)(w0 + nt < a.n ? w0 + nt : a.n) : first;
+            full = full && first == INT_MAX;
+        }
+        if (sel == INT_MAX) break;  // no room anywhere: the batch ends here
+        if (tid == 0) a.snew[f] = sel;
+        __syncthreads();
+    }
+    __syncthreads();
+    if (tid == 0) a.st->room = room;
+    for (int f = tid; f < F; f += nt)
+        if (ldv(a.snew + f) >= 0) a.used[ldv(a.snew + f)] = 0;
+    __syncthreads();
+}
+
 // The round's proposals against the last round's: entries sorted by source,
 // the current ones written past their sources' degrees in fix-up order (the
 // slots the sequential loop would give them).  One CTA.
 __global__ void __launch_bounds__(1024) fix_propose_kernel(FixArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *ent = reinterpret_cast<uint64_t *>(smem);
-    __shared__ int sh_n, sh_first, sh_none;
+    __shared__ int sh_n, sh_first, sh_none, sh_found[2], sh_sum[32];
     FixState *st = a.st;
     const int tid = threadIdx.x, nt = blockDim.x;
     if (st->settled) return;
@@ -408,6 +469,8 @@ __global__ void __launch_bounds__(1024) fix_propose_kernel(FixArgs a) {
         sh_none = INT_MAX;
     }
     withdraw(a, F, 0, st->nent);
+    __syncthreads();
+    fix_fallback(a, F, reinterpret_cast<int *>(smem), sh_sum, sh_found);
     __syncthreads();
     for (int f = tid; f < F; f += nt) {
         const int was = a.scur[f], now = a.snew[f];
@@ -471,9 +534,8 @@ __global__ void __launch_bounds__(1024) fix_propose_kernel(FixArgs a) {
     }
 }
 
-// The final prefix of the batch enters the graph; a fix-up whose pool has no
-// room (the first one, if any) takes the smallest reached id with a free slot.
-// One CTA.
+// The final prefix of the batch enters the graph; a fix-up for which nothing had
+// room is tried once more against the graph itself.  One CTA.
 __global__ void __launch_bounds__(1024) fix_commit_kernel(FixArgs a) {
     __shared__ int sh_found;
     FixState *st = a.st;
@@ -549,8 +611,8 @@ cudaError_t run_connect(const ConnectLaunch &l, int out_host[4], cudaStream_t st
         need += (bytes + 255) & ~size_t(255);
         return at;
     };
-    const size_t o_reached = plan(4 * nwords), o_stamp = plan(4 * n), o_head = plan(8 * n), o_st = plan(sizeof(FixState)),
-                 o_lev = plan(4 * (BFS_LEVELS + 1)), zeroed = need;
+    const size_t o_reached = plan(4 * nwords), o_stamp = plan(4 * n), o_used = plan(4 * n), o_head = plan(8 * n),
+                 o_st = plan(sizeof(FixState)), o_lev = plan(4 * (BFS_LEVELS + 1)), zeroed = need;
     const size_t o_label = plan(4 * n), o_qa = plan(4 * n), o_qb = plan(4 * n), o_touched = plan(4 * n),
                  o_list = plan(4 * BMAX), o_fix = plan(4 * BMAX), o_flab = plan(4 * BMAX), o_xcnt = plan(4 * BMAX),
                  o_psize = plan(4 * BMAX), o_snew = plan(4 * BMAX), o_scur = plan(4 * BMAX), o_slot = plan(4 * BMAX),
@@ -579,6 +641,7 @@ cudaError_t run_connect(const ConnectLaunch &l, int out_host[4], cudaStream_t st
     a.max_steps = l.max_steps;
     a.reached = reinterpret_cast<uint32_t *>(at(o_reached));
     a.stamp = reinterpret_cast<int *>(at(o_stamp));
+    a.used = reinterpret_cast<int *>(at(o_used));
     a.bmax = BMAX;
     a.head = reinterpret_cast<int2 *>(at(o_head));
     a.st = reinterpret_cast<FixState *>(at(o_st));
