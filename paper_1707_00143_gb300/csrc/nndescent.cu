@@ -279,10 +279,15 @@ __global__ void nd_member_fill_kernel(NdArgs a) {
 // registers; held to 64 registers for 8 blocks it spills, 28.5 -> 33.8 ms of
 // kNN stage): reading the members one after the other, three dependent loads
 // each, took the stage of 150,000 DEEP-shaped rows (K = 64, 6 iterations) 31.2
-// ms, with them read ahead it takes 28.5 ms.
+// ms, with them read ahead it takes 28.5 ms.  Rows of more than 256 values are
+// bound by their bytes: 24 warps or fewer, and the registers to the row gathers
+// instead of offers read ahead (50,000 x 400 uniform rows, K = 40, 5 iterations: 119 ms
+// before, 140 at 28 warps with offers ahead, 103 at 24, 96 at 24 without; 20,000
+// x 960 GIST-shaped 10.5, 11.3, 9.7, 8.9).
 template <int G, int V, int U, bool U8>
-__global__ void __launch_bounds__(128, V <= 4 ? 7 : 1) nd_join_kernel(NdArgs a) {
+__global__ void __launch_bounds__(128, G < 32 ? 7 : V <= 4 ? 6 : V <= 8 ? 4 : 3) nd_join_kernel(NdArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
+    constexpr bool AHEAD = G < 32;
     const int warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const unsigned lane = lane_id();
     NdSmem s = nd_carve(smem + warp * nd_warp_bytes(a.K, true), a.K, true);
@@ -323,15 +328,15 @@ __global__ void __launch_bounds__(128, V <= 4 ? 7 : 1) nd_join_kernel(NdArgs a) 
                     const int j = b + (int)lane;
                     return j < c ? __ldg(a.NEWs + r + j) : (j < t ? __ldg(a.OLDs + r + j - c) : -1);
                 };
-                int x0 = offer(0, 0), x1 = offer(0, 32);
+                int x0 = AHEAD ? offer(0, 0) : 0, x1 = AHEAD ? offer(0, 32) : 0;
                 for (int i = 0; i < members; ++i) {
                     const int y0 = x0, y1 = x1, t = __shfl_sync(NSG_FULL, tot, i);
-                    if (i + 1 < members) {
+                    if (AHEAD && i + 1 < members) {
                         x0 = offer(i + 1, 0);
                         x1 = offer(i + 1, 32);
                     }
                     for (int b = 0; b < t; b += 32) {
-                        const int x = b == 0 ? y0 : b == 32 ? y1 : offer(i, b);
+                        const int x = AHEAD && b == 0 ? y0 : AHEAD && b == 32 ? y1 : offer(i, b);
                         // p itself is among its own offers (p is in NEW(v)); the visited set
                         // may have forgotten it, so it is excluded by id
                         const bool fresh = x >= 0 && x != (int)p && visit(s.hash, hmask, hshift, x);
