@@ -77,14 +77,16 @@ __device__ __forceinline__ void collect_body(const CollectArgs &a) {
 
 // 20 warps per SM by the lists' shared memory: rows of up to 512 values on 80
 // registers without spills (the compiler's own choice is 64 with some: 612 -> 705
-// ms for 1,000,000 uniform rows of 128 values, K = 100, L = 60), wider ones on
-// the compiler's own budget.
+// ms for 1,000,000 uniform rows of 128 values, K = 100, L = 60).  Wider rows: 5
+// blocks of 128 threads up to 1,024 values (20,000 x 960, K = 40, L = 40, C = 200:
+// 12.6 ms on the compiler's own budget, 11.0), 4 above (20,000 x 1,500: 24.1 free,
+// with 12 warps on 160 registers; 21.9).
 template <int G, int V, int U>
 __global__ void __launch_bounds__(256, 3) collect_kernel(CollectArgs a) {
     collect_body<G, V, U>(a);
 }
 template <int G, int V, int U>
-__global__ void __launch_bounds__(256) collect_wide_kernel(CollectArgs a) {
+__global__ void __launch_bounds__(128, V > 8 ? 4 : 5) collect_wide_kernel(CollectArgs a) {
     collect_body<G, V, U>(a);
 }
 template <int G, int V, int U>
@@ -137,13 +139,13 @@ __device__ __forceinline__ void collect_log_body(const CollectArgs &a) {
 }
 
 // As for the searches: rows of up to 512 values at 64 registers and 32 warps
-// per SM, wider ones on the compiler's own budget.
+// per SM; wider ones as above.
 template <int G, int V, int U, bool U8>
 __global__ void __launch_bounds__(256, 4) collect_log_kernel(CollectArgs a) {
     collect_log_body<G, V, U, U8>(a);
 }
 template <int G, int V, int U, bool U8>
-__global__ void __launch_bounds__(256) collect_log_wide_kernel(CollectArgs a) {
+__global__ void __launch_bounds__(128, V > 8 ? 4 : 5) collect_log_wide_kernel(CollectArgs a) {
     collect_log_body<G, V, U, U8>(a);
 }
 template <int G, int V, int U>
@@ -165,7 +167,7 @@ void (*collect_log_entry(bool u8))(CollectArgs) {
 // first-copy flags are one register.
 constexpr int SEL_BINS = 1024;
 constexpr int LOG_CAP_MAX = 16384;
-constexpr int LOG_LONG = 6400;  // run_collect_log
+constexpr int LOG_LONG = 12;  // run_collect_log
 
 template <int NT>
 struct SelectShared {
@@ -434,9 +436,10 @@ static CollectLaunch part_of(const CollectLaunch &l, int64_t j0, int64_t nv) {
 // selection gets the shared memory that the slice's longest log needs.  The
 // host reads that number between the two: ~15 us a slice.  A node whose log
 // fills is searched again with a merged list.  What a log costs grows with every
-// key, a merged list's cost only with the keys that enter: FP32 searches that
-// pass LOG_LONG keys are merged (uniform rows of 128 values, K = 100, L = 60,
-// 1,000,000: 1,105 ms logged, 612 merged; 30,000, 6,600 keys: equal), 8-bit ones
+// key, a merged list's cost only with the keys that enter, which C bounds: FP32
+// searches that pass LOG_LONG C keys are merged (uniform rows of 128 values, K =
+// 100, L = 60, C = 500, 1,000,000: 1,105 ms logged, 612 merged; 30,000, 6,600
+// keys: equal; 20,000 x 960, K = L = 40, C = 200: 13.4 and 11.4), 8-bit ones
 // as long as logs hold them are not (300,000 such rows: 103 ms logged, 156
 // merged on FP32 rows).  Merged lists alone -> logs: 1,000,000 SIFT-shaped rows
 // 295 -> 138 ms, 10,000,000 DEEP-shaped 2,614 -> 2,040 (with logs of L K / 2 that
@@ -485,7 +488,7 @@ cudaError_t run_collect_log(const CollectLaunch &l, CollectLog &log, cudaStream_
         if (err == cudaSuccess && seen[1] > 0) err = launch_merge(slice, true, st);
         if (err != cudaSuccess) return err;
         log.merge = (seen[1] == 0 || a.log_cap == LOG_CAP_MAX) &&
-                    seen[0] > (a.rows.u8 != nullptr ? LOG_CAP_MAX : LOG_LONG);
+                    seen[0] > (a.rows.u8 != nullptr ? LOG_CAP_MAX : LOG_LONG * l.C);
         log.cap = std::min(std::max((seen[0] + seen[0] / 4 + l.K + 31) & ~31, 1024), LOG_CAP_MAX);
         j0 += nodes;
     }
