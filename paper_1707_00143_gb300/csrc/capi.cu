@@ -288,34 +288,28 @@ nsg_status exact8_copy(const float *base, int64_t n, int dp, int d, DevBuf<unsig
     x = nsg::Exact8{};
     const int dpl = (d + 15) / 16 * 16;
     if ((int64_t)d * 65025 >= (1 << 24)) return NSG_OK;
-    size_t free = 0, total = 0;
-    NSG_CK(cudaMemGetInfo(&free, &total));
-    if (free < (size_t)n * dpl + reserve) return NSG_OK;
     DevBuf<unsigned> flags;
     NSG_CK(flags.alloc(4));
     unsigned mm[3] = {0xffffffffu, 0u, 0u};
     NSG_CK(cudaMemcpyAsync(flags.p, mm, sizeof(mm), cudaMemcpyHostToDevice, st));
-    NSG_CK(nsg::launch_minmax(base, n, dp, d, flags.p, st));
+    NSG_CK(nsg::launch_whole_range(base, n, dp, d, flags.p, st));
     NSG_CK(cudaMemcpyAsync(mm, flags.p, sizeof(mm), cudaMemcpyDeviceToHost, st));
     NSG_CK(cudaStreamSynchronize(st));
     const float mn = nsg::float_from_order_key(mm[0]), mx = nsg::float_from_order_key(mm[1]);
     if (mm[2] != 0 || !((double)mx - (double)mn <= 255.0)) return NSG_OK;
+    size_t free = 0, total = 0;
+    NSG_CK(cudaMemGetInfo(&free, &total));
+    if (free < (size_t)n * dpl + reserve) return NSG_OK;
     if (buf.alloc((size_t)n * dpl) != cudaSuccess) {
         cudaGetLastError();
         return NSG_OK;
     }
-    NSG_CK(cudaMemsetAsync(flags.p, 0, sizeof(unsigned), st));
-    NSG_CK(nsg::launch_to_lowp(base, n, dp, d, NSG_PREC_U8, 1.0f, mn, buf.p, dpl, reinterpret_cast<int *>(flags.p),
-                               st));
-    unsigned inexact = 0;
-    NSG_CK(cudaMemcpyAsync(&inexact, flags.p, sizeof(inexact), cudaMemcpyDeviceToHost, st));
+    NSG_CK(nsg::launch_exact8(base, n, dp, d, mn, buf.p, dpl / 16, st));
     NSG_CK(cudaStreamSynchronize(st));
-    if (inexact == 0) {
-        x.rows = buf.p;
-        x.chunks = dpl / 16;
-        x.d = d;
-        x.lo = mn;
-    }
+    x.rows = buf.p;
+    x.chunks = dpl / 16;
+    x.d = d;
+    x.lo = mn;
     return NSG_OK;
 }
 
@@ -843,8 +837,8 @@ static nsg_status build_index(const float *base_dev, int64_t n, int32_t d, int32
     auto t0 = std::chrono::steady_clock::now();
     if (!s && !nnd) s = knn_run(base.p, n, ix->dp, base.p, n, 0, K, 1, knn.p, nullptr, st);
     // what the stages to come cannot do without: candidate lists, the connectivity
-    // pass's arrays (28 bytes per row and up to 512 MB of pools), nn-descent's
-    size_t reserve = std::max((size_t)collect_chunk(n, C) * ((size_t)C * 8 + 8), 28 * (size_t)n + (size_t(512) << 20));
+    // pass's arrays (32 bytes per row and up to 512 MB of pools), nn-descent's
+    size_t reserve = std::max((size_t)collect_chunk(n, C) * ((size_t)C * 8 + 8), 32 * (size_t)n + (size_t(512) << 20));
     if (nnd) reserve = std::max(reserve, nsg::nndescent_scratch_bytes(n, K, nnd->sample, nnd->reverse));
     if (!s) s = exact8_copy(base.p, n, ix->dp, d, u8buf, u8, st, reserve + kExact8Reserve);
     if (!s && nnd) s = nndescent_run(base.p, n, ix->dp, d, K, *nnd, u8, knn.p, nullptr, &ix->knn_iters, nullptr,

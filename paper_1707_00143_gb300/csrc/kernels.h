@@ -158,6 +158,10 @@ cudaError_t launch_absmax(const float *x, int64_t count, unsigned *out_bits, cud
 // Order-preserving keys of min x and max x (out[0], out[1]; start them at
 // 0xffffffff and 0) and out[2] |= 1 when some x is not an integer.
 cudaError_t launch_minmax(const float *x, int64_t n, int dp, int d, unsigned *out, cudaStream_t st);
+// The same for rows [n][dp] of d values, 16-byte aligned, the keys only if all are
+// integers; and the 8-bit copy x - lo of integers of [lo, lo + 255].
+cudaError_t launch_whole_range(const float *x, int64_t n, int dp, int d, unsigned *out, cudaStream_t st);
+cudaError_t launch_exact8(const float *x, int64_t n, int dp, int d, float lo, void *dst, int chunks, cudaStream_t st);
 // (key of f: sign bit set -> all bits flipped, else the sign bit set)
 inline float float_from_order_key(unsigned k) {
     unsigned b = (k & 0x80000000u) ? (k & 0x7fffffffu) : ~k;
