@@ -520,9 +520,9 @@ void destroy(nsg_index *ix) {
     if (ix->deg) cudaFree(ix->deg);
     if (ix->flag) cudaFree(ix->flag);
     if (ix->work) cudaFree(ix->work);
-    if (ix->exact8_buf) cudaFree(ix->exact8_buf);
     for (void *p : ix->lowp)
-        if (p) cudaFree(p);
+        if (p && p != ix->exact8_buf) cudaFree(p);
+    if (ix->exact8_buf) cudaFree(ix->exact8_buf);
     for (void *p : ix->lowp_map)
         if (p) cudaFree(p);
     if (ix->host_q) cudaFree(ix->host_q);
@@ -1623,6 +1623,14 @@ nsg_status nsg_stop_train(const float *feat_dev, const uint8_t *flag_dev, const 
 nsg_status nsg_index_prepare(nsg_index *idx, int32_t precision, void *stream) {
     if (!idx || precision < NSG_PREC_BF16 || precision > NSG_PREC_U8) return NSG_EINVAL;
     if (idx->lowp[precision]) return NSG_OK;
+    if (precision == NSG_PREC_U8 && idx->exact8.rows) {  // the same bytes: x - lo, every distance exact
+        idx->lowp[precision] = idx->exact8_buf;
+        idx->lowp_dpl[precision] = idx->exact8.chunks * 16;
+        idx->lowp_scale[precision] = 1.0f;
+        idx->lowp_lo[precision] = idx->exact8.lo;
+        idx->lowp_exact[precision] = 1;
+        return NSG_OK;
+    }
     cudaStream_t st = S(stream);
     const int epc = precision == NSG_PREC_BF16 ? 8 : 16;  // values per 16-byte chunk
     const int dpl = (idx->d + epc - 1) / epc * epc;
@@ -1749,7 +1757,7 @@ nsg_status nsg_index_info(const nsg_index *idx, nsg_index_info_t *info) {
     info->u8_scale = idx->lowp[NSG_PREC_U8] ? idx->lowp_scale[NSG_PREC_U8] : 0.0f;
     info->prune_examined = idx->prune_examined;
     for (int p = 1; p <= 3; ++p)
-        if (idx->lowp[p]) info->device_bytes += (int64_t)idx->n * idx->lowp_dpl[p] * (p == 1 ? 2 : 1);
+        if (idx->lowp[p] && idx->lowp[p] != idx->exact8_buf) info->device_bytes += (int64_t)idx->n * idx->lowp_dpl[p] * (p == 1 ? 2 : 1);
     if (idx->exact8.rows) info->device_bytes += (int64_t)idx->n * idx->exact8.chunks * 16;
     info->ms_knn = idx->ms[0];
     info->ms_centroid_nav = idx->ms[1];

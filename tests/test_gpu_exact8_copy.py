@@ -58,3 +58,19 @@ def test_copy_costs_a_read(nsg):
     whole = seconds(base)
     base[0, 0] = 0.5
     assert whole - seconds(base) < 0.6e-3  # 1.0 ms a value at a time
+
+
+def test_prepared_copy_is_the_same_one(nsg):
+    rng = np.random.default_rng(1)
+    base = torch.from_numpy(rng.integers(-50, 200, (4000, 40)).astype(np.float32)).cuda()
+    adj = torch.from_numpy(rng.integers(0, 4000, (4000, 16)).astype(np.int32)).cuda()
+    idx = nsg.nsg_index_from_graph(base, adj, 3)
+    q = base[:300].contiguous()
+    want = idx.search(q, 10, 50)
+    before = idx.info()["device_bytes"]
+    idx.prepare(nsg.PREC_U8)
+    info = idx.info()
+    assert info["device_bytes"] == before
+    out = idx.search_ex(q, 10, 50, params=nsg.SearchParams(precision=nsg.PREC_U8))
+    assert torch.equal(out["ids"], want[0]) and torch.equal(out["d2"], want[1])
+    idx.free()
