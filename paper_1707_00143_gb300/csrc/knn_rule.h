@@ -26,7 +26,9 @@ inline int knn_sample_tiles(int64_t ntiles, int rank) {
 // Bounded, the units' scan is the faster one and their pre-pass, rings and
 // launches are what short bases do not pay back: 200 us more for one query,
 // and for many queries on few rows (12,000 x 128, KL = 10: 8,000 queries
-// 1.04 times the units' speed, 1,500 0.73).  Unbounded, nearly every
+// 1.04 times the units' speed, 1,500 0.73).  Rows in tight clusters side by side
+// get little from the pre-pass (20,000-row graph, K = 10, clusters of 100: 2,604 us,
+// units 4,156; 60,000 rows: equal).  Unbounded, nearly every
 // column is a candidate and merging is the work: a unit's wave takes ~1.8 times
 // a CTA wave (40,000 x 96, KL = 150, 10,000 queries: 4,845 us, units 6,763), so
 // units win when they finish in one wave where the CTAs need two (26,000-row
@@ -37,7 +39,7 @@ inline int knn_sample_tiles(int64_t ntiles, int rank) {
 inline bool knn_small(int64_t n, int64_t nq, int KL, bool bounded, int sms) {
     const int64_t ctas = (nq + 127) / 128, units = (nq + 255) / 256;
     const bool one_wave = ctas > sms && units <= sms;
-    if (bounded) return !(n >= 20480 || (n >= 8192 && one_wave) || (n >= (nq < 32 ? 16384 : 8192) && 3 * nq <= n));
+    if (bounded) return !(n >= 20480 || (n >= (nq < 32 ? 16384 : 8192) && 3 * nq <= n && nq <= 2048));
     return !(KL >= 64 && ((n >= 10240 && nq <= 2048) || (n >= 20000 && one_wave && 3 * units > 2 * sms)));
 }
 

@@ -15,7 +15,7 @@ TIMED = [
     (12000, 1500, 10, 0, 0, 1442, 1722), (12000, 1500, 10, 1, 0, 902, 659), (18000, 1500, 10, 0, 0, 1700, 1300),
     (26000, 300, 100, 0, 0, 3861, 2788), (26000, 26000, 100, 1, 1, 5340, 4319), (26000, 24000, 200, 1, 0, 9742, 15484),
     (40000, 40000, 100, 0, 1, 12861, 20223), (40000, 10000, 100, 0, 0, 4845, 6763), (40000, 1500, 100, 1, 0, 3321, 1064),
-    (40000, 4000, 100, 1, 0, 3360, 1598), (40000, 40000, 100, 1, 1, 9160, 7000), (20000, 24000, 30, 1, 0, 2465, 1539),
+    (40000, 4000, 100, 1, 0, 3360, 1598), (40000, 40000, 100, 1, 1, 9160, 7000), (20000, 20000, 10, 0, 1, 2604, 4156),  # the last: rows in tight clusters
     (1000000, 1000, 100, 0, 0, 47300, 6500), (10000, 100, 10, 1, 0, 760, 490),
 ]
 
