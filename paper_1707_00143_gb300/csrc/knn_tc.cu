@@ -816,7 +816,10 @@ __global__ void __launch_bounds__(256) knn_merge_kernel(const int *ids_in, const
 // Row-wise BF16 copy with K padded to DK, squared norms of the rounded values
 // (+inf past the last row: such a column is never a candidate), and a flag
 // raised when a value is not an integer in 0..255.  Bound by memory: a warp
-// has four rows of 16-byte loads in flight.
+// has four rows of 16-byte loads in flight.  The norms are summed lane by lane,
+// value c in lane c % 32 (read again, from L1), as they have always been: where
+// keys tie but for rounding (clusters far from the origin, whose rows round to few
+// values) the order of the sum decides which candidates are kept.
 __global__ void __launch_bounds__(256) bf16_rows_kernel(const float4 *__restrict__ src, int64_t rows, int dp4,
                                                         uint2 *dst, int dk4, float *norms, int64_t rows_pad,
                                                         int *nonint) {
@@ -824,10 +827,12 @@ __global__ void __launch_bounds__(256) bf16_rows_kernel(const float4 *__restrict
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const unsigned lane = lane_id();
+    const float *flat = reinterpret_cast<const float *>(src);
     bool bad = false;
     for (int64_t r0 = warp * RW; r0 < rows_pad; r0 += nw * RW) {
         float acc[RW] = {0.0f, 0.0f, 0.0f, 0.0f};
-        for (int c = lane; c < dk4; c += 32) {
+        for (int c0 = 0; c0 < dk4; c0 += 32) {
+            const int c = c0 + (int)lane;
             float4 v[RW];
 #pragma unroll
             for (int j = 0; j < RW; ++j)
@@ -839,15 +844,23 @@ __global__ void __launch_bounds__(256) bf16_rows_kernel(const float4 *__restrict
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const __nv_bfloat16 b = __float2bfloat16_rn(f[e]);
-                    const float hv = __bfloat162float(b);
-                    acc[j] += hv * hv;
                     bad |= !(f[e] >= 0.0f && f[e] <= 255.0f && f[e] == rintf(f[e]));
                     h[e] = __bfloat16_as_ushort(b);
                 }
-                if (r0 + j < rows)
+                if (r0 + j < rows && c < dk4)
                     dst[(r0 + j) * dk4 + c] =
                         make_uint2(h[0] | ((unsigned)h[1] << 16), h[2] | ((unsigned)h[3] << 16));
             }
+            const int at = 4 * c0 + (int)lane;  // the chunk's values of this lane
+#pragma unroll
+            for (int j = 0; j < RW; ++j)
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const int i = at + 32 * t;
+                    const float f = r0 + j < rows && i < 4 * dp4 ? __ldg(flat + (r0 + j) * 4 * dp4 + i) : 0.0f;
+                    const float hv = __bfloat162float(__float2bfloat16_rn(f));
+                    acc[j] += hv * hv;
+                }
         }
 #pragma unroll
         for (int j = 0; j < RW; ++j) {

@@ -91,3 +91,18 @@ def test_far_queries(nsg, monkeypatch, scale):
     if scale > 1e19:
         assert np.isinf(out[0][1]).all()
         assert np.array_equal(out[0][0], np.tile(np.arange(10), (400, 1)))
+
+
+@pytest.mark.parametrize("d", [24, 100, 200])
+def test_tied_clusters(nsg, monkeypatch, d):
+    """Clusters far from the origin, whose rows round to few BF16 values: which candidates a full list keeps is
+    decided by the norms' last bits, the same for both kernels."""
+    rng = np.random.default_rng(d)
+    n = 24000
+    base = (100 * rng.standard_normal((n // 100, d))).repeat(100, 0) + rng.random((n, d))
+    base = base.astype(np.float32)
+    out = []
+    for e in ("units", "small"):
+        monkeypatch.setenv("NSG_KNN_ENGINE", e)
+        out.append([t.cpu().numpy() for t in nsg.nsg_knn_query(T(base), T(base[::50] + np.float32(0.01)), 10)])
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
