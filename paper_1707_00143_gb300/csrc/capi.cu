@@ -1083,7 +1083,6 @@ nsg_status nsg_build_partitioned(const float *base_dev, int64_t n, int32_t d, co
 
 namespace {
 
-// Validated launch description for nsg_search_ex / nsg_search_trace.
 // The plain form on integer rows takes its keys from the index's 8-bit copy.
 void use_exact8(const nsg_index *idx, nsg::SearchLaunch &l) {
     if (!idx->exact8.rows) return;
@@ -1093,6 +1092,7 @@ void use_exact8(const nsg_index *idx, nsg::SearchLaunch &l) {
     l.lowp_lo = idx->exact8.lo;
 }
 
+// Validated launch description for nsg_search_ex / nsg_search_trace.
 nsg_status make_search(const nsg_index *idx, const float *queries_dev, int64_t nq, int32_t k, int32_t L,
                        const nsg_search_params *params, int32_t *ids_dev, float *d2_dev, int32_t *n_expand_dev,
                        int32_t *n_dist_dev, int32_t *status_dev, nsg::SearchLaunch &l) {

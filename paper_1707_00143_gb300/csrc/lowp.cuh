@@ -288,14 +288,14 @@ struct Exact8Shape {
 
 // The distance functor for row v as the query: FP32 rows, or the exact 8-bit
 // copy (a quarter of the bytes, the same keys), laid out as the 8-bit search
-// form lays it out (lanes of 2 16-byte chunks, 3 row groups in flight; 8 for
-// rows of 513..1024 values).
+// form lays it out (lanes of 2 16-byte chunks, 3 row groups in flight).  The
+// copy's rows end at 258 values.
 template <int G, int V, int U, bool U8, class F>
 __device__ __forceinline__ void with_row_dist(const ExactRows &r, int64_t v, F &&f) {
     if constexpr (U8) {
+        static_assert(V <= 4);
         using S = Exact8Shape<G, V>;
-        constexpr int R8 = V == 8 ? 8 : (V > 8 ? 2 : 3);
-        DistU8<S::lanes, S::chunks, R8> dist{{}, r.u8, r.dc};
+        DistU8<S::lanes, S::chunks, 3> dist{{}, r.u8, r.dc};
         dist.Q.load(reinterpret_cast<const float *>(r.base4 + v * r.dp4), r.d, r.lo, 1.0f);
         f(dist);
     } else {

@@ -529,8 +529,10 @@ cudaError_t launch_nndescent(const NnDescentLaunch &l, cudaStream_t st) {
     const int dp4 = a.rows.dp4;
     const bool u8 = a.rows.u8 != nullptr;
     NSG_DISPATCH_DP4(dp4, {
-        e = u8 ? warp_launch(nd_init_kernel<G_, V_, U_, true>, a, per_warp, st)
-               : warp_launch(nd_init_kernel<G_, V_, U_, false>, a, per_warp, st);
+        void (*init)(NdArgs) = nd_init_kernel<G_, V_, U_, false>;
+        if constexpr (V_ <= 4)  // no 8-bit copy of wider rows
+            if (u8) init = nd_init_kernel<G_, V_, U_, true>;
+        e = warp_launch(init, a, per_warp, st);
     });
     if (e != cudaSuccess) return e;
     int it = 0;
@@ -552,8 +554,10 @@ cudaError_t launch_nndescent(const NnDescentLaunch &l, cudaStream_t st) {
         if ((e = cudaMemsetAsync(a.mcnt, 0, 4ull * n, st)) != cudaSuccess) return e;
         nd_member_fill_kernel<<<grid_for(n * std::max(W2, 1), 256), 256, 0, st>>>(a);
         NSG_DISPATCH_DP4(dp4, {
-            e = u8 ? warp_launch(nd_join_kernel<G_, V_, U_, true>, a, join_warp, st)
-                   : warp_launch(nd_join_kernel<G_, V_, U_, false>, a, join_warp, st);
+            void (*join)(NdArgs) = nd_join_kernel<G_, V_, U_, false>;
+            if constexpr (V_ <= 4)
+                if (u8) join = nd_join_kernel<G_, V_, U_, true>;
+            e = warp_launch(join, a, join_warp, st);
         });
         if (e != cudaSuccess) return e;
         if ((e = cudaMemcpyAsync(&upd, a.updates, 8, cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
