@@ -23,9 +23,12 @@
 // the rows' sorted lists, which live in the output arrays, and publishes the
 // new k-th distances.  A scan with an older bound only finds more candidates.
 //
-// Bound by the scan's instructions and the accumulator hand-over, not the
-// tensor pipe: a column costs half a packed FMA and half a 3-input min per
-// row, and a candidate's group ~10 warp instructions whatever the other 31
+// Bound by latency: at 262,144 x 128 the tensor pipe is active 25 % of the cycles
+// and issue 42 %; a scanning warp loads 32 columns, waits and tests them with
+// nothing in flight behind (long scoreboard 3.8 per instruction), and the
+// accumulator hand-over holds the MMAs to that pace.  A column costs half a packed
+// FMA and half a 3-input min per row, and a candidate's group ~10 warp
+// instructions whatever the other 31
 // rows do.  What the structure is for:
 //  (a) merging takes ~5,000 cycles of dependent loads and shuffles; done by
 //      the scanning warps it held up the accumulators, and with them every
