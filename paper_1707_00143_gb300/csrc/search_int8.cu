@@ -21,14 +21,14 @@ __global__ void __launch_bounds__(256) queries_held_kernel(const float *queries,
 
 // One kernel that has both paths, or a kernel each of which the batch as a
 // whole takes one.  In one kernel warps on different paths evict each other's
-// instructions once the SMs are full (10,000 queries on 50,000 x 200 rows, k =
-// 10, L = 150: 2,444 us with fractions in every other query, 2,192 with fractions
-// throughout, 2,121 on FP32 rows alone), and with pools in global memory it
-// spills (50 queries, L = 1,500: 5 % slower than FP32 rows alone; apart
-// 1 %).  Apart, two more launches cost ~15 us: 10 % of a single query's search
-// (L = 30), 1 to 3 % of 10,000 queries'.  So batches of 2,048 queries and pools in
-// global memory take them apart: every other query a fraction 2,127 us, fractions
-// throughout 2,101, none 1,440.
+// instructions once the SMs are full, the more so the longer the row's code (10,000
+// queries on 50,000 x 200 rows, k = 10, L = 150: 2,435 us with fractions in every
+// other query, 2,181 with fractions throughout, 1,502 with none, 2,107 on FP32 rows
+// alone), and with pools in global memory it spills (50 queries, L = 1,500: 5 %
+// slower than FP32 rows alone; apart 1 %).  Apart: 2,121, 2,096 and 1,442 us;
+// but the two more launches cost ~15 us, 10 % of a single query's search (L = 30), 4 %
+// of 2,500 queries', and rows of up to 64 values have little code to evict (10,000
+// queries on 50,000 x 32: every other one a fraction 1,606 us apart, 1,539 in one).
 template <bool GP>
 static cudaError_t launch_apart(SearchArgs a, const SearchLaunch &l, size_t per_warp, int wpq, cudaStream_t st) {
     int *left = l.work + WORK_LEFT;
@@ -45,7 +45,7 @@ static cudaError_t launch_apart(SearchArgs a, const SearchLaunch &l, size_t per_
 
 cudaError_t launch_search_int8(const SearchArgs &a, const SearchLaunch &l, size_t per_warp, int wpq, cudaStream_t st) {
     if (a.gpool != nullptr) return launch_apart<true>(a, l, per_warp, wpq, st);
-    if (l.nq >= 2048) return launch_apart<false>(a, l, per_warp, wpq, st);
+    if (l.nq >= 4096 && l.d > 64) return launch_apart<false>(a, l, per_warp, wpq, st);
     return launch_search_args<false, false, PREC_F32_EITHER>(a, l, per_warp, 0, false, wpq, st);
 }
 
