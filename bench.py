@@ -213,8 +213,9 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(sm)}
 
 
-SEARCH_SOURCES = ("common.cuh", "search_core.cuh", "lowp.cuh", "stage.cuh", "search_kern.cuh", "search.cu")
-PRUNE_SOURCES = ("common.cuh", "search_core.cuh", "build.cu")
+SEARCH_SOURCES = ("common.cuh", "search_core.cuh", "lowp.cuh", "stage.cuh", "search_kern.cuh", "search.cu",
+                  "search_int8.cu")
+PRUNE_SOURCES = ("common.cuh", "search_core.cuh", "lowp.cuh", "build.cu")
 
 
 def refine_L(pts, t, recall_at, qps_at):
@@ -773,8 +774,13 @@ def main():
     n_expand = cnt["n_expand"].to(torch.int64).sum().item()
     R = info["R"]
     base_form = chosen_form.split("+")[0]
-    row_bytes = {"plain": d * 4, "bf16": ((d + 7) // 8) * 16, "fp8": ((d + 15) // 16) * 16,
+    # integer rows of 8 bits: the plain form and the edge selection read the exact 8-bit copy
+    plain_bytes = (d + 15) // 16 * 16 if W.get("integer") and d * 65025 < 1 << 24 else d * 4
+    row_bytes = {"plain": plain_bytes, "bf16": ((d + 7) // 8) * 16, "fp8": ((d + 15) // 16) * 16,
                  "u8": ((d + 15) // 16) * 16}[base_form]
+    # four kernels for the visiting order and the search; the plain form on 8-bit
+    # rows looks through a large batch first and takes one of two search kernels
+    launches = 7 if chosen_form == "plain" and plain_bytes < d * 4 and nq >= 4096 and d > 64 else 5
     lossy = {"plain": False, "bf16": info["has_bf16"] == 1, "fp8": info["has_fp8"] == 1,
              "u8": info["has_u8"] == 1}[base_form]
     bytes_launch = (n_dist * row_bytes + n_expand * R * 4 + nq * (d * 4 + kc * 8)
@@ -914,9 +920,9 @@ def main():
                           "frac": iach / ipeak, "instructions_per_query": ins, "kernel_src": src,
                           "peak_from": "SMs x 4 schedulers x max SM clock"}
     # MRNG edge selection over the whole build: every examined candidate's id,
-    # distance and FP32 row read once, the adjacency row, degree and candidate
-    # count per node; over the prune launches' CUDA-event time
-    prune_bytes = info["prune_examined"] * (4 * d + 8) + n * (4 * BUILD["R"] + 8)
+    # distance and row (FP32 or the exact 8-bit copy) read once, the adjacency row,
+    # degree and candidate count per node; over the prune launches' CUDA-event time
+    prune_bytes = info["prune_examined"] * (plain_bytes + 8) + n * (4 * BUILD["R"] + 8)
     prune_roofline = {"bound": "hbm", "achieved": prune_bytes / (info["ms_prune"] / 1e3) / 1e9 if info["ms_prune"] else None,
                       "peak": peak, "unit": "GB/s", "peak_kind": peak_kind, "kernel": "prune_kernel",
                       "algorithmic_bytes": prune_bytes, "examined_per_node": info["prune_examined"] / n,
@@ -956,8 +962,8 @@ def main():
             "e2e": {"value": job_qps(world, nq, e2e_ms), "unit": UNIT,
                     "h2d_bytes_per_step": nq * d * 4, "d2h_bytes_per_step": nq * kc * 4,
                     "call": "nsg_search_host", "same_ids_as_device_call": e2e_same},
-            # per step: the visiting order (distance, bucket, scan, scatter) and the search
-            "gpu_launches": 5 * args.steps,
+            # per step: the visiting order (distance, bucket, scan, scatter) and the search (above)
+            "gpu_launches": launches * args.steps,
             "clocks": clocks,
             "build_seconds": build_s,
             "build_ms": {k: info[k] for k in ("ms_knn", "ms_centroid_nav", "ms_collect", "ms_prune",
