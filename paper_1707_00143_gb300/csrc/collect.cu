@@ -460,8 +460,11 @@ cudaError_t run_collect_log(const CollectLaunch &l, CollectLog &log, cudaStream_
     for (int64_t j0 = 0; j0 < l.nv;) {
         a.log_cap = log.cap > 0 ? log.cap : log.first_cap > 0 ? log.first_cap : first_log_cap(l.L, l.K);
         a.log_cap = std::min(a.log_cap, LOG_CAP_MAX);
+        // a few waves at most: one slice, with the logs there is room for
+        const bool one = log.cap == 0 && log.first_cap == 0 && l.nv <= first_nodes() * 5 / 2 && log.size >= 1024 * l.nv;
+        if (one) a.log_cap = (int)std::min<int64_t>(a.log_cap, log.size / l.nv);
         int64_t nodes = std::min(l.nv - j0, log.size / a.log_cap);
-        if (log.cap == 0) nodes = std::min(nodes, first_nodes());
+        if (log.cap == 0 && !one) nodes = std::min(nodes, first_nodes());
         if (log.merge || nodes < 1) return launch_merge(part_of(l, j0, l.nv - j0), false, st);
         const CollectLaunch slice = part_of(l, j0, nodes);
         a.v0 = slice.v0;
